@@ -1002,7 +1002,7 @@ def run_realistic(args, dev, rates, clk) -> dict:
         "pairs": {"logical_per_step": p.pairs, "evaluated_training_forward": ev[512],
                   "evaluated_dv_sweep": ev[1024],
                   "note": "value counts every logical (i, j) pair; the grid kernels leave out the pairs whose "
-                          "FP32 exp2 flushes to exactly 0 (scaled distance^2 > 170), so results are identical to "
+                          "FP32 exp2 flushes to exactly 0 (scaled distance^2 > 127), so results are identical to "
                           "evaluating all of them; the roofline counts evaluated pairs"},
         "roofline": {"bound": "alu", "achieved": d["achieved"], "peak": d["peak"], "unit": UNIT,
                      "frac": d["frac"], "traffic": measured_traffic("realistic: " + dom), "kernel": dom,
@@ -1266,7 +1266,7 @@ def run_large(args, rank, local, world, dist, dev):
         "pairs": {"logical_per_step": p.pairs, "evaluated_forward": pf, "evaluated_backward": pb,
                   "slots_forward": sf, "slots_backward": sb,
                   "note": "value counts every logical (i, j) pair, as the metric defines it; the culled sweeps "
-                          "leave out the pairs whose FP32 exp2 flushes to exactly 0 (scaled distance^2 > 170), so "
+                          "leave out the pairs whose FP32 exp2 flushes to exactly 0 (scaled distance^2 > 127), so "
                           "results are bitwise those of evaluating all of them (tested); the roofline counts the "
                           "evaluated pairs"},
         "roofline": {"bound": "alu", "achieved": d["achieved"], "peak": d["peak"], "unit": UNIT,

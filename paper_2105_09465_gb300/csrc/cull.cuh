@@ -23,8 +23,8 @@
 // Exact skipping. A pair with t > 126 has an exponent below -126, where the
 // flush-to-zero exp2 returns exactly 0. A row block (or one warp of it) leaves
 // out every group and chunk whose box is farther than sqrt(kSkipT) =
-// sqrt(170) scaled units from its own box; the margin over 126 absorbs the
-// FP32 rounding of both distances. A left-out chunk's partial sums are exact
+// sqrt(127) scaled units from its own box; the margin over 126 absorbs the
+// FP32 rounding of both distances (below 1e-4 there). A left-out chunk's partial sums are exact
 // zeros, and the kernels fold a chunk's sums into the row totals only when
 // they are nonzero (the forward) or add them plainly (the moments, where
 // adding +0 changes nothing), so culled and unculled sweeps give the same

@@ -99,8 +99,8 @@ __device__ __forceinline__ void bw_load_pair(const BwArgs& A, int t, int p, floa
     const float xb = (b < cnt) ? A.sc * (grid_x(A.src.g, c0 + b) - o) : 0.f;
     if (SPLIT) {
       // split exponent: v~ = v 2^-x'^2 and its first two x' moments
-      const float va = (a < cnt) ? __ldg(A.v + j0 + a) * ex2_approx(-xa * xa) : 0.f;
-      const float vb = (b < cnt) ? __ldg(A.v + j0 + b) * ex2_approx(-xb * xb) : 0.f;
+      const float va = (a < cnt) ? __ldg(A.v + j0 + a) * split_factor(xa) : 0.f;
+      const float vb = (b < cnt) ? __ldg(A.v + j0 + b) * split_factor(xb) : 0.f;
       P = make_float4(xa, xb, va, vb);
       V = f2(va * xa, vb * xb);
       Gp = f2(va * xa * xa, vb * xb * xb);
@@ -350,7 +350,7 @@ __device__ __forceinline__ void bwd_rows_body(const BwArgs& A, int rb, int chunk
           if (SPLIT) {
             const float4 Q = sP[buf][j >> 1];
             const float xj = (j & 1) ? Q.y : Q.x;
-            sdv *= ex2_approx(-xj * xj);
+            sdv *= split_factor(xj);
           }
           dst[j] = sdv;
         }
@@ -491,8 +491,8 @@ __device__ __forceinline__ void train_load_pair(const BwArgs& A, const GridTile&
   const bool ina = T.cs + a < T.cnt, inb = T.cs + b < T.cnt;
   const float xa = ina ? A.sc * (gxa - o) : 0.f;
   const float xb = inb ? A.sc * (gxb - o) : 0.f;
-  const float va = ina ? __ldg(A.v + j0 + a) * ex2_approx(-xa * xa) : 0.f;
-  const float vb = inb ? __ldg(A.v + j0 + b) * ex2_approx(-xb * xb) : 0.f;
+  const float va = ina ? __ldg(A.v + j0 + a) * split_factor(xa) : 0.f;
+  const float vb = inb ? __ldg(A.v + j0 + b) * split_factor(xb) : 0.f;
   const float ua = A.sc * (gxa - xc), ub = A.sc * (gxb - xc);
   P = make_float4(xa, xb, va, vb);
   VG = make_float4(va * ua, vb * ub, va * ua * ua, vb * ub * ub);
@@ -882,7 +882,7 @@ __device__ __forceinline__ void dv_rows_body(const BwArgs& A, int rb, int chunk,
       if (SPLIT) {
         const float2 Xp = sm.sX[buf][jj >> 1];
         const float xj = 0.5f * ((jj & 1) ? Xp.y : Xp.x);  // the record holds -2x'
-        sdv *= ex2_approx(-xj * xj);
+        sdv *= split_factor(xj);
       }
       dst[j] = sdv;
     }

@@ -5,20 +5,22 @@
 // raster order: the lens map is continuous, so a tile's ray-traced points
 // stay compact and a row block's bounding box is small.
 //
-// Skipping is exact. In the grid paths the weight of a pair is 2^-t with
-// t = sc^2 d^2 (unsplit form), or 2^(bracket) v~ with
-// bracket = x'^2 - t <= 30.25 (split form). When every pair between a row
-// block and a source sub-segment has t > kSkipT = 170 (measured from the
-// row block's bounding box to the sub-segment's abscissa range and row), both
-// exponent arguments are below -126, where the flush-to-zero exp2 returns
-// exactly 0. So leaving those pairs out changes no result bit.
-// The 14-unit margin over 156 absorbs the FP32 rounding of either distance.
+// What is skipped. The kernel value of a pair is 2^-t with t = sc^2 d^2. Past
+// t = 126 it is below the smallest normal FP32 number, which the kernels' exp2
+// flushes to 0 (ex2.approx.ftz): in the unsplit form, where 2^-t is formed as
+// it is, leaving out pairs with t > kSkipT = 127 changes no result bit (the
+// FP32 rounding of t is below 1e-4 there, the unit of margin covers it). The
+// split form 2^(x'^2 - t) (v 2^(-x'^2)) could still carry a pair to t = 156,
+// at most 2^-126 |v|: there the same line is drawn, so that both forms leave
+// out a kernel value that FP32 does not hold. The line at 170 (156 and a margin)
+// that served both forms before reached 1.34 times the area: at the realistic
+// size 1.18e9 instead of ~0.95e9 evaluated pairs.
 #pragma once
 #include "grid.cuh"
 
 namespace lr {
 
-constexpr float kSkipT = 170.f;
+constexpr float kSkipT = 127.f;
 constexpr int kRowTileW = 32;  // image-tile width of a row block (pixels)
 
 struct RowMap {
@@ -77,7 +79,7 @@ __device__ __forceinline__ bool seg_far(const RowBlockInfo& B, float xa, float x
 // outside is far from the whole box (so are all columns when the row itself is
 // out of reach: then lo > hi). The tile covers columns c0 .. c0 + cnt - 1.
 // The bound is computed in FP32; one column of margin on each side absorbs its
-// rounding, and the threshold's own 14-unit margin covers the kernels'
+// rounding, and the threshold's own unit of margin covers the kernels'
 // rounding of the distances.
 __device__ __forceinline__ void reach_cols(const RowBlockInfo& B, const GridDev& g, float y, float sc, int c0, int cnt,
                                            int& lo, int& hi) {
