@@ -32,26 +32,4 @@ __device__ __forceinline__ float2 grid_point(const GridDev& g, int64_t k) {
   return make_float2(grid_x(g, col), grid_y(g, row));
 }
 
-// 2^(-x^2), the per-source factor of the split exponent (|x| <= 5.5), once per
-// source and tile. It multiplies every pair of its source, so its error does
-// not average out over the rows: rounding x^2 to FP32 would put up to 1e-6 into
-// the exponent, so the square's remainder l goes into the argument, and the
-// hardware exp2 (which truncates) is replaced by a Taylor polynomial of exp
-// rounded to nearest. Row sums of equal weights over 128 x 128 sources, against
-// 64 bits: rms error 1.1e-7 to 1.9e-7 before, 0.8e-7 to 1.3e-7 now.
-__device__ __forceinline__ float split_factor(float x) {
-  const float h = x * x;
-  const float l = fmaf(x, x, -h);
-  const float n = rintf(-h);
-  const float u = 0.69314718f * ((-h - n) - l);  // |u| <= 0.35
-  float p = fmaf(u, 1.f / 5040.f, 1.f / 720.f);
-  p = fmaf(u, p, 1.f / 120.f);
-  p = fmaf(u, p, 1.f / 24.f);
-  p = fmaf(u, p, 1.f / 6.f);
-  p = fmaf(u, p, 0.5f);
-  p = fmaf(u, p, 1.f);
-  p = fmaf(u, p, 1.f);
-  return __int_as_float(__float_as_int(p) + ((int)n << 23));  // n >= -31: stays normal
-}
-
 }  // namespace lr

@@ -82,7 +82,7 @@ __device__ __forceinline__ void load_pair(const SrcDesc& S, const float* __restr
     // (x', v~) of the pair in one 16-byte word (one shared load per pair);
     // the unsplit form stores (-x', v)
     if (split)
-      P = make_float4(xa, xb, va * split_factor(xa), vb * split_factor(xb));
+      P = make_float4(xa, xb, va * ex2_approx(-xa * xa), vb * ex2_approx(-xb * xb));
     else
       P = make_float4(-xa, -xb, va, vb);
     V = f2(0.f, 0.f);

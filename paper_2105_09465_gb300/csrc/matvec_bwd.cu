@@ -99,8 +99,8 @@ __device__ __forceinline__ void bw_load_pair(const BwArgs& A, int t, int p, floa
     const float xb = (b < cnt) ? A.sc * (grid_x(A.src.g, c0 + b) - o) : 0.f;
     if (SPLIT) {
       // split exponent: v~ = v 2^-x'^2 and its first two x' moments
-      const float va = (a < cnt) ? __ldg(A.v + j0 + a) * split_factor(xa) : 0.f;
-      const float vb = (b < cnt) ? __ldg(A.v + j0 + b) * split_factor(xb) : 0.f;
+      const float va = (a < cnt) ? __ldg(A.v + j0 + a) * ex2_approx(-xa * xa) : 0.f;
+      const float vb = (b < cnt) ? __ldg(A.v + j0 + b) * ex2_approx(-xb * xb) : 0.f;
       P = make_float4(xa, xb, va, vb);
       V = f2(va * xa, vb * xb);
       Gp = f2(va * xa * xa, vb * xb * xb);
@@ -350,7 +350,7 @@ __device__ __forceinline__ void bwd_rows_body(const BwArgs& A, int rb, int chunk
           if (SPLIT) {
             const float4 Q = sP[buf][j >> 1];
             const float xj = (j & 1) ? Q.y : Q.x;
-            sdv *= split_factor(xj);
+            sdv *= ex2_approx(-xj * xj);
           }
           dst[j] = sdv;
         }
@@ -446,9 +446,9 @@ __device__ __forceinline__ bool train_compact(const BwArgs& A, int rb) {
 // A tile of a grid-source sweep (the training forward and the d_v sweep):
 // grid row `grow`, columns c0 .. c0 + cnt - 1,
 // the columns [clo, chi] within reach of the row block (empty: clo > chi),
-// and cs, the tile-local column where the tile's records start: clo rounded
-// down to a quarter (4 columns). The sub-segments are laid from cs on, so
-// all but the last one in reach are whole.
+// and cs, the tile-local column where the tile's records start: the first
+// column within kLayT (rowmap.cuh), rounded down to a quarter (4 columns). The
+// sub-segments are laid from cs on, so most in reach are whole.
 struct GridTile {
   int grow, c0, cnt, clo, chi, cs;
   float yt;
@@ -463,20 +463,39 @@ __device__ __forceinline__ GridTile grid_tile(const BwArgs& A, const RowBlockInf
   T.yt = grid_y(A.src.g, grow);
   T.clo = 0;
   T.chi = T.cnt - 1;
-  if (A.info) reach_cols_fast(B, A.src.g, T.yt, A.sc, inv_sc, inv_h, T.c0, T.cnt, T.clo, T.chi);
-  T.cs = T.clo <= T.chi ? (T.clo & ~(2 * kQuarterPairs - 1)) : 0;
+  T.cs = 0;
+  if (A.info) {
+    reach_cols_fast(B, A.src.g, T.yt, A.sc, inv_sc, inv_h, T.c0, T.cnt, kSkipT, T.clo, T.chi);
+    if (T.clo <= T.chi) {
+      int lo, hi;
+      reach_cols_fast(B, A.src.g, T.yt, A.sc, inv_sc, inv_h, T.c0, T.cnt, kLayT, lo, hi);
+      T.cs = lo & ~(2 * kQuarterPairs - 1);
+    }
+  }
   return T;
 }
 
-// What the sweep of a tile needs: its quarters in reach from cs on (every
-// column outside is exactly zero), the grid column of cs, and the row's y.
+// The quarters [qa, qb) in reach, counted from cs (every column outside is
+// exactly zero; none: qa == qb == 0).
+__device__ __forceinline__ void tile_quarters(const GridTile& T, int& qa, int& qb) {
+  const bool any = T.clo <= T.chi;
+  qa = any ? (T.clo - T.cs) / (2 * kQuarterPairs) : 0;
+  qb = any ? (T.chi - T.cs) / (2 * kQuarterPairs) + 1 : 0;
+}
+
+// What the sweep of a tile needs: its quarters in reach, the grid column of
+// cs, and the row's y.
 struct TileRun {
-  int nq, ccs;
+  int qa, qb, ccs;
   float yt;
 };
 
 __device__ __forceinline__ TileRun tile_run(const GridTile& T) {
-  return TileRun{T.clo <= T.chi ? (T.chi - T.cs) / (2 * kQuarterPairs) + 1 : 0, T.c0 + T.cs, T.yt};
+  TileRun r;
+  tile_quarters(T, r.qa, r.qb);
+  r.ccs = T.c0 + T.cs;
+  r.yt = T.yt;
+  return r;
 }
 
 // Pair p of tile T's records: columns cs + 2p and cs + 2p + 1 (zero past the
@@ -491,8 +510,8 @@ __device__ __forceinline__ void train_load_pair(const BwArgs& A, const GridTile&
   const bool ina = T.cs + a < T.cnt, inb = T.cs + b < T.cnt;
   const float xa = ina ? A.sc * (gxa - o) : 0.f;
   const float xb = inb ? A.sc * (gxb - o) : 0.f;
-  const float va = ina ? __ldg(A.v + j0 + a) * split_factor(xa) : 0.f;
-  const float vb = inb ? __ldg(A.v + j0 + b) * split_factor(xb) : 0.f;
+  const float va = ina ? __ldg(A.v + j0 + a) * ex2_approx(-xa * xa) : 0.f;
+  const float vb = inb ? __ldg(A.v + j0 + b) * ex2_approx(-xb * xb) : 0.f;
   const float ua = A.sc * (gxa - xc), ub = A.sc * (gxb - xc);
   P = make_float4(xa, xb, va, vb);
   VG = make_float4(va * ua, vb * ub, va * ua * ua, vb * ub * ub);
@@ -557,7 +576,7 @@ __device__ __forceinline__ void train_rows_body(const BwArgs& A, int rb, int chu
   // tile's reach is found one tile ahead, with its records
   const int segs = A.src.segs;
   int grow = t0 / segs, seg = t0 - grow * segs;
-  TileRun run{0, 0, 0.f};
+  TileRun run{0, 0, 0, 0.f};
   float4 P, VG;
   if (t0 < t1) {
     const GridTile T = grid_tile(A, B, grow, seg, inv_sc, inv_h);
@@ -573,11 +592,11 @@ __device__ __forceinline__ void train_rows_body(const BwArgs& A, int rb, int chu
     const bool wrap = seg + 1 == segs;
     grow = wrap ? grow + 1 : grow;
     seg = wrap ? 0 : seg + 1;
-    TileRun next{0, 0, 0.f};
+    TileRun next{0, 0, 0, 0.f};
     if (t + 1 < t1) {
       const GridTile T = grid_tile(A, B, grow, seg, inv_sc, inv_h);
       next = tile_run(T);
-      train_load_pair(A, T, tid, xc, P, VG);
+      if (next.qb) train_load_pair(A, T, tid, xc, P, VG);
     }
     const float yt = run.yt;
     float dyr[R], ndy2[R];
@@ -589,10 +608,9 @@ __device__ __forceinline__ void train_rows_body(const BwArgs& A, int rb, int chu
       ndy2[r] = -d * d;
       S0[r] = S1[r] = S2[r] = f2(0.f, 0.f);
     }
-    // sub-segments of 4 quarters from cs on: all whole but the last
-    const int nsg = (run.nq + 3) / 4;
-    for (int sg = 0; sg < nsg; ++sg) {
-      const int qn = min(4, run.nq - 4 * sg);
+    // sub-segments of 4 quarters from cs on
+    for (int sg = run.qa / 4; 4 * sg < run.qb; ++sg) {
+      const int q_lo = max(run.qa - 4 * sg, 0), q_hi = min(4, run.qb - 4 * sg);
       const float ds = A.sc * (grid_x(A.src.g, run.ccs + kBwSeg * sg + kBwSeg / 2) - xc);  // delta_s
       float2 q2[R], ar[R];
 #pragma unroll
@@ -603,13 +621,13 @@ __device__ __forceinline__ void train_rows_body(const BwArgs& A, int rb, int chu
         ar[r] = f2(a, a);
       }
       const float4* rec = &sm.sT[buf][2 * sg * (kBwSeg / 2)];
-      if (qn == 4) {
+      if (q_hi - q_lo == 4) {
         // a whole sub-segment: one block without quarter tests
         train_pairs<R, kBwSeg / 2>(rec, q2, ar, S0, S1, S2);
       } else {
 #pragma unroll
-        for (int qq = 0; qq < 3; ++qq) {
-          if (qq >= qn) break;  // the quarters past the reach: exactly zero
+        for (int qq = 0; qq < 4; ++qq) {
+          if (qq < q_lo || qq >= q_hi) continue;  // a quarter out of reach: exactly zero
           train_pairs<R, kQuarterPairs>(rec + 4 * qq, q2, ar, S0, S1, S2);
         }
       }
@@ -720,14 +738,20 @@ __device__ __forceinline__ void dv_load_pair(const BwArgs& A, const GridTile& T,
 
 // What the d_v sweep of a tile needs (see GridTile and TileRun).
 struct DvRun {
-  int nq, cs, c0, cnt;
+  int qa, qb, cs, c0, cnt;
   int64_t j0;
   float yt;
 };
 
 __device__ __forceinline__ DvRun dv_run(const BwArgs& A, const GridTile& T) {
-  return DvRun{T.clo <= T.chi ? (T.chi - T.cs) / (2 * kQuarterPairs) + 1 : 0, T.cs, T.c0, T.cnt,
-               (int64_t)T.grow * A.src.g.W + T.c0, T.yt};
+  DvRun r;
+  tile_quarters(T, r.qa, r.qb);
+  r.cs = T.cs;
+  r.c0 = T.c0;
+  r.cnt = T.cnt;
+  r.j0 = (int64_t)T.grow * A.src.g.W + T.c0;
+  r.yt = T.yt;
+  return r;
 }
 
 // NP consecutive source pairs (records X[0 .. NP)) against the thread's rows:
@@ -798,10 +822,10 @@ __device__ __forceinline__ void dv_rows_body(const BwArgs& A, int rb, int chunk,
   }
   // tile t = grow * segs + seg, stepped without a division per tile; each
   // tile's reach is found one tile ahead, with its records, and its
-  // sub-segments are laid from cs on (all whole but the last)
+  // sub-segments are laid from cs on
   const int segs = A.src.segs;
   int grow = t0 / segs, seg = t0 - grow * segs;
-  DvRun run{0, 0, 0, 0, 0, 0.f};
+  DvRun run{0, 0, 0, 0, 0, 0, 0.f};
   float2 X = f2(0.f, 0.f);
   if (t0 < t1) {
     const GridTile T = grid_tile(A, B, grow, seg, inv_sc, inv_h);
@@ -815,7 +839,7 @@ __device__ __forceinline__ void dv_rows_body(const BwArgs& A, int rb, int chunk,
     const bool wrap = seg + 1 == segs;
     grow = wrap ? grow + 1 : grow;
     seg = wrap ? 0 : seg + 1;
-    DvRun next{0, 0, 0, 0, 0, 0.f};
+    DvRun next{0, 0, 0, 0, 0, 0, 0.f};
     if (t + 1 < t1) {
       const GridTile T = grid_tile(A, B, grow, seg, inv_sc, inv_h);
       next = dv_run(A, T);
@@ -827,9 +851,9 @@ __device__ __forceinline__ void dv_rows_body(const BwArgs& A, int rb, int chunk,
       const float d = A.sc * (yq[r] - run.yt);
       dy2[r] = d * d;
     }
-    const int nsg = (run.nq + 3) / 4;
-    for (int sg = 0; sg < nsg; ++sg) {
-      const int qn = min(4, run.nq - 4 * sg);
+    const int sg0 = run.qa / 4, sg1 = (run.qb + 3) / 4;
+    for (int sg = sg0; sg < sg1; ++sg) {
+      const int q_lo = max(run.qa - 4 * sg, 0), q_hi = min(4, run.qb - 4 * sg);
       const float o = grid_x(A.src.g, run.c0 + run.cs + kBwSeg * sg + kBwSeg / 2);
       // split: (-q, -(q^2 + dy'^2)) against records -2x'; unsplit: (q, dy'^2)
       float2 qa[kDvR], qb[kDvR];
@@ -848,7 +872,7 @@ __device__ __forceinline__ void dv_rows_body(const BwArgs& A, int rb, int chunk,
       }
       float kgs[kBwSeg];
       const float2* Xs = &sm.sX[buf][sg * (kBwSeg / 2)];
-      if (qn == 4) {
+      if (q_hi - q_lo == 4) {
         // a whole sub-segment: one block without quarter tests, in the
         // lane-permuted order
         dv_pairs_perm<SPLIT>(Xs, qa, qb, gq, kgs, tid & 31);
@@ -856,7 +880,7 @@ __device__ __forceinline__ void dv_rows_body(const BwArgs& A, int rb, int chunk,
       } else {
 #pragma unroll
         for (int qi = 0; qi < 4; ++qi) {
-          if (qi >= qn) {  // a quarter past the reach: exactly zero
+          if (qi < q_lo || qi >= q_hi) {  // a quarter out of reach: exactly zero
 #pragma unroll
             for (int c = 4 * qi; c < 4 * qi + 4; ++c) kgs[c] = 0.f;
             continue;
@@ -872,7 +896,7 @@ __device__ __forceinline__ void dv_rows_body(const BwArgs& A, int rb, int chunk,
     float* dst = A.dv_part + (int64_t)rb * A.src.m + run.j0;
     for (int j = tid; j < run.cnt; j += kBwThreads) {
       const int jj = j - run.cs;
-      if (jj < 0 || jj >= nsg * kBwSeg) {
+      if (jj < sg0 * kBwSeg || jj >= sg1 * kBwSeg) {
         dst[j] = 0.f;
         continue;
       }
@@ -882,7 +906,7 @@ __device__ __forceinline__ void dv_rows_body(const BwArgs& A, int rb, int chunk,
       if (SPLIT) {
         const float2 Xp = sm.sX[buf][jj >> 1];
         const float xj = 0.5f * ((jj & 1) ? Xp.y : Xp.x);  // the record holds -2x'
-        sdv *= split_factor(xj);
+        sdv *= ex2_approx(-xj * xj);
       }
       dst[j] = sdv;
     }

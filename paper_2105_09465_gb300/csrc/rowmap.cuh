@@ -12,15 +12,20 @@
 // FP32 rounding of t is below 1e-4 there, the unit of margin covers it). The
 // split form 2^(x'^2 - t) (v 2^(-x'^2)) could still carry a pair to t = 156,
 // at most 2^-126 |v|: there the same line is drawn, so that both forms leave
-// out a kernel value that FP32 does not hold. The line at 170 (156 and a margin)
-// that served both forms before reached 1.34 times the area: at the realistic
-// size 1.18e9 instead of ~0.95e9 evaluated pairs.
+// out a kernel value that FP32 does not hold. A line at 170 (156 and a margin),
+// which served both forms before, takes in 1.34 times the area.
+//
+// Where the work is laid out. The range of grid rows that the chunks of a row
+// block share out, and the columns from which a tile's sub-segments are laid,
+// go by kLayT = 170: they set the order and the rounding of the sums, not
+// what is summed, and a row's sums keep their bits whatever kSkipT leaves out.
 #pragma once
 #include "grid.cuh"
 
 namespace lr {
 
 constexpr float kSkipT = 127.f;
+constexpr float kLayT = 170.f;
 constexpr int kRowTileW = 32;  // image-tile width of a row block (pixels)
 
 struct RowMap {
@@ -29,8 +34,8 @@ struct RowMap {
   int32_t TW, TH;  // tiles per image row / column
 };
 
-// Per row block: bounding box of its rows and the range of source tiles that
-// can hold a contributing pair ([t_lo, t_hi), empty when t_lo >= t_hi).
+// Per row block: bounding box of its rows and the range of source tiles that its
+// chunks share out ([t_lo, t_hi), empty when t_lo >= t_hi).
 struct RowBlockInfo {
   float xlo, ylo, xhi, yhi;
   int32_t t_lo, t_hi, pad0, pad1;
@@ -66,12 +71,12 @@ __device__ __forceinline__ int64_t map_row(const RowMap& m, int64_t n, int rows_
 }
 
 // True when every pair between the box and the source segment
-// [xa, xb] x {y} has sc^2 d^2 > kSkipT.
+// [xa, xb] x {y} has sc^2 d^2 > kLayT.
 __device__ __forceinline__ bool seg_far(const RowBlockInfo& B, float xa, float xb, float y, float sc) {
   const float dx = fmaxf(fmaxf(B.xlo - xb, xa - B.xhi), 0.f);
   const float dy = fmaxf(fmaxf(B.ylo - y, y - B.yhi), 0.f);
   const float sx = sc * dx, sy = sc * dy;
-  return fmaf(sx, sx, sy * sy) > kSkipT;
+  return fmaf(sx, sx, sy * sy) > kLayT;
 }
 
 // Tile-local columns [lo, hi] of a source grid row at ordinate y that can
@@ -101,16 +106,18 @@ __device__ __forceinline__ void reach_cols(const RowBlockInfo& B, const GridDev&
   hi = (int)fh;
 }
 
-// reach_cols with the divisions replaced by the reciprocals inv_sc = 1/sc and
-// inv_h = 1/h (their extra rounding is far inside the one-column margin).
+// reach_cols for the line at t = line, with the divisions replaced by the
+// reciprocals inv_sc = 1/sc and inv_h = 1/h (their extra rounding is far inside
+// the one-column margin).
 __device__ __forceinline__ void reach_cols_fast(const RowBlockInfo& B, const GridDev& g, float y, float sc,
-                                                float inv_sc, float inv_h, int c0, int cnt, int& lo, int& hi) {
+                                                float inv_sc, float inv_h, int c0, int cnt, float line, int& lo,
+                                                int& hi) {
   lo = 0x3fffffff;
   hi = -1;
   if (!(B.xlo <= B.xhi)) return;  // a row block without rows
   const float dy = fmaxf(fmaxf(B.ylo - y, y - B.yhi), 0.f);
   const float sy = sc * dy;
-  const float rem = kSkipT - sy * sy;
+  const float rem = line - sy * sy;
   if (!(rem > 0.f)) return;
   const float w = sqrtf(rem) * inv_sc;  // reach along the row
   const float cl = fmaf(B.xlo - w - g.cx, inv_h, g.c0x);
