@@ -55,19 +55,22 @@ __device__ __forceinline__ float4 warp_box(float4 b) {
 constexpr float4 kEmptyBox = {INFINITY, INFINITY, -INFINITY, -INFINITY};
 
 // ---------------------------------------------------------------------------
-// Prepare: one warp per chunk (lane = slot) writes the chunk's box and record.
-__global__ void __launch_bounds__(256) cull_prep_kernel(const __grid_constant__ CullPrepP P) {
-  const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (c >= P.L.n_chunks) return;  // warp-uniform
+// Prepare: one CTA per group, one warp per chunk at a time (lane = slot). Writes
+// the chunks' boxes and records and, from them, the group's box and smallest
+// reach scale. Bound by the records' writes; one launch for chunks and groups.
+constexpr int kPrepThreads = 1024;
+
+__device__ __forceinline__ void prep_chunk(const CullPrepP& P, int c, int lane, float4& obox, float& oreach) {
   const int64_t i = chunk_point(P.L, c, lane);
   const bool valid = i >= 0;
-  const float2 pv = valid ? P.pts[i] : f2(0.f, 0.f);
+  const float2 pv = valid ? (P.pts ? P.pts[i] : grid_point(P.grid, i)) : f2(0.f, 0.f);
   const float4 box = warp_box(valid ? make_float4(pv.x, pv.y, pv.x, pv.y) : kEmptyBox);
   // an empty slot sits at its chunk's box corner with weight 0
   const float2 p = valid ? pv : f2(box.x, box.y);
   const int RB = rec_bytes(P.nw);
   char* rec = P.rec + (int64_t)c * RB;
+  obox = box;
+  oreach = INFINITY;
   if (lane == 0) P.cbox[c] = box;
   if (!(box.x <= box.z)) {  // an empty chunk: never within reach
     float* w = reinterpret_cast<float*>(rec);
@@ -92,6 +95,7 @@ __global__ void __launch_bounds__(256) cull_prep_kernel(const __grid_constant__ 
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) reach = fminf(reach, __shfl_xor_sync(0xffffffffu, reach, o));
+  oreach = reach;
   if (lane == 0) {
     *reinterpret_cast<float4*>(rec) = box;
     *reinterpret_cast<float4*>(rec + 16) = make_float4((float)n_valid, reach, 0.f, 0.f);
@@ -106,6 +110,12 @@ __global__ void __launch_bounds__(256) cull_prep_kernel(const __grid_constant__ 
   float* w = reinterpret_cast<float*>(rec + kRecHead + kRecXY);  // [nw][32], pairs consecutive
   if (P.kind == kCullOut) {
     for (int k = 0; k < P.nw; ++k) w[k * kChunkPts + lane] = valid ? P.a[i * P.stride + k] : 0.f;
+  } else if (P.kind == kCullLay) {
+    const int nr = P.nw / P.layers;
+    for (int l = 0; l < P.layers; ++l) {
+      const float* al = P.a + ((int64_t)P.lay_src[l] * P.L.n + i) * nr;
+      for (int k = 0; k < nr; ++k) w[(l * nr + k) * kChunkPts + lane] = valid ? P.lay_var[l] * al[k] : 0.f;
+    }
   } else if (P.kind == kCullWin || P.kind == kCullWinRows) {
     w[lane] = valid ? P.a[i] : 0.f;
   } else if (P.kind == kCullWinCols) {
@@ -118,6 +128,33 @@ __global__ void __launch_bounds__(256) cull_prep_kernel(const __grid_constant__ 
     for (int k = 0; k < nr; ++k) {
       w[k * kChunkPts + lane] = valid ? P.a[i * P.stride + k] : 0.f;
       w[(nr + k) * kChunkPts + lane] = valid ? P.b[i * P.stride + k] : 0.f;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kPrepThreads) cull_prep_kernel(const __grid_constant__ CullPrepP P) {
+  __shared__ float4 sbox[kGroupChunks];
+  __shared__ float sreach[kGroupChunks];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = blockIdx.x;
+  if (P.ticket && g == 0 && threadIdx.x < 2) P.ticket[threadIdx.x] = 0;
+  for (int k = warp; k < kGroupChunks; k += kPrepThreads / 32) {
+    float4 box;
+    float reach;
+    prep_chunk(P, g * kGroupChunks + k, lane, box, reach);
+    if (lane == 0) {
+      sbox[k] = box;
+      sreach[k] = reach;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const float4 b = warp_box(box_merge(sbox[lane], sbox[32 + lane]));
+    if (lane == 0) P.gbox[g] = b;
+    if (P.gsc) {
+      float r = fminf(sreach[lane], sreach[32 + lane]);
+#pragma unroll
+      for (int o = 16; o; o >>= 1) r = fminf(r, __shfl_xor_sync(0xffffffffu, r, o));
+      if (lane == 0) P.gsc[g] = r;
     }
   }
 }
@@ -144,29 +181,9 @@ __global__ void __launch_bounds__(256) window_prep_kernel(const float* __restric
   wreach[i] = sqrtf(0.72134752044448170f / lmax);  // sqrt(log2(e) / (2 lambda_max))
 }
 
-// Group boxes (and, with csc, the groups' smallest reach scales): one warp
-// per group.
-__global__ void __launch_bounds__(256) cull_group_box_kernel(const float4* __restrict__ cbox,
-                                                             const float* __restrict__ csc, int n_groups,
-                                                             float4* __restrict__ gbox, float* __restrict__ gsc) {
-  const int g = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (g >= n_groups) return;
-  const int64_t c0 = (int64_t)g * kGroupChunks;
-  float4 b = box_merge(cbox[c0 + lane], cbox[c0 + 32 + lane]);
-  b = warp_box(b);
-  if (lane == 0) gbox[g] = b;
-  if (csc) {
-    float r = fminf(csc[c0 + lane], csc[c0 + 32 + lane]);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) r = fminf(r, __shfl_xor_sync(0xffffffffu, r, o));
-    if (lane == 0) gsc[g] = r;
-  }
-}
-
 // ---------------------------------------------------------------------------
 // The sweep.
-template <int KIND, int NW>
+template <int KIND, int NW, int L = 1>
 struct CullTraits;
 template <int NW>
 struct CullTraits<kCullOut, NW> {
@@ -182,15 +199,15 @@ struct CullTraits<kCullSelf, NW> {  // NW / 2 right-hand sides
 };
 template <>
 struct CullTraits<kCullWin, 1> {
-  static constexpr int K = 1, R = 4, BATCH = 32;
+  static constexpr int K = 1, R = 1, BATCH = 16;
 };
 template <>
 struct CullTraits<kCullWinRows, 1> {
-  static constexpr int K = 6, R = 2, BATCH = 32;
+  static constexpr int K = 6, R = 1, BATCH = 16;
 };
 template <>
 struct CullTraits<kCullWinCols, 4> {
-  static constexpr int K = 3, R = 4, BATCH = 16;
+  static constexpr int K = 3, R = 1, BATCH = 8;
 };
 
 // Row outputs of one row (totals t[K]) for splits == 1, or of the merge.
@@ -202,6 +219,9 @@ __device__ __forceinline__ void cull_finalize(const CullArgs& A, int64_t i, cons
   if constexpr (KIND == kCullOut) {
 #pragma unroll
     for (int k = 0; k < K; ++k) A.out[i * A.nrhs + k] = A.var * t[k];
+  } else if constexpr (KIND == kCullLay) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) A.out[i * A.nrhs + k] = t[k];
   } else if constexpr (KIND == kCullWin) {
     float o = A.wcoef[i].w * t[0];
     if (A.lik_data) {
@@ -295,28 +315,275 @@ __device__ __forceinline__ int cta_compact(bool pred, int value, int* out, int b
   return total;
 }
 
-template <int KIND, int NW>
+template <int NW, int L>
+struct CullTraits<kCullLay, NW, L> {  // NW / L right-hand sides; two batches within 28 KB
+  static constexpr int K = NW / L, R = K <= 2 ? 4 : 2;
+  static constexpr int BATCH = 14336 / rec_bytes(NW) < 32 ? 14336 / rec_bytes(NW) : 32;
+};
+
+// Inclusive scan of one int per thread over the CTA's kCullThreads threads.
+__device__ __forceinline__ int cta_scan(int v, int* wsum, int& total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += u;
+  }
+  if (lane == 31) wsum[w] = v;
+  __syncthreads();
+  int off = 0;
+  total = 0;
+#pragma unroll
+  for (int k = 0; k < kCullThreads / 32; ++k) {
+    if (k < w) off += wsum[k];
+    total += wsum[k];
+  }
+  __syncthreads();
+  return v + off;
+}
+
+constexpr int kScan = 8;  // row blocks a thread and pass of the plan's last CTA
+
+// Parts of a sweep (cull.cuh): per row block the chunks within reach of its
+// box, per group and in all; the last CTA to finish cuts the lists. The row
+// blocks' tests are the sweep's own, so its lists hold exactly these chunks.
+__global__ void __launch_bounds__(kCullThreads) cull_plan_kernel(const __grid_constant__ CullPartsP P) {
+  __shared__ float4 sbox[kCullThreads / 32];
+  __shared__ float sws[kCullThreads / 32];
+  __shared__ int gsel[kCullThreads], wcnt[kCullThreads / 32], stot[kCullThreads / 32];
+  __shared__ int sparts[kScan * kCullThreads];
+  __shared__ int last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rb = blockIdx.x;
+  float4 box = kEmptyBox;
+  float rs = INFINITY;
+  for (int w = tid; w < P.rows_per_cta; w += kCullThreads) {
+    const int64_t i = map_row(P.map, P.n, P.rows_per_cta, rb, w);
+    if (i < 0) continue;
+    const float2 p = P.x[i];
+    box = box_merge(box, make_float4(p.x, p.y, p.x, p.y));
+    if (P.wreach) rs = fminf(rs, P.wreach[i]);
+  }
+  box = warp_box(box);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) rs = fminf(rs, __shfl_xor_sync(0xffffffffu, rs, o));
+  if (lane == 0) {
+    sbox[warp] = box;
+    sws[warp] = rs;
+  }
+  __syncthreads();
+  box = sbox[0];
+  rs = sws[0];
+#pragma unroll
+  for (int k = 1; k < kCullThreads / 32; ++k) {
+    box = box_merge(box, sbox[k]);
+    rs = fminf(rs, sws[k]);
+  }
+  const float sc = P.wreach ? rs : P.sc;
+  int total = 0;  // of this warp's groups
+  uint8_t* gcnt = P.gcnt + (int64_t)rb * P.n_groups;
+  for (int g0 = 0; g0 < P.n_groups; g0 += kCullThreads) {
+    const int g = g0 + tid;
+    const bool near = g < P.n_groups && !boxes_far(box, P.gbox[g], P.gsc ? P.gsc[g] : sc);
+    if (g < P.n_groups && !near) gcnt[g] = 0;
+    const int ng = cta_compact(near, g, gsel, 0, wcnt);
+#pragma unroll 4
+    for (int k = warp; k < ng; k += kCullThreads / 32) {
+      const int c = gsel[k] * kGroupChunks + lane;
+      const bool a = !boxes_far(box, P.cbox[c], P.csc ? P.csc[c] : sc);
+      const bool b = !boxes_far(box, P.cbox[c + 32], P.csc ? P.csc[c + 32] : sc);
+      const int n = __popc(__ballot_sync(0xffffffffu, a)) + __popc(__ballot_sync(0xffffffffu, b));
+      if (lane == 0) gcnt[gsel[k]] = (uint8_t)n;
+      total += n;
+    }
+    __syncthreads();
+  }
+  if (lane == 0) stot[warp] = total;
+  __syncthreads();
+  if (tid == 0) {
+    int t = 0;
+    for (int k = 0; k < kCullThreads / 32; ++k) t += stot[k];
+    P.count[rb] = t;
+    atomicAdd(P.ticket + 1, (unsigned long long)t);
+    __threadfence();
+    last = atomicAdd(P.ticket, 1ull) == (unsigned long long)(P.row_blocks - 1);
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const long long sum = (long long)__ldcg(P.ticket + 1);
+  const long long q = (sum + P.extra - 1) / P.extra;
+  const int Q = (int)(q > kMinPart ? q : kMinPart);
+  int base = 0;
+  for (int k0 = 0; k0 < P.row_blocks; k0 += kScan * kCullThreads) {
+    // kScan row blocks a thread and pass, loaded together
+#pragma unroll
+    for (int j = 0; j < kScan; ++j) {
+      const int k = k0 + j * kCullThreads + tid;
+      const int cnt = k < P.row_blocks ? __ldcg(P.count + k) : 0;
+      sparts[j * kCullThreads + tid] = k < P.row_blocks ? max(1, (cnt + Q - 1) / Q) : 0;
+    }
+    __syncthreads();
+    int mine = 0, tot;
+#pragma unroll
+    for (int j = 0; j < kScan; ++j) mine += sparts[tid * kScan + j];
+    int at = base + cta_scan(mine, wcnt, tot) - mine;
+#pragma unroll
+    for (int j = 0; j < kScan; ++j) {
+      const int k = k0 + tid * kScan + j, parts = sparts[tid * kScan + j];
+      if (k < P.row_blocks) P.start[k] = at;
+      for (int i = 0; i < parts; ++i) P.task_rb[at + i] = k;
+      at += parts;
+    }
+    base += tot;
+    __syncthreads();
+  }
+  if (tid == 0) P.start[P.row_blocks] = base;
+}
+
+// The chunks of one part. list() fills sm.clist with the chunks at positions
+// [p0, p1) of the row block's ascending list (p1 - p0 <= kMaxList). Every warp
+// takes whole groups: a group's first position is known from the counts, so the
+// warps need no barrier between groups.
+struct PartList {
+  int gsel[kCullThreads], gpos[kCullThreads], wcnt[kCullThreads / 32];
+  int bound[2];
+};
+
+template <bool COLS>
+__device__ __noinline__ void part_list(const CullArgs& A, int rb, float4 cb, float sc, int p0, int p1, int* clist,
+                                       PartList& S) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint8_t* gcnt = A.gcnt + (int64_t)rb * A.n_groups;
+  int pos = 0;
+  for (int g0 = 0; g0 < A.n_groups && pos < p1; g0 += kCullThreads) {
+    const int g = g0 + tid;
+    const int c = g < A.n_groups ? gcnt[g] : 0;
+    int tot;
+    const int first = pos + cta_scan(c, S.wcnt, tot) - c;
+    const bool sel = c > 0 && first < p1 && first + c > p0;
+    const int ng = cta_compact(sel, g, S.gsel, 0, S.wcnt);
+    cta_compact(sel, first, S.gpos, 0, S.wcnt);
+    for (int k = warp; k < ng; k += kCullThreads / 32) {
+      const int c0 = S.gsel[k] * kGroupChunks + lane;
+#pragma unroll
+      for (int h = 0, at = S.gpos[k]; h < 2; ++h) {
+        const int ch = c0 + 32 * h;
+        const bool in = !boxes_far(cb, A.cbox[ch], COLS ? A.csc[ch] : sc);
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        const int p = at + __popc(m & ((1u << lane) - 1u));
+        if (in && p >= p0 && p < p1) clist[p - p0] = ch;
+        at += __popc(m);
+      }
+    }
+    pos += tot;
+    __syncthreads();
+  }
+  __syncthreads();
+}
+
+// Unculled sweeps in parts: the chunk index range [bound[0], bound[1]) that
+// holds the part [lo, hi) of the culled list and the chunks out of reach after
+// its entries (before the first entry too for the first part).
+template <bool COLS>
+__device__ __noinline__ void part_bounds(const CullArgs& A, int rb, float4 cb, float sc, int lo, int hi, bool last,
+                                         int* clist, PartList& S) {
+  if (threadIdx.x == 0) {
+    S.bound[0] = 0;
+    S.bound[1] = A.n_chunks;
+  }
+  __syncthreads();
+  if (lo > 0) {
+    part_list<COLS>(A, rb, cb, sc, lo - 1, lo, clist, S);
+    if (threadIdx.x == 0) S.bound[0] = clist[0] + 1;
+  }
+  if (!last) {
+    __syncthreads();
+    part_list<COLS>(A, rb, cb, sc, hi - 1, hi, clist, S);
+    if (threadIdx.x == 0) S.bound[1] = clist[0] + 1;
+  }
+  __syncthreads();
+}
+
+template <int KIND, int NW, int L = 1>
 struct CullSmem {
-  static constexpr int BATCH = CullTraits<KIND, NW>::BATCH;
+  static constexpr int BATCH = CullTraits<KIND, NW, L>::BATCH;
   alignas(128) char buf[2][BATCH * rec_bytes(NW)];
   uint64_t bar[2];
   float4 wbox[kCullThreads / 32];
   float wsc[kCullThreads / 32];
   int clist[kMaxList];
-  int gsel[kCullThreads];
-  int wcnt[kCullThreads / 32];
+  PartList part;
   float red[2 * kCullThreads / 32];
 };
 
-template <int KIND, int NW>
-__global__ void __launch_bounds__(kCullThreads) cull_kernel(const __grid_constant__ CullArgs A) {
-  using T = CullTraits<KIND, NW>;
+// One chunk of a kCullLay sweep with its first NA layers in reach: the pair's
+// squared distance once, per layer one scale, one exp2 and one FMA per
+// right-hand side (5 + L + L H FP32 lanes per pair at NA = L).
+template <int R, int H, int NA>
+__device__ __forceinline__ void lay_chunk(const float4* xy, const float2* wt, const float2 (&NQ)[R],
+                                          const float2 (&NP)[R], const float* c, float2 (&acc)[R][H]) {
+  float2 NC[NA];
+#pragma unroll
+  for (int l = 0; l < NA; ++l) NC[l] = f2(-c[l], -c[l]);
+#pragma unroll 2
+  for (int pp = 0; pp < kChunkPairs; ++pp) {
+    const float4 P = xy[pp];
+    const float2 X = f2(P.x, P.y), Y = f2(P.z, P.w);
+    float2 W[NA * H];
+#pragma unroll
+    for (int w = 0; w < NA * H; ++w) W[w] = wt[w * kChunkPairs + pp];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float2 dx = __fadd2_rn(X, NQ[r]), dy = __fadd2_rn(Y, NP[r]);
+      const float2 t = __ffma2_rn(dy, dy, __fmul2_rn(dx, dx));
+#pragma unroll
+      for (int l = 0; l < NA; ++l) {
+        const float2 e = __fmul2_rn(t, NC[l]);
+        const float2 kk = f2(ex2_approx(e.x), ex2_approx(e.y));
+#pragma unroll
+        for (int h = 0; h < H; ++h) acc[r][h] = __ffma2_rn(kk, W[l * H + h], acc[r][h]);
+      }
+    }
+  }
+}
+
+// Resident CTAs that the compiler leaves registers for (0: its own choice). The
+// windowed kinds ran fastest at 8 (1.07 -> 1.02 ms for a 400 x 400 layer).
+constexpr int cull_min_blocks(int kind) {
+  return kind == kCullWin || kind == kCullWinRows || kind == kCullWinCols ? 8 : 0;
+}
+
+// PARTS: one CTA per part (cull.cuh) instead of one per row block. A kernel of its
+// own: with both forms in one, the self-kernel backward at 2.56M points, which
+// takes one CTA per row block, went from 5.16 to 5.50 ms.
+// Folds the sums of a run of chunks into the row totals (Kahan; only nonzero
+// ones, so that chunks left out and chunks of exact zeros agree bitwise).
+constexpr int kLayFold = 4;  // consecutive chunk indices summed plainly
+
+template <int R, int K>
+__device__ __forceinline__ void lay_fold(float2 (&acc)[R][K], float (&tot)[R][K], float (&comp)[R][K]) {
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int h = 0; h < K; ++h) {
+      const float sum = acc[r][h].x + acc[r][h].y;
+      if (sum != 0.f) kahan_add(tot[r][h], comp[r][h], sum);
+      acc[r][h] = f2(0.f, 0.f);
+    }
+}
+
+template <int KIND, int NW, int L, bool PARTS>
+__global__ void __launch_bounds__(kCullThreads, cull_min_blocks(KIND)) cull_kernel(const __grid_constant__ CullArgs A) {
+  using T = CullTraits<KIND, NW, L>;
   constexpr int R = T::R, K = T::K, BATCH = T::BATCH, RB = rec_bytes(NW);
   constexpr bool WROW = KIND == kCullWin || KIND == kCullWinRows;  // rows carry windows
-  constexpr bool WBWD = KIND == kCullWinRows || KIND == kCullWinCols;
-  __shared__ CullSmem<KIND, NW> sm;
+  __shared__ CullSmem<KIND, NW, L> sm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int rb = blockIdx.x / A.splits, split = blockIdx.x - rb * A.splits;
+  int rb = blockIdx.x;
+  if constexpr (PARTS) {
+    if (rb >= A.start[A.row_blocks]) return;
+    rb = A.task_rb[rb];
+  }
 
   // rows
   float xr[R], yr[R];
@@ -324,7 +591,7 @@ __global__ void __launch_bounds__(kCullThreads) cull_kernel(const __grid_constan
   float4 mybox = kEmptyBox;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    irow[r] = map_row(A.map, A.n, A.rows_per_cta, rb, tid * R + r);
+    irow[r] = cull_row(A.map, A.n, A.rows_per_cta, R, rb, tid, r);
     const float2 p = irow[r] >= 0 ? A.x[irow[r]] : f2(0.f, 0.f);
     xr[r] = p.x;
     yr[r] = p.y;
@@ -392,36 +659,72 @@ __global__ void __launch_bounds__(kCullThreads) cull_kernel(const __grid_constan
       comp[r][k] = 0.f;
     }
 
+  // kCullLay: the plain sums of the current run of kLayFold chunk indices
+  float2 lacc[KIND == kCullLay ? R : 1][KIND == kCullLay ? K : 1];
+  int lgrp = -1;
+  if constexpr (KIND == kCullLay) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int h = 0; h < K; ++h) lacc[r][h] = f2(0.f, 0.f);
+  }
+
   uint32_t phases = 0u;  // bit k: parity of buffer k's next completion
   bool failed = false;
-  const int g_lo = (int)((int64_t)split * A.n_groups / A.splits);
-  const int g_hi = (int)((int64_t)(split + 1) * A.n_groups / A.splits);
-  int gpos = g_lo;
-  while (gpos < g_hi && !failed) {
+  // the listed positions: of the part's list of chunks in reach, of the chunk
+  // indices (parts, not culled), or of the groups (one CTA per row block)
+  int pos = 0, end = A.n_groups;
+  if constexpr (PARTS) {
+    const int p = blockIdx.x - A.start[rb], np = A.start[rb + 1] - A.start[rb], cnt = A.count[rb];
+    pos = (int)((int64_t)p * cnt / np);
+    end = (int)((int64_t)(p + 1) * cnt / np);
+    if (!cull) {
+      part_bounds<KIND == kCullWinCols>(A, rb, cb, sc_b, pos, end, p + 1 == np, sm.clist, sm.part);
+      pos = sm.part.bound[0];
+      end = sm.part.bound[1];
+    }
+  }
+  while (pos < end && !failed) {
     // ---- list the chunks within reach, in ascending order, up to kMaxList
     int count = 0;
-    bool full = false;
-    while (gpos < g_hi && !full) {
-      const int g = gpos + tid;
-      const bool gs = g < g_hi && !(cull && boxes_far(cb, A.gbox[g], KIND == kCullWinCols ? A.gsc[g] : sc_b));
-      const int ng = cta_compact(gs, g, sm.gsel, 0, sm.wcnt);
-      int k = 0;
-      for (; k < ng; ++k) {
-        if (count + kGroupChunks > kMaxList) break;
-        const int gg = sm.gsel[k];
-        const int c = gg * kGroupChunks + (tid & (kGroupChunks - 1));
-        const bool cs = tid < kGroupChunks &&
-                        !(cull ? boxes_far(cb, A.cbox[c], KIND == kCullWinCols ? A.csc[c] : sc_b)
-                               : !(A.cbox[c].x <= A.cbox[c].z));
-        count += cta_compact(cs, c, sm.clist, count, sm.wcnt);
-      }
-      if (k < ng) {
-        gpos = sm.gsel[k];
-        full = true;
+    if constexpr (PARTS) {
+      if (cull) {
+        count = min(end - pos, kMaxList);
+        part_list<KIND == kCullWinCols>(A, rb, cb, sc_b, pos, pos + count, sm.clist, sm.part);
+        pos += count;
       } else {
-        gpos = min(gpos + kCullThreads, g_hi);
+        const int e = min(end, pos + kMaxList);
+        for (int c0 = pos; c0 < e; c0 += kCullThreads) {
+          const int c = c0 + tid;
+          const bool in = c < e && A.cbox[c].x <= A.cbox[c].z;
+          count += cta_compact(in, c, sm.clist, count, sm.part.wcnt);
+        }
+        pos = e;
       }
-      __syncthreads();  // gsel is rewritten by the next window
+    } else {
+      bool full = false;
+      while (pos < end && !full) {
+        const int g = pos + tid;
+        const bool gs = g < end && !(cull && boxes_far(cb, A.gbox[g], KIND == kCullWinCols ? A.gsc[g] : sc_b));
+        const int ng = cta_compact(gs, g, sm.part.gsel, 0, sm.part.wcnt);
+        int k = 0;
+        for (; k < ng; ++k) {
+          if (count + kGroupChunks > kMaxList) break;
+          const int gg = sm.part.gsel[k];
+          const int c = gg * kGroupChunks + (tid & (kGroupChunks - 1));
+          const bool cs = tid < kGroupChunks &&
+                          !(cull ? boxes_far(cb, A.cbox[c], KIND == kCullWinCols ? A.csc[c] : sc_b)
+                                 : !(A.cbox[c].x <= A.cbox[c].z));
+          count += cta_compact(cs, c, sm.clist, count, sm.part.wcnt);
+        }
+        if (k < ng) {
+          pos = sm.part.gsel[k];
+          full = true;
+        } else {
+          pos = min(pos + kCullThreads, end);
+        }
+        __syncthreads();  // gsel is rewritten by the next window
+      }
     }
     // ---- stream the listed chunks through shared memory, two batches in flight
     const int nb = (count + BATCH - 1) / BATCH;
@@ -453,10 +756,10 @@ __global__ void __launch_bounds__(kCullThreads) cull_kernel(const __grid_constan
         const float4 box = *reinterpret_cast<const float4*>(rec);
         const float4 head = *reinterpret_cast<const float4*>(rec + 16);  // (valid points, reach scale)
         if (cull && boxes_far(wb, box, KIND == kCullWinCols ? head.y : sc_w)) continue;  // warp-uniform
-        if (A.count && lane == 0) {
+        if (A.count_out && lane == 0) {
           const float nv = head.x;
-          atomicAdd(A.count, (unsigned long long)(warp_rows * (int)nv));
-          atomicAdd(A.count + 1, (unsigned long long)(32 * R * kChunkPts));
+          atomicAdd(A.count_out, (unsigned long long)(warp_rows * (int)nv));
+          atomicAdd(A.count_out + 1, (unsigned long long)(32 * R * kChunkPts));
         }
         const float4* xy = reinterpret_cast<const float4*>(rec + kRecHead);
         const float2* wt = reinterpret_cast<const float2*>(rec + kRecHead + kRecXY);
@@ -492,13 +795,31 @@ __global__ void __launch_bounds__(kCullThreads) cull_kernel(const __grid_constan
               const float sum = acc[r][w].x + acc[r][w].y;
               if (sum != 0.f) kahan_add(tot[r][w], comp[r][w], sum);
             }
+        } else if constexpr (KIND == kCullLay) {
+          // The layers come in descending length scale, so the ones in reach
+          // of the chunk are the first nact; the others' values are 0.
+          int nact = L;
+          if (cull)
+            while (nact > 1 && boxes_far(wb, box, A.lay_sc[nact - 1])) --nact;  // warp-uniform
+          const int grp = sm.clist[b * BATCH + k] / kLayFold;
+          if (grp != lgrp) {
+            lay_fold<R, K>(lacc, tot, comp);
+            lgrp = grp;
+          }
+          if (nact == 1) lay_chunk<R, K, 1>(xy, wt, NQ, NP, A.lay_c, lacc);
+          if constexpr (L >= 2)
+            if (nact == 2) lay_chunk<R, K, 2>(xy, wt, NQ, NP, A.lay_c, lacc);
+          if constexpr (L >= 3)
+            if (nact == 3) lay_chunk<R, K, 3>(xy, wt, NQ, NP, A.lay_c, lacc);
+          if constexpr (L >= 4)
+            if (nact == 4) lay_chunk<R, K, 4>(xy, wt, NQ, NP, A.lay_c, lacc);
         } else if constexpr (KIND == kCullWin) {
           // G' v = 2^(-|w|^2) v, w = (a d_x + b d_y, c d_y), d = x_j - x_i:
           // 8 FP32 lanes per pair
           float2 acc[R];
 #pragma unroll
           for (int r = 0; r < R; ++r) acc[r] = f2(0.f, 0.f);
-#pragma unroll 2
+#pragma unroll 4
           for (int pp = 0; pp < kChunkPairs; ++pp) {
             const float4 P = xy[pp];
             const float2 X = f2(P.x, P.y), Y = f2(P.z, P.w);
@@ -526,7 +847,7 @@ __global__ void __launch_bounds__(kCullThreads) cull_kernel(const __grid_constan
           for (int r = 0; r < R; ++r)
 #pragma unroll
             for (int k2 = 0; k2 < 6; ++k2) acc[r][k2] = f2(0.f, 0.f);
-#pragma unroll 2
+#pragma unroll 4
           for (int pp = 0; pp < kChunkPairs; ++pp) {
             const float4 P = xy[pp];
             const float2 X = f2(P.x, P.y), Y = f2(P.z, P.w);
@@ -561,7 +882,7 @@ __global__ void __launch_bounds__(kCullThreads) cull_kernel(const __grid_constan
           for (int r = 0; r < R; ++r)
 #pragma unroll
             for (int k2 = 0; k2 < 3; ++k2) acc[r][k2] = f2(0.f, 0.f);
-#pragma unroll 2
+#pragma unroll 4
           for (int pp = 0; pp < kChunkPairs; ++pp) {
             const float4 P = xy[pp];
             const float2 X = f2(P.x, P.y), Y = f2(P.z, P.w);
@@ -638,47 +959,49 @@ __global__ void __launch_bounds__(kCullThreads) cull_kernel(const __grid_constan
       __syncthreads();  // the buffer is refilled two batches on
     }
   }
-  if (failed || A.count) return;
+  if (failed || A.count_out) return;
+  if constexpr (KIND == kCullLay) lay_fold<R, K>(lacc, tot, comp);
 
   // ---- outputs
   float sl = 0.f, sv = 0.f;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    if (irow[r] < 0) continue;
     float t[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) t[k] = (KIND == kCullOut || KIND == kCullWin) ? tot[r][k] - comp[r][k] : tot[r][k];
-    if constexpr (WBWD) {
+    for (int k = 0; k < K; ++k)
+      t[k] = (KIND == kCullOut || KIND == kCullLay || KIND == kCullWin) ? tot[r][k] - comp[r][k] : tot[r][k];
+    if constexpr (KIND == kCullLay) {
+      // a row that is not a number has no reach, but it has a value
+      if (isnan(xr[r]) || isnan(yr[r]))
 #pragma unroll
-      for (int k = 0; k < K; ++k) A.partial[((int64_t)split * K + k) * A.n + irow[r]] = t[k];
-    } else if (A.splits == 1) {
+        for (int k = 0; k < K; ++k) t[k] = NAN;
+    }
+    if constexpr (PARTS) {
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        A.partial[((int64_t)blockIdx.x * K + k) * A.rows_per_cta + r * kCullThreads + tid] = t[k];
+    } else if (irow[r] >= 0) {
       float a, b;
       cull_finalize<KIND, K>(A, irow[r], t, a, b);
       sl += a;
       sv += b;
-    } else {
-#pragma unroll
-      for (int k = 0; k < K; ++k) A.partial[((int64_t)split * K + k) * A.n + irow[r]] = t[k];
     }
   }
-  if (A.splits == 1 && A.scal_part) cta_scalar_partials(sl, sv, A.scal_part, blockIdx.x, sm.red);
+  if (!PARTS && A.scal_part) cta_scalar_partials(sl, sv, A.scal_part, blockIdx.x, sm.red);
 }
 
-// Fixed-order merge of the group-range partials [splits][K][n], then the
-// outputs as the sweep would have written them.
+// Merge of a sweep's parts, then the outputs as the sweep would have written
+// them.
 template <int KIND, int K>
-__global__ void __launch_bounds__(256) cull_merge_kernel(const __grid_constant__ CullArgs A) {
-  __shared__ float red[16];
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kCullThreads) cull_merge_kernel(const __grid_constant__ CullArgs A,
+                                                                  const __grid_constant__ CullParts P) {
+  __shared__ float red[2 * kCullThreads / 32];
+  int rb, slot;
+  const int64_t i = cull_part_row(P, rb, slot);
   float sl = 0.f, sv = 0.f;
-  if (i < A.n) {
+  if (i >= 0) {
     float t[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      float s = 0.f, c = 0.f;
-      for (int sp = 0; sp < A.splits; ++sp) kahan_add(s, c, A.partial[((int64_t)sp * K + k) * A.n + i]);
-      t[k] = s - c;
-    }
+    cull_part_sums<K>(P, rb, slot, t);
     cull_finalize<KIND, K>(A, i, t, sl, sv);
   }
   if (A.scal_part) cta_scalar_partials(sl, sv, A.scal_part, blockIdx.x, red);
@@ -721,12 +1044,36 @@ __global__ void __launch_bounds__(256) cull_scalar_final_kernel(const double* __
 
 int cull_enabled() { return g_pair_culling.load(std::memory_order_relaxed); }
 
-template <int KIND, int NW>
+template <int KIND, int NW, int L = 1>
 static const void* cull_fn() {
-  return reinterpret_cast<const void*>(&cull_kernel<KIND, NW>);
+  return reinterpret_cast<const void*>(&cull_kernel<KIND, NW, L, true>);
 }
 
-static const void* cull_kernel_ptr(int kind, int nw) {
+template <int L, int H>
+static const void* lay_fn() {
+  return cull_fn<kCullLay, L * H, L>();
+}
+
+template <int L>
+static const void* lay_fn_h(int h) {
+  switch (h) {
+    case 1: return lay_fn<L, 1>();
+    case 2: return lay_fn<L, 2>();
+    case 3: return lay_fn<L, 3>();
+    default: return lay_fn<L, 4>();
+  }
+}
+
+static const void* cull_kernel_ptr(int kind, int nw, int layers) {
+  if (kind == kCullLay) {
+    const int h = nw / layers;
+    switch (layers) {
+      case 1: return lay_fn_h<1>(h);
+      case 2: return lay_fn_h<2>(h);
+      case 3: return lay_fn_h<3>(h);
+      default: return lay_fn_h<4>(h);
+    }
+  }
   if (kind == kCullOut) {
     switch (nw) {
       case 1: return cull_fn<kCullOut, 1>();
@@ -747,19 +1094,23 @@ static const void* cull_kernel_ptr(int kind, int nw) {
   }
 }
 
-static int cull_rows_per_thread(int kind, int nw) {
+static int cull_rows_per_thread(int kind, int nw, int layers) {
+  if (kind == kCullLay) return nw / layers <= 2 ? 4 : 2;
   if (kind == kCullOut) return nw <= 2 ? 4 : 2;
-  if (kind == kCullWin || kind == kCullWinCols) return 4;
+  if (kind == kCullWin) return CullTraits<kCullWin, 1>::R;
+  if (kind == kCullWinRows) return CullTraits<kCullWinRows, 1>::R;
+  if (kind == kCullWinCols) return CullTraits<kCullWinCols, 4>::R;
   return (kind == kCullSelf && nw > 2) ? 1 : 2;
 }
 
 lr_status plan_cull(int kind, int nrhs, int64_t n, const lr_grid* qlayout, int64_t m, const lr_grid* slayout,
-                    CullPlan* out) {
+                    CullPlan* out, int layers, bool allow_parts) {
   CullPlan P{};
   P.kind = kind;
-  P.nw = cull_nw(kind, nrhs);
+  P.layers = layers;
+  P.nw = cull_nw(kind, nrhs, layers);
   P.L = make_chunk_layout(slayout, m);
-  P.rows_per_cta = kCullThreads * cull_rows_per_thread(kind, P.nw);
+  P.rows_per_cta = kCullThreads * cull_rows_per_thread(kind, P.nw, layers);
   if (qlayout) {
     P.map.W = qlayout->nx * qlayout->ss;
     P.map.H = qlayout->ny * qlayout->ss;
@@ -772,24 +1123,19 @@ lr_status plan_cull(int kind, int nrhs, int64_t n, const lr_grid* qlayout, int64
   int dev = 0, n_sm = 1, occ = 1;
   LR_CHECK_CUDA(cudaGetDevice(&dev));
   LR_CHECK_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-  LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cull_kernel_ptr(kind, P.nw), kCullThreads, 0));
-  // group ranges per row block: only when the row blocks alone leave most of
-  // the resident CTA slots empty (small query sets). Windowed points differ
-  // in reach by orders of magnitude (pixels next to the lens centre reach
-  // arcseconds, half the image), so the work of a row block does too: there
-  // many more group ranges spread the heaviest row blocks over the GPU.
+  LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cull_kernel_ptr(kind, P.nw, layers), kCullThreads, 0));
+  // In parts (cull.cuh) where the row blocks are under kFewWaves waves of the
+  // resident CTA slots (above, one CTA per row block keeps its sums in
+  // registers, and a band of rows gives the whole problem's bits), and always for windowed points: they differ in reach by orders of
+  // magnitude (pixels next to the lens centre reach arcseconds, half the
+  // image), and so do their row blocks.
   const int64_t slots = (int64_t)(occ > 0 ? occ : 1) * n_sm;
-  // (measured on the 400 x 400 image: 48 for the sweeps whose rows carry the
-  // windows, 16 for the column sweep, against 2 for the stationary sweeps)
-  const int64_t target = (kind == kCullWin || kind == kCullWinRows) ? 48 * slots
-                         : kind == kCullWinCols                       ? 16 * slots
-                                                                      : 2 * slots;
-  int64_t splits = 1;
-  if (P.row_blocks > 0 && P.row_blocks < target) splits = (target + P.row_blocks - 1) / P.row_blocks;
-  if (splits > P.L.n_groups) splits = P.L.n_groups > 0 ? P.L.n_groups : 1;
-  P.splits = (int32_t)splits;
-  P.K = cull_k(kind, P.nw);
-  const bool wbwd = kind == kCullWinRows || kind == kCullWinCols;
+  const bool windowed = kind == kCullWin || kind == kCullWinRows || kind == kCullWinCols;
+  P.R = cull_rows_per_thread(kind, P.nw, layers);
+  P.extra = (int32_t)(kPartWaves * slots);
+  P.parts = P.row_blocks > 0 && P.L.n_groups > 0 &&
+            (windowed || (allow_parts && m > kPartSources && P.row_blocks < kFewWaves * slots));
+  P.K = cull_k(kind, P.nw, layers);
   size_t off = 0;
   P.off_rec = off;
   off += align256((size_t)P.L.n_chunks * rec_bytes(P.nw));
@@ -803,9 +1149,22 @@ lr_status plan_cull(int kind, int nrhs, int64_t n, const lr_grid* qlayout, int64
     P.off_gsc = off;
     off += align256(sizeof(float) * (size_t)(P.L.n_groups > 0 ? P.L.n_groups : 1));
   }
-  P.off_partial = off;
-  if (P.splits > 1 || wbwd) off += align256(sizeof(float) * (size_t)P.splits * P.K * (size_t)n);
-  P.scal_blocks = P.splits > 1 ? (n + 255) / 256 : P.row_blocks * P.splits;
+  const int64_t tasks = P.row_blocks + P.extra;
+  P.off_gcnt = P.off_count = P.off_ticket = P.off_start = P.off_task = P.off_partial = off;
+  if (P.parts) {
+    off += align256((size_t)P.row_blocks * (size_t)P.L.n_groups);
+    P.off_count = off;
+    off += align256(sizeof(int32_t) * (size_t)P.row_blocks);
+    P.off_ticket = off;
+    off += align256(2 * sizeof(unsigned long long));
+    P.off_start = off;
+    off += align256(sizeof(int32_t) * (size_t)(P.row_blocks + 1));
+    P.off_task = off;
+    off += align256(sizeof(int32_t) * (size_t)tasks);
+    P.off_partial = off;
+    off += align256(sizeof(float) * (size_t)tasks * P.K * (size_t)P.rows_per_cta);
+  }
+  P.scal_blocks = P.parts ? P.row_blocks * P.R : P.row_blocks;
   P.off_scal = off;
   off += align256(sizeof(double) * 2 * (size_t)(P.scal_blocks > 0 ? P.scal_blocks : 1));
   P.bytes = off;
@@ -822,11 +1181,32 @@ lr_status launch_window_prep(const float* z, int64_t n, float lengthscale, float
   return LR_OK;
 }
 
+static unsigned long long* plan_ticket(const CullPlan& P, char* ws) {
+  return reinterpret_cast<unsigned long long*>(ws + P.off_ticket);
+}
+
+CullParts cull_parts(const CullPlan& P, int64_t n, const char* ws) {
+  return CullParts{reinterpret_cast<const float*>(ws + P.off_partial),
+                   reinterpret_cast<const int32_t*>(ws + P.off_start), P.map, n, P.rows_per_cta, P.R};
+}
+
+static lr_status launch_prep_kernels(const CullPlan& P, CullPrepP& Q, char* ws, cudaStream_t s) {
+  Q.rec = ws + P.off_rec;
+  Q.cbox = reinterpret_cast<float4*>(ws + P.off_cbox);
+  Q.gbox = reinterpret_cast<float4*>(ws + P.off_gbox);
+  if (P.L.n_chunks == 0) return LR_OK;
+  if (P.parts) Q.ticket = plan_ticket(P, ws);
+  cull_prep_kernel<<<(unsigned)P.L.n_groups, kPrepThreads, 0, s>>>(Q);
+  LR_CHECK_CUDA(cudaGetLastError());
+  return LR_OK;
+}
+
 lr_status launch_cull_prep(const CullPlan& P, const float2* pts, float sc, const float* a, const float* b,
                            int32_t stride, int32_t col, char* ws, cudaStream_t s, const float4* wcoef,
-                           const float* wreach) {
+                           const float* wreach, const lr_grid* grid) {
   CullPrepP Q{};
   Q.pts = pts;
+  if (grid) Q.grid = grid_dev(*grid);
   Q.L = P.L;
   Q.sc = sc;
   Q.kind = P.kind;
@@ -835,38 +1215,60 @@ lr_status launch_cull_prep(const CullPlan& P, const float2* pts, float sc, const
   Q.b = b;
   Q.stride = stride;
   Q.col = col;
-  Q.rec = ws + P.off_rec;
-  Q.cbox = reinterpret_cast<float4*>(ws + P.off_cbox);
-  Q.gbox = reinterpret_cast<float4*>(ws + P.off_gbox);
   Q.wcoef = wcoef;
   Q.wreach = wreach;
   if (P.kind == kCullWinCols) {
     Q.csc = reinterpret_cast<float*>(ws + P.off_csc);
     Q.gsc = reinterpret_cast<float*>(ws + P.off_gsc);
   }
-  if (P.L.n_chunks == 0) return LR_OK;
-  const int64_t warps = P.L.n_chunks;
-  cull_prep_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(Q);
-  LR_CHECK_CUDA(cudaGetLastError());
-  cull_group_box_kernel<<<(unsigned)(((int64_t)P.L.n_groups * 32 + 255) / 256), 256, 0, s>>>(
-      Q.cbox, Q.csc, P.L.n_groups, Q.gbox, Q.gsc);
-  LR_CHECK_CUDA(cudaGetLastError());
-  return LR_OK;
+  return launch_prep_kernels(P, Q, ws, s);
 }
 
-template <int KIND, int NW>
+lr_status launch_cull_prep_layers(const CullPlan& P, const float2* pts, const lr_grid* grid, const float* v,
+                                  const int32_t* src, const float* var, char* ws, cudaStream_t s) {
+  CullPrepP Q{};
+  Q.pts = pts;
+  if (grid) Q.grid = grid_dev(*grid);
+  Q.L = P.L;
+  Q.kind = P.kind;
+  Q.nw = P.nw;
+  Q.a = v;
+  Q.layers = P.layers;
+  for (int l = 0; l < P.layers; ++l) {
+    Q.lay_src[l] = src[l];
+    Q.lay_var[l] = var[l];
+  }
+  return launch_prep_kernels(P, Q, ws, s);
+}
+
+template <int KIND, int NW, int L = 1>
 static lr_status launch_sweep_t(const CullPlan& P, const CullArgs& A, cudaStream_t s) {
-  const unsigned grid = (unsigned)(P.row_blocks * P.splits);
-  cull_kernel<KIND, NW><<<grid, kCullThreads, 0, s>>>(A);
+  constexpr bool WINDOWED = KIND == kCullWin || KIND == kCullWinRows || KIND == kCullWinCols;
+  if (P.parts)
+    cull_kernel<KIND, NW, L, true><<<(unsigned)(P.row_blocks + P.extra), kCullThreads, 0, s>>>(A);
+  else if constexpr (!WINDOWED)
+    cull_kernel<KIND, NW, L, false><<<(unsigned)P.row_blocks, kCullThreads, 0, s>>>(A);
   LR_CHECK_CUDA(cudaGetLastError());
   // the windowed backward kinds leave their partials to the caller's merge
   if constexpr (KIND != kCullWinRows && KIND != kCullWinCols) {
-    if (P.splits > 1 && !A.count) {
-      cull_merge_kernel<KIND, CullTraits<KIND, NW>::K><<<(unsigned)((A.n + 255) / 256), 256, 0, s>>>(A);
+    if (P.parts && !A.count_out) {
+      CullParts M{A.partial, A.start, P.map, A.n, P.rows_per_cta, P.R};
+      cull_merge_kernel<KIND, CullTraits<KIND, NW, L>::K>
+          <<<(unsigned)(P.row_blocks * P.R), kCullThreads, 0, s>>>(A, M);
       LR_CHECK_CUDA(cudaGetLastError());
     }
   }
   return LR_OK;
+}
+
+template <int L>
+static lr_status launch_lay_h(const CullPlan& P, const CullArgs& A, cudaStream_t s) {
+  switch (P.K) {
+    case 1: return launch_sweep_t<kCullLay, L, L>(P, A, s);
+    case 2: return launch_sweep_t<kCullLay, 2 * L, L>(P, A, s);
+    case 3: return launch_sweep_t<kCullLay, 3 * L, L>(P, A, s);
+    default: return launch_sweep_t<kCullLay, 4 * L, L>(P, A, s);
+  }
 }
 
 lr_status launch_cull_sweep(const CullPlan& P, CullArgs A, char* ws, int timer_id, cudaStream_t s) {
@@ -879,14 +1281,41 @@ lr_status launch_cull_sweep(const CullPlan& P, CullArgs A, char* ws, int timer_i
   A.gbox = reinterpret_cast<const float4*>(ws + P.off_gbox);
   A.n_chunks = P.L.n_chunks;
   A.n_groups = P.L.n_groups;
-  A.splits = P.splits;
-  A.partial = reinterpret_cast<float*>(ws + P.off_partial);
+  A.row_blocks = (int32_t)P.row_blocks;
   if (P.kind == kCullWinCols) {
     A.csc = reinterpret_cast<const float*>(ws + P.off_csc);
     A.gsc = reinterpret_cast<const float*>(ws + P.off_gsc);
   }
   A.fault = fault_ptr();
   LR_REQUIRE(A.fault != nullptr, "could not resolve the device fault word");
+  if (P.parts) {
+    CullPartsP Q{};
+    Q.x = A.x;
+    Q.n = A.n;
+    Q.map = P.map;
+    Q.rows_per_cta = P.rows_per_cta;
+    Q.row_blocks = (int32_t)P.row_blocks;
+    Q.n_groups = P.L.n_groups;
+    Q.extra = P.extra;
+    Q.sc = A.sc;
+    Q.wreach = A.wreach;
+    Q.csc = A.csc;
+    Q.gsc = A.gsc;
+    Q.cbox = A.cbox;
+    Q.gbox = A.gbox;
+    Q.gcnt = reinterpret_cast<uint8_t*>(ws + P.off_gcnt);
+    Q.count = reinterpret_cast<int32_t*>(ws + P.off_count);
+    Q.start = reinterpret_cast<int32_t*>(ws + P.off_start);
+    Q.task_rb = reinterpret_cast<int32_t*>(ws + P.off_task);
+    Q.ticket = plan_ticket(P, ws);
+    cull_plan_kernel<<<(unsigned)P.row_blocks, kCullThreads, 0, s>>>(Q);
+    LR_CHECK_CUDA(cudaGetLastError());
+    A.start = Q.start;
+    A.task_rb = Q.task_rb;
+    A.count = Q.count;
+    A.gcnt = Q.gcnt;
+    A.partial = reinterpret_cast<float*>(ws + P.off_partial);
+  }
   if (timer_id >= 0) ktimer_begin(timer_id, s);
   lr_status st;
   if (P.kind == kCullOut) {
@@ -895,6 +1324,13 @@ lr_status launch_cull_sweep(const CullPlan& P, CullArgs A, char* ws, int timer_i
       case 2: st = launch_sweep_t<kCullOut, 2>(P, A, s); break;
       case 3: st = launch_sweep_t<kCullOut, 3>(P, A, s); break;
       default: st = launch_sweep_t<kCullOut, 4>(P, A, s); break;
+    }
+  } else if (P.kind == kCullLay) {
+    switch (P.layers) {
+      case 1: st = launch_lay_h<1>(P, A, s); break;
+      case 2: st = launch_lay_h<2>(P, A, s); break;
+      case 3: st = launch_lay_h<3>(P, A, s); break;
+      default: st = launch_lay_h<4>(P, A, s); break;
     }
   } else if (P.kind == kCullMom) {
     st = launch_sweep_t<kCullMom, 1>(P, A, s);
@@ -1000,7 +1436,7 @@ extern "C" lr_status lr_cull_pairs_evaluated(const lr_points* query, const lr_po
   A.c = (float)c;
   A.nrhs = 1;
   A.stride = 1;
-  A.count = cnt;
+  A.count_out = cnt;
   st = launch_cull_sweep(P, A, ws, -1, s);
   if (st != LR_OK) return done(st);
   unsigned long long h[2] = {0, 0};

@@ -38,6 +38,19 @@
 // when the rows carry the windows, of the chunk (stored with its box) when
 // the sources do.
 //
+// Parts. A sweep whose row blocks alone would leave the GPU idle or unevenly
+// loaded (few rows, or rows that differ in reach) is cut into parts of about
+// equal work: cull_plan_kernel counts, per row block and group, the chunks
+// within reach, and cuts each row block's ascending list of them into parts of
+// at most Q chunks, Q the total over kPartWaves resident waves (at least
+// kMinPart). One CTA takes one part; a part's sums go to its own rows of the
+// partials and a merge adds a row's parts in order (Kahan). Cutting by the
+// chunks in reach, not by group ranges, is what balances it: of the 91 group
+// ranges that a row block of a 400 x 400 image-plane layer had before, most held
+// nothing in reach and the rest differed by 100 x, and every range wrote its
+// partials. The cuts depend on the points alone (culled counts, whether or not
+// the sweep culls), so culled and unculled sweeps still agree bitwise.
+//
 // Window precision. At the paper's narrow image-plane kernels (2 to 10 mas)
 // the windows of magnified pixels are thin ellipses: C_i has a condition
 // number kappa of order 100. Forming det C_i or the quadratic form
@@ -125,16 +138,22 @@ enum CullKind : int32_t {
   kCullWinCols = 5,  // windowed backward, column sums: the sources (the
                      // windowed points) carry their window constants (a, b, c)
                      // and g N as their four weights
+  kCullLay = 6,      // layers x nrhs weights: var_l v_l, layers in descending
+                     // length scale (forward, sum of layers)
 };
 
-__host__ __device__ constexpr int cull_nw(int kind, int nrhs) {
-  return kind == kCullOut ? nrhs
+constexpr int kMaxLayers = 4;
+
+__host__ __device__ constexpr int cull_nw(int kind, int nrhs, int layers = 1) {
+  return kind == kCullOut   ? nrhs
+         : kind == kCullLay ? layers * nrhs
                           : (kind == kCullSelf ? 2 * nrhs : (kind == kCullWinCols ? 4 : 1));
 }
 
 // Sums per row of a sweep.
-__host__ __device__ constexpr int cull_k(int kind, int nw) {
-  return kind == kCullOut ? nw
+__host__ __device__ constexpr int cull_k(int kind, int nw, int layers = 1) {
+  return kind == kCullOut   ? nw
+         : kind == kCullLay ? nw / layers
                           : kind == kCullMom ? 4
                           : kind == kCullSelf ? 7 * (nw / 2)
                           : kind == kCullWin ? 1
@@ -147,7 +166,8 @@ lr_status launch_window_prep(const float* z, int64_t n, float lengthscale, float
                              cudaStream_t s);
 
 struct CullPrepP {
-  const float2* pts;  // [n] source points
+  const float2* pts;  // [n] source points, or NULL: the points of `grid`
+  GridDev grid;
   ChunkLayout L;
   float sc;
   int32_t kind, nw;
@@ -163,10 +183,17 @@ struct CullPrepP {
   const float* wreach;
   float* csc;         // [n_chunks]
   float* gsc;         // [n_groups]
+  unsigned long long* ticket;  // the plan kernel's block counter and total, zeroed here (or NULL)
+  // kCullLay: a is v [layers][m][nrhs]; layer k of the records is a's layer
+  // lay_src[k], its weights times lay_var[k]
+  int32_t layers;
+  int32_t lay_src[kMaxLayers];
+  float lay_var[kMaxLayers];
 };
 
 // Outputs of a culled sweep, by kind:
 //  kCullOut:  out[i][r] = var * sum_j k_ij v_j[r]
+//  kCullLay:  out[i][r] = sum_l sum_j 2^(-lay_c[l] d_ij^2) w_lj[r]
 //  kCullMom:  row moments of a over the sources:
 //             A = sum k a, Bx/By = sum k a (x_j - x_i), C = sum k a d^2;
 //             with g == NULL they are written to mom [4][n] (and out = var A);
@@ -180,8 +207,8 @@ struct CullPrepP {
 //             sums S = sum v G', P = sum v G' u, Q = sum v G' u u^T (xx, xy, yy)
 //  kCullWinCols: per row (a source of the windowed reduction), with
 //             d = x_i - y_j and u = k^2 C_j^-1 d, T = sum gN G', U = sum gN G' u
-//             The two backward kinds write partial[split][K][n] whatever the
-//             split count; the windowed backward merges them.
+//             The two backward kinds are always cut into parts; the windowed
+//             backward merges them.
 struct CullArgs {
   const float2* x;   // [n] query points
   int64_t n;
@@ -194,7 +221,14 @@ struct CullArgs {
   const float4* cbox;
   const float4* gbox;
   int32_t n_chunks, n_groups;
-  int32_t splits;    // group ranges per row block (> 1: partials + merge)
+  // parts (start != NULL): CTA t takes part t - start[task_rb[t]] of row block
+  // task_rb[t]; gcnt [row_blocks][n_groups] and count [row_blocks] are the
+  // chunks within reach
+  const int32_t* start;    // [row_blocks + 1]
+  const int32_t* task_rb;
+  const int32_t* count;
+  const uint8_t* gcnt;
+  int32_t row_blocks;
   int32_t nrhs;      // kCullOut: weights per source
   float var;
   float dx_scale;    // var / l^2
@@ -208,7 +242,7 @@ struct CullArgs {
   int32_t dx_accumulate;  // add into d_x (later right-hand sides)
   float* d_v;        // kCullSelf: [n][stride] at column col
   double* scal_part; // [partial blocks][2]: d_l, d_var partials
-  float* partial;    // splits > 1: [splits][K][n]
+  float* partial;    // parts: [part][K][rows_per_cta], rows in (row of the thread, thread) order
   const float4* wcoef;  // kCullWin, kCullWinRows: the rows' window constants (a, b, c, N)
   const float* wreach;  // and reach scales (launch_window_prep)
   // kCullWin with a Gaussian likelihood in the epilogue (lik_data != NULL):
@@ -220,38 +254,140 @@ struct CullArgs {
   float* lik_g;
   const float* csc;  // kCullWinCols: reach scales of the chunks and groups
   const float* gsc;
+  // kCullLay: log2(e) / (2 l^2) per layer in descending length scale, and the
+  // skipping test's scales (their square roots; A.sc is the first)
+  float lay_c[kMaxLayers], lay_sc[kMaxLayers];
   int* fault;        // device fault word (a bulk-copy wait that ran out)
-  unsigned long long* count;  // diagnostic: [0] valid pairs, [1] pair slots evaluated
-                              // (non-NULL: count only, no outputs written)
+  unsigned long long* count_out;  // diagnostic: [0] valid pairs, [1] pair slots evaluated
+                                  // (non-NULL: count only, no outputs written)
 };
 
-// Plan of one culled sweep: source chunks, query row blocks, group ranges per
-// row block and the workspace offsets (records, boxes, partials, scalars).
+constexpr int kPartWaves = 4;  // parts: the resident CTA slots times this, beyond one per row block
+constexpr int kFewWaves = 2;   // a stationary sweep of fewer waves of row blocks is cut into parts
+constexpr int kPartSources = 512;  // up to so many sources the plan and merge launches cost more than they give
+constexpr int kMinPart = 4;    // fewest chunks worth a part of their own
+
+// The plan kernel's arguments (see "Parts" above).
+struct CullPartsP {
+  const float2* x;
+  int64_t n;
+  RowMap map;
+  int32_t rows_per_cta, row_blocks, n_groups, extra;
+  float sc;
+  const float* wreach;  // rows that carry windows: their reach scales
+  const float* csc;     // kCullWinCols: reach scales of the chunks and groups
+  const float* gsc;
+  const float4* cbox;
+  const float4* gbox;
+  uint8_t* gcnt;
+  int32_t* count;
+  int32_t* start;
+  int32_t* task_rb;
+  unsigned long long* ticket;  // [0] CTAs done, [1] chunks in reach in all
+};
+
+// The partials of a sweep in parts, for its merge: one thread per (row of a
+// thread, thread), kCullThreads threads a block, R blocks per row block.
+struct CullParts {
+  const float* partial;
+  const int32_t* start;
+  RowMap map;
+  int64_t n;
+  int32_t rows_per_cta, R;
+};
+
+// Index of row r (of the thread's R) of thread tid in row block rb, or -1
+// (padding). Rows in an image layout come in tiles of kCullTileW pixels a row;
+// a warp's 32 R rows are an 8 x 4 R block of pixels (16 x 8 at R = 4), as square
+// as they come: the box of a warp is what decides which chunks it evaluates.
+__device__ __forceinline__ int64_t cull_row(const RowMap& m, int64_t n, int rows_per_cta, int R, int rb, int tid,
+                                            int r) {
+  int w = tid * R + r;
+  if (m.W && R < 4) {
+    const int warp = tid >> 5, l = (tid & 31) * R + r;
+    w = ((warp >> 1) * 4 * R + (l >> 3)) * kCullTileW + (warp & 1) * 8 + (l & 7);
+  }
+  return map_row(m, n, rows_per_cta, rb, w);
+}
+
+// Row index (or -1, padding) of this merge thread; rb and slot name its partials.
+__device__ __forceinline__ int64_t cull_part_row(const CullParts& P, int& rb, int& slot) {
+  rb = blockIdx.x / P.R;
+  const int r = blockIdx.x - rb * P.R;
+  slot = r * kCullThreads + threadIdx.x;
+  return cull_row(P.map, P.n, P.rows_per_cta, P.R, rb, threadIdx.x, r);
+}
+
+// The row's K sums over its parts in order (Kahan), 4 parts' loads in flight: a
+// wide window's row block has ~60 parts, and one after the other their latency
+// was the merge's time (46 us for the 6 sums of a 400 x 400 image-plane layer).
+template <int K>
+__device__ __forceinline__ void cull_part_sums(const CullParts& P, int rb, int slot, float (&s)[K]) {
+  const int t0 = P.start[rb], t1 = P.start[rb + 1];
+  const int64_t step = P.rows_per_cta;
+  const float* p = P.partial + (int64_t)t0 * K * step + slot;
+  float c[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) s[k] = c[k] = 0.f;
+  for (int t = t0; t < t1; t += 4, p += 4 * K * step) {
+    float v[4][K];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int k = 0; k < K; ++k) v[j][k] = t + j < t1 ? p[(j * K + k) * step] : 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const float y = v[j][k] - c[k];
+        const float u = s[k] + y;
+        c[k] = (u - s[k]) - y;
+        s[k] = u;
+      }
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) s[k] -= c[k];
+}
+
+// Plan of one culled sweep: source chunks, query row blocks, parts and the
+// workspace offsets (records, boxes, counts, partials, scalars).
 struct CullPlan {
-  int32_t kind, nw, K;
+  int32_t kind, nw, K, layers;
   ChunkLayout L;
   RowMap map;
   int32_t rows_per_cta;
   int64_t row_blocks;
-  int32_t splits;
+  int32_t R;            // rows per thread
+  int32_t parts;        // cut into parts (else one CTA per row block)
+  int32_t extra;        // parts beyond one per row block
   int64_t scal_blocks;  // blocks that write scalar partials
-  size_t off_rec, off_cbox, off_gbox, off_csc, off_gsc, off_partial, off_scal, bytes;
+  size_t off_rec, off_cbox, off_gbox, off_csc, off_gsc, off_gcnt, off_count, off_ticket, off_start, off_task, off_partial,
+      off_scal, bytes;
 };
 
 // 1 unless lr_set_pair_culling(0) switched exact skipping off.
 int cull_enabled();
 // Plans a sweep of n query points (image layout qlayout or NULL) against m
-// sources (layout slayout or NULL) with nrhs right-hand sides (kCullOut).
+// sources (layout slayout or NULL) with nrhs right-hand sides (kCullOut,
+// kCullLay) and, for kCullLay, `layers` layers. allow_parts = false keeps a
+// stationary sweep to one CTA per row block (a smaller workspace).
 lr_status plan_cull(int kind, int nrhs, int64_t n, const lr_grid* qlayout, int64_t m, const lr_grid* slayout,
-                    CullPlan* P);
-// Writes the source chunks' boxes and records into ws (offsets of P):
+                    CullPlan* P, int layers = 1, bool allow_parts = true);
+// The partials of a sweep that ran in parts in workspace ws.
+CullParts cull_parts(const CullPlan& P, int64_t n, const char* ws);
+// Writes the source chunks' boxes and records into ws (offsets of P); pts ==
+// NULL: the points of `grid`.
 // kCullOut weights a [m][stride] (all nrhs columns), kCullMom column col of a,
 // kCullSelf column col of a and of b, kCullWin / kCullWinRows a [m],
 // kCullWinCols the points' window constants (wcoef, wreach) and g = a [m].
 lr_status launch_cull_prep(const CullPlan& P, const float2* pts, float sc, const float* a, const float* b,
                            int32_t stride, int32_t col, char* ws, cudaStream_t s, const float4* wcoef = nullptr,
-                           const float* wreach = nullptr);
-// The sweep (and merge when P.splits > 1); A carries the kind's outputs.
+                           const float* wreach = nullptr, const lr_grid* grid = nullptr);
+// The records of a kCullLay sweep: v [layers][m][nrhs], record layer k taken
+// from v's layer src[k] times var[k].
+lr_status launch_cull_prep_layers(const CullPlan& P, const float2* pts, const lr_grid* grid, const float* v,
+                                  const int32_t* src, const float* var, char* ws, cudaStream_t s);
+// The sweep (with its plan and merge when it runs in parts); A carries the kind's outputs.
 // timer_id: an LR_KT_* launch-timer id, or -1.
 lr_status launch_cull_sweep(const CullPlan& P, CullArgs A, char* ws, int timer_id, cudaStream_t s);
 // d_len, d_var from nblk scalar partials (fixed order, FP64).

@@ -332,7 +332,8 @@ struct MvPlan {
   size_t off_qbeta, off_sbeta, off_partial, off_info, off_cull, bytes;
 };
 
-static lr_status plan_matvec(const lr_points* q, const lr_points* s, int32_t nrhs, bool have_beta_out, MvPlan* P) {
+static lr_status plan_matvec(const lr_points* q, const lr_points* s, int32_t nrhs, bool have_beta_out, MvPlan* P,
+                             bool allow_parts = true) {
   lr_status st = validate_points(q, "gp_kernel_matvec(query)", false);
   if (st != LR_OK) return st;
   if (s) {
@@ -349,9 +350,9 @@ static lr_status plan_matvec(const lr_points* q, const lr_points* s, int32_t nrh
   p.s_raytrace = !p.self && has_lens(s);
   p.s_grid = !p.self && !p.s_raytrace && s->xy == nullptr;
   LR_REQUIRE(nrhs >= 1 && nrhs <= 4, "gp_kernel_matvec: nrhs = %d; 1..4 right-hand sides", nrhs);
-  // several right-hand sides over grid sources: the grid's points are
-  // written out and reduced by the culled sweep, which shares each pair's
-  // exp2 across the right-hand sides
+  // several right-hand sides over grid sources: the grid's points go into the
+  // culled sweep's records, and the sweep shares each pair's exp2 across the
+  // right-hand sides
   p.s_mat = p.s_grid && nrhs > 1;
   if (p.s_mat) p.s_grid = false;
   size_t off = 0;
@@ -359,12 +360,12 @@ static lr_status plan_matvec(const lr_points* q, const lr_points* s, int32_t nrh
   p.off_qbeta = off;
   if (need_qbuf) off += align256(sizeof(float2) * (size_t)p.n);
   p.off_sbeta = off;
-  if (p.s_raytrace || p.s_mat) off += align256(sizeof(float2) * (size_t)p.m);
+  if (p.s_raytrace) off += align256(sizeof(float2) * (size_t)p.m);
   const lr_grid* layout = query_layout(q);
   if (!p.s_grid) {
     // explicit, ray-traced or self sources: the culled sweep
     const lr_grid* slayout = p.self ? layout : query_layout(s);
-    st = plan_cull(kCullOut, nrhs, p.n, layout, p.m, slayout, &p.cull);
+    st = plan_cull(kCullOut, nrhs, p.n, layout, p.m, slayout, &p.cull, 1, allow_parts);
     if (st != LR_OK) return st;
     p.off_cull = off;
     off += p.cull.bytes;
@@ -407,12 +408,10 @@ extern "C" lr_status lr_matvec_workspace_size(const lr_points* query, const lr_p
   return LR_OK;
 }
 
-extern "C" lr_status gp_kernel_matvec(const lr_points* query, const lr_points* source, const float* v, int32_t nrhs,
-                                      float lengthscale, float variance, float* out, float* beta_out,
-                                      void* workspace, size_t workspace_bytes, lr_stream stream) {
-  MvPlan P;
-  lr_status st = plan_matvec(query, source, nrhs, beta_out != nullptr, &P);
-  if (st != LR_OK) return st;
+static lr_status run_matvec(const MvPlan& P, const lr_points* query, const lr_points* source, const float* v,
+                            float lengthscale, float variance, float* out, float* beta_out, void* workspace,
+                            size_t workspace_bytes, lr_stream stream) {
+  lr_status st;
   LR_REQUIRE(isfinite(lengthscale) && lengthscale > 0.f, "gp_kernel_matvec: lengthscale = %g must be > 0",
              (double)lengthscale);
   LR_REQUIRE(isfinite(variance), "gp_kernel_matvec: variance is not finite");
@@ -447,12 +446,11 @@ extern "C" lr_status gp_kernel_matvec(const lr_points* query, const lr_points* s
   S.segs = P.segs;
   if (P.self) {
     S.xy = xq;
-  } else if (P.s_raytrace || P.s_mat) {
+  } else if (P.s_raytrace) {
     float2* sb = reinterpret_cast<float2*>(ws + P.off_sbeta);
-    st = P.s_raytrace ? launch_raytrace(source, sb, nullptr, s) : launch_grid_points(source->grid, sb, s);
-    if (st != LR_OK) return st;
+    if ((st = launch_raytrace(source, sb, nullptr, s)) != LR_OK) return st;
     S.xy = sb;
-  } else if (P.s_grid) {
+  } else if (P.s_grid || P.s_mat) {
     S.xy = nullptr;
     S.g = grid_dev(source->grid);
   } else {
@@ -462,7 +460,8 @@ extern "C" lr_status gp_kernel_matvec(const lr_points* query, const lr_points* s
   if (!P.s_grid) {
     // explicit, ray-traced or self sources: culled sweep over chunk records
     char* cws = ws + P.off_cull;
-    st = launch_cull_prep(P.cull, S.xy, sc, v, nullptr, P.nrhs, 0, cws, s);
+    st = launch_cull_prep(P.cull, S.xy, sc, v, nullptr, P.nrhs, 0, cws, s, nullptr, nullptr,
+                          P.s_mat ? &source->grid : nullptr);
     if (st != LR_OK) return st;
     CullArgs C{};
     C.x = xq;
@@ -501,6 +500,15 @@ extern "C" lr_status gp_kernel_matvec(const lr_points* query, const lr_points* s
     LR_CHECK_CUDA(cudaGetLastError());
   }
   return LR_OK;
+}
+
+extern "C" lr_status gp_kernel_matvec(const lr_points* query, const lr_points* source, const float* v, int32_t nrhs,
+                                      float lengthscale, float variance, float* out, float* beta_out,
+                                      void* workspace, size_t workspace_bytes, lr_stream stream) {
+  MvPlan P;
+  const lr_status st = plan_matvec(query, source, nrhs, beta_out != nullptr, &P);
+  if (st != LR_OK) return st;
+  return run_matvec(P, query, source, v, lengthscale, variance, out, beta_out, workspace, workspace_bytes, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -542,6 +550,9 @@ extern "C" lr_status gp_kernel_matvec_static_scratch(const lr_points* query, con
                                                      float* out, float* beta_out, lr_stream stream) {
   MvPlan P;
   lr_status st = plan_matvec(query, source, nrhs, beta_out != nullptr, &P);
+  // a sweep in parts keeps partials: where they do not fit, one CTA per row block
+  if (st == LR_OK && P.bytes > kStaticScratchBytes)
+    st = plan_matvec(query, source, nrhs, beta_out != nullptr, &P, false);
   if (st != LR_OK) return st;
   LR_REQUIRE(P.bytes <= kStaticScratchBytes,
              "gp_kernel_matvec_static_scratch: this problem needs %zu bytes of scratch but the static scratch "
@@ -553,6 +564,5 @@ extern "C" lr_status gp_kernel_matvec_static_scratch(const lr_points* query, con
   // Every word of scratch this call reads is written earlier in the same
   // call (query/source points, then each chunk partial exactly once), so
   // nothing needs clearing between calls.
-  return gp_kernel_matvec(query, source, v, nrhs, lengthscale, variance, out, beta_out, scratch,
-                          kStaticScratchBytes, stream);
+  return run_matvec(P, query, source, v, lengthscale, variance, out, beta_out, scratch, kStaticScratchBytes, stream);
 }

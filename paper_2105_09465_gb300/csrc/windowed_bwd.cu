@@ -21,18 +21,9 @@ namespace lr {
 
 constexpr float kTwoLn2 = 1.3862943611198906f;
 
-__device__ __forceinline__ void wb_kahan(float& s, float& c, float x) {
-  const float y = x - c;
-  const float t = s + y;
-  c = (t - s) - y;
-  s = t;
-}
-
 // ---- merges
 struct WbMergeArgs {
-  const float* partial;
-  int32_t chunks;
-  int64_t n;
+  CullParts parts;
   const float4* wcoef;  // rows: window constants (a, b, c, N), k R = [[a, b], [0, c]], R^T R = C^-1
   const float* g;
   const float* v;  // columns: source weights
@@ -42,20 +33,14 @@ struct WbMergeArgs {
   double* scal;    // rows: per-block d_l partials
 };
 
-__device__ __forceinline__ float wb_merge(const float* partial, int chunks, int K, int k, int64_t n, int64_t i) {
-  float s = 0.f, c = 0.f;
-  for (int ch = 0; ch < chunks; ++ch) wb_kahan(s, c, partial[((int64_t)ch * K + k) * n + i]);
-  return s - c;
-}
-
-__global__ void __launch_bounds__(256) wn_rows_merge_kernel(const __grid_constant__ WbMergeArgs M) {
-  __shared__ double red[8];
-  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+__global__ void __launch_bounds__(kCullThreads) wn_rows_merge_kernel(const __grid_constant__ WbMergeArgs M) {
+  __shared__ double red[kCullThreads / 32];
+  int rb, slot;
+  const int64_t i = cull_part_row(M.parts, rb, slot);
   double dl = 0.0;
-  if (i < M.n) {
+  if (i >= 0) {
     float s[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) s[k] = wb_merge(M.partial, M.chunks, 6, k, M.n, i);
+    cull_part_sums<6>(M.parts, rb, slot, s);
     // C^-1 = R^T R = (2 ln 2) [[a^2, a b], [a b, b^2 + c^2]] (k^2 = 1 / (2 ln 2)):
     // products and a sum of squares, no cancellation
     const float4 wc = M.wcoef[i];
@@ -84,7 +69,7 @@ __global__ void __launch_bounds__(256) wn_rows_merge_kernel(const __grid_constan
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += red[w];
+    for (int w = 0; w < kCullThreads / 32; ++w) t += red[w];
     M.scal[blockIdx.x] = t;
   }
 }
@@ -104,16 +89,18 @@ __global__ void wn_scalar_final_kernel(const double* __restrict__ part, int nblk
   }
 }
 
-__global__ void wn_cols_merge_kernel(const __grid_constant__ WbMergeArgs M) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= M.n) return;
-  const float T = wb_merge(M.partial, M.chunks, 3, 0, M.n, k);
-  if (M.d_a) M.d_a[k] = T;
+__global__ void __launch_bounds__(kCullThreads) wn_cols_merge_kernel(const __grid_constant__ WbMergeArgs M) {
+  int rb, slot;
+  const int64_t k = cull_part_row(M.parts, rb, slot);
+  if (k < 0) return;
+  float s[3];
+  cull_part_sums<3>(M.parts, rb, slot, s);
+  if (M.d_a) M.d_a[k] = s[0];
   if (M.d_b) {
     // d_q = v (2 ln 2) U with u' evaluated at q - p
     const float vk = kTwoLn2 * M.v[k];
-    M.d_b[2 * k] = vk * wb_merge(M.partial, M.chunks, 3, 1, M.n, k);
-    M.d_b[2 * k + 1] = vk * wb_merge(M.partial, M.chunks, 3, 2, M.n, k);
+    M.d_b[2 * k] = vk * s[1];
+    M.d_b[2 * k + 1] = vk * s[2];
   }
 }
 
@@ -187,7 +174,7 @@ static lr_status plan_windowed_bwd(int64_t n, const lr_grid* layout, const lr_po
   WbPlan p{};
   if ((st = plan_cull(kCullWinRows, 1, n, layout, m, sl, &p.R)) != LR_OK) return st;
   if ((st = plan_cull(kCullWinCols, 1, m, sl, n, layout, &p.C)) != LR_OK) return st;
-  p.merge_blocks = (n + 255) / 256;
+  p.merge_blocks = p.R.row_blocks * p.R.R;
   size_t o = 0;
   p.off_rows = o;
   o += align256(p.R.bytes);
@@ -262,16 +249,14 @@ extern "C" lr_status gp_windowed_matvec_bwd(const float* p, const float* z, int6
     A.wreach = wreach;
     if ((st = launch_cull_sweep(P.R, A, wr, -1, s)) != LR_OK) return st;
     WbMergeArgs M{};
-    M.partial = reinterpret_cast<const float*>(wr + P.R.off_partial);
-    M.chunks = P.R.splits;
-    M.n = n;
+    M.parts = cull_parts(P.R, n, wr);
     M.wcoef = wcoef;
     M.g = g;
     M.ell = lengthscale;
     M.d_a = d_p;
     M.d_b = d_z;
     M.scal = reinterpret_cast<double*>(ws + P.off_scal);
-    wn_rows_merge_kernel<<<(unsigned)P.merge_blocks, 256, 0, s>>>(M);
+    wn_rows_merge_kernel<<<(unsigned)P.merge_blocks, kCullThreads, 0, s>>>(M);
     LR_CHECK_CUDA(cudaGetLastError());
     if (d_lengthscale) {
       wn_scalar_final_kernel<<<1, 256, 0, s>>>(M.scal, (int)P.merge_blocks, d_lengthscale);
@@ -288,13 +273,11 @@ extern "C" lr_status gp_windowed_matvec_bwd(const float* p, const float* z, int6
     A.stride = 1;
     if ((st = launch_cull_sweep(P.C, A, wc, -1, s)) != LR_OK) return st;
     WbMergeArgs M{};
-    M.partial = reinterpret_cast<const float*>(wc + P.C.off_partial);
-    M.chunks = P.C.splits;
-    M.n = m;
+    M.parts = cull_parts(P.C, m, wc);
     M.v = v;
     M.d_a = d_v;
     M.d_b = d_q;
-    wn_cols_merge_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(M);
+    wn_cols_merge_kernel<<<(unsigned)(P.C.row_blocks * P.C.R), kCullThreads, 0, s>>>(M);
     LR_CHECK_CUDA(cudaGetLastError());
   }
   return LR_OK;
@@ -345,7 +328,7 @@ extern "C" lr_status lr_windowed_pairs_evaluated(const float* p, const float* z,
   CullArgs A{};
   A.nrhs = 1;
   A.stride = 1;
-  A.count = cnt;
+  A.count_out = cnt;
   if (sweep == 2) {
     st = launch_cull_prep(C, pp, 0.f, w, nullptr, 1, 0, ws, s, wcoef, wreach);
     A.x = qq;
