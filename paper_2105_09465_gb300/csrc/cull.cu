@@ -839,9 +839,10 @@ __global__ void __launch_bounds__(kCullThreads, cull_min_blocks(KIND)) cull_kern
             if (sum != 0.f) kahan_add(tot[r][0], comp[r][0], sum);
           }
         } else if constexpr (KIND == kCullWinRows) {
-          // with w = R_i d (scaled), d = x_j - x_i and u = R_i^T w =
-          // k^2 C_i^-1 d (= M'_i (x_i - x_j) with M' = -k^2 C^-1, the merge's
-          // form): S += v G', P += v G' u, Q += v G' u u^T
+          // with w = R_i d (scaled), d = x_j - x_i: S += v G', A += v G' w,
+          // B += v G' w w^T. R_i is the row's own, so the merge turns the sums
+          // into those of u = R_i^T w = k^2 C_i^-1 d: 16 FP32 lanes per pair
+          // instead of 19 with u formed per pair.
           float2 acc[R][6];
 #pragma unroll
           for (int r = 0; r < R; ++r)
@@ -857,16 +858,15 @@ __global__ void __launch_bounds__(kCullThreads, cull_min_blocks(KIND)) cull_kern
               const float2 dx = __fadd2_rn(X, NQ[r]), dy = __fadd2_rn(Y, NP[r]);
               const float2 w1 = __ffma2_rn(MA[r], dx, __fmul2_rn(MB[r], dy)), w2 = __fmul2_rn(MC[r], dy);
               const float2 t = __ffma2_rn(w1, w1, __fmul2_rn(w2, w2));
-              const float2 ux = __fmul2_rn(MA[r], w1), uy = __ffma2_rn(MB[r], w1, __fmul2_rn(MC[r], w2));
               const float2 kv = __fmul2_rn(f2(ex2_approx(-t.x), ex2_approx(-t.y)), W);
-              const float2 kx = __fmul2_rn(kv, ux), ky = __fmul2_rn(kv, uy);
+              const float2 k1 = __fmul2_rn(kv, w1), k2 = __fmul2_rn(kv, w2);
               float2* a = acc[r];
               a[0] = __fadd2_rn(a[0], kv);
-              a[1] = __fadd2_rn(a[1], kx);
-              a[2] = __fadd2_rn(a[2], ky);
-              a[3] = __ffma2_rn(kx, ux, a[3]);
-              a[4] = __ffma2_rn(kx, uy, a[4]);
-              a[5] = __ffma2_rn(ky, uy, a[5]);
+              a[1] = __fadd2_rn(a[1], k1);
+              a[2] = __fadd2_rn(a[2], k2);
+              a[3] = __ffma2_rn(k1, w1, a[3]);
+              a[4] = __ffma2_rn(k1, w2, a[4]);
+              a[5] = __ffma2_rn(k2, w2, a[5]);
             }
           }
 #pragma unroll

@@ -203,8 +203,9 @@ struct CullPrepP {
 //             (the pair's exp2 shared): d_v = var sum_j k g_j per column,
 //             d_x both roles summed over the columns, scalar partials.
 //  kCullWin:  out[i] = N_i sum_j G'_ij v_j, G' = 2^(-|R_i d|^2 k^2)
-//  kCullWinRows: per row, with d = x_i - y_j and u = k^2 C_i^-1 d, the six
-//             sums S = sum v G', P = sum v G' u, Q = sum v G' u u^T (xx, xy, yy)
+//  kCullWinRows: per row, with d = y_j - x_i and w = k R_i d (the scaled
+//             Cholesky factor), the six sums S = sum v G', A = sum v G' w,
+//             B = sum v G' w w^T (11, 12, 22)
 //  kCullWinCols: per row (a source of the windowed reduction), with
 //             d = x_i - y_j and u = k^2 C_j^-1 d, T = sum gN G', U = sum gN G' u
 //             The two backward kinds are always cut into parts; the windowed

@@ -4,7 +4,7 @@
 // C_i = Z_i + (l^2/2) I, with d = p_i - q_k, M = C_i^-1 and u = M d:
 //   dG/dp_i = -G u,  dG/dq_k = G u,  dG/dC_i = G (u u^T - M) / 2,  dC_i/dl = l I.
 // Two culled sweeps over the pairs (cull.cu, explicit sources):
-//   rows:    per query row, sum_k v G [1, u, u u^T]     -> d_p, d_Z, d_l
+//   rows:    per query row, sum_k v G [1, w, w w^T]     -> d_p, d_Z, d_l  (w = R d)
 //   columns: per source,    sum_i g G [1, u]            -> d_v, d_q
 // Inside a sweep the exponent uses u' = M' d with M' = -(log2 e / 2) M, so
 // that G = N 2^(d . u') and u = -2 ln2 u'; N = 1/(2 pi sqrt(det C)) is applied
@@ -41,21 +41,22 @@ __global__ void __launch_bounds__(kCullThreads) wn_rows_merge_kernel(const __gri
   if (i >= 0) {
     float s[6];
     cull_part_sums<6>(M.parts, rb, slot, s);
-    // C^-1 = R^T R = (2 ln 2) [[a^2, a b], [a b, b^2 + c^2]] (k^2 = 1 / (2 ln 2)):
-    // products and a sum of squares, no cancellation
+    // The sums are over w = k R d, d = q - p (k^2 = 1 / (2 ln 2), k R = [[a, b],
+    // [0, c]], R^T R = C^-1), with C^-1 d = (2 ln 2) (k R)^T w:
+    //   d_p = g N (2 ln 2) (k R)^T A
+    //   D = g N / 2 (C^-1 d d^T C^-1 - C^-1 summed)
+    //     = g N / 2 (2 ln 2) (k R)^T ((2 ln 2) B - S I) (k R)
     const float4 wc = M.wcoef[i];
-    const float ixx = kTwoLn2 * (wc.x * wc.x), ixy = kTwoLn2 * (wc.x * wc.y),
-                iyy = kTwoLn2 * fmaf(wc.y, wc.y, wc.z * wc.z);
-    const float gn = M.g[i] * wc.w;
-    // d_p = g N (2 ln 2) P';  D = g N ((2 ln 2)^2 Q' - S C^-1) / 2
+    const float gn = M.g[i] * wc.w * kTwoLn2, h = 0.5f * gn;
     if (M.d_a) {
-      M.d_a[2 * i] = gn * kTwoLn2 * s[1];
-      M.d_a[2 * i + 1] = gn * kTwoLn2 * s[2];
+      M.d_a[2 * i] = gn * (wc.x * s[1]);
+      M.d_a[2 * i + 1] = gn * fmaf(wc.y, s[1], wc.z * s[2]);
     }
-    const float k2 = kTwoLn2 * kTwoLn2, h = 0.5f * gn;
-    const float Dxx = h * fmaf(k2, s[3], -s[0] * ixx);
-    const float Dxy = h * fmaf(k2, s[4], -s[0] * ixy);
-    const float Dyy = h * fmaf(k2, s[5], -s[0] * iyy);
+    const float e11 = fmaf(kTwoLn2, s[3], -s[0]), e12 = kTwoLn2 * s[4], e22 = fmaf(kTwoLn2, s[5], -s[0]);
+    const float r1 = fmaf(wc.y, e11, wc.z * e12), r2 = fmaf(wc.y, e12, wc.z * e22);
+    const float Dxx = h * (wc.x * wc.x * e11);
+    const float Dxy = h * (wc.x * r1);
+    const float Dyy = h * fmaf(wc.y, r1, wc.z * r2);
     if (M.d_b) {
       M.d_b[3 * i] = Dxx;
       M.d_b[3 * i + 1] = 2.0f * Dxy;
@@ -191,6 +192,61 @@ static lr_status plan_windowed_bwd(int64_t n, const lr_grid* layout, const lr_po
   return LR_OK;
 }
 
+// The row sweep and its merge: d_p, d_Z, d_l.
+static lr_status windowed_bwd_rows(const WbPlan& P, const float2* pp, const float2* qq, int64_t n, const float* v,
+                                   float lengthscale, const float* g, const float4* wcoef, const float* wreach,
+                                   float* d_p, float* d_z, double* d_lengthscale, char* ws, cudaStream_t s) {
+  char* wr = ws + P.off_rows;
+  lr_status st = launch_cull_prep(P.R, qq, 0.f, v, nullptr, 1, 0, wr, s);
+  if (st != LR_OK) return st;
+  CullArgs A{};
+  A.x = pp;
+  A.n = n;
+  A.nrhs = 1;
+  A.stride = 1;
+  A.wcoef = wcoef;
+  A.wreach = wreach;
+  if ((st = launch_cull_sweep(P.R, A, wr, -1, s)) != LR_OK) return st;
+  WbMergeArgs M{};
+  M.parts = cull_parts(P.R, n, wr);
+  M.wcoef = wcoef;
+  M.g = g;
+  M.ell = lengthscale;
+  M.d_a = d_p;
+  M.d_b = d_z;
+  M.scal = reinterpret_cast<double*>(ws + P.off_scal);
+  wn_rows_merge_kernel<<<(unsigned)P.merge_blocks, kCullThreads, 0, s>>>(M);
+  LR_CHECK_CUDA(cudaGetLastError());
+  if (d_lengthscale) {
+    wn_scalar_final_kernel<<<1, 256, 0, s>>>(M.scal, (int)P.merge_blocks, d_lengthscale);
+    LR_CHECK_CUDA(cudaGetLastError());
+  }
+  return LR_OK;
+}
+
+// The column sweep and its merge: d_v, d_q.
+static lr_status windowed_bwd_cols(const WbPlan& P, const float2* pp, const float2* qq, int64_t n, int64_t m,
+                                   const float* v, const float* g, const float4* wcoef, const float* wreach,
+                                   float* d_v, float* d_q, char* ws, cudaStream_t s) {
+  char* wc = ws + P.off_cols;
+  lr_status st = launch_cull_prep(P.C, pp, 0.f, g, nullptr, 1, 0, wc, s, wcoef, wreach);
+  if (st != LR_OK) return st;
+  CullArgs A{};
+  A.x = qq;
+  A.n = m;
+  A.nrhs = 1;
+  A.stride = 1;
+  if ((st = launch_cull_sweep(P.C, A, wc, -1, s)) != LR_OK) return st;
+  WbMergeArgs M{};
+  M.parts = cull_parts(P.C, m, wc);
+  M.v = v;
+  M.d_a = d_v;
+  M.d_b = d_q;
+  wn_cols_merge_kernel<<<(unsigned)(P.C.row_blocks * P.C.R), kCullThreads, 0, s>>>(M);
+  LR_CHECK_CUDA(cudaGetLastError());
+  return LR_OK;
+}
+
 }  // namespace lr
 
 using namespace lr;
@@ -237,50 +293,17 @@ extern "C" lr_status gp_windowed_matvec_bwd(const float* p, const float* z, int6
   float4* wcoef = reinterpret_cast<float4*>(ws + P.off_wcoef);
   float* wreach = reinterpret_cast<float*>(ws + P.off_wreach);
   if ((st = launch_window_prep(z, n, lengthscale, wcoef, wreach, s)) != LR_OK) return st;
-  if (d_p || d_z || d_lengthscale) {
-    char* wr = ws + P.off_rows;
-    if ((st = launch_cull_prep(P.R, qq, 0.f, v, nullptr, 1, 0, wr, s)) != LR_OK) return st;
-    CullArgs A{};
-    A.x = pp;
-    A.n = n;
-    A.nrhs = 1;
-    A.stride = 1;
-    A.wcoef = wcoef;
-    A.wreach = wreach;
-    if ((st = launch_cull_sweep(P.R, A, wr, -1, s)) != LR_OK) return st;
-    WbMergeArgs M{};
-    M.parts = cull_parts(P.R, n, wr);
-    M.wcoef = wcoef;
-    M.g = g;
-    M.ell = lengthscale;
-    M.d_a = d_p;
-    M.d_b = d_z;
-    M.scal = reinterpret_cast<double*>(ws + P.off_scal);
-    wn_rows_merge_kernel<<<(unsigned)P.merge_blocks, kCullThreads, 0, s>>>(M);
-    LR_CHECK_CUDA(cudaGetLastError());
-    if (d_lengthscale) {
-      wn_scalar_final_kernel<<<1, 256, 0, s>>>(M.scal, (int)P.merge_blocks, d_lengthscale);
-      LR_CHECK_CUDA(cudaGetLastError());
-    }
-  }
-  if (d_v || d_q) {
-    char* wc = ws + P.off_cols;
-    if ((st = launch_cull_prep(P.C, pp, 0.f, g, nullptr, 1, 0, wc, s, wcoef, wreach)) != LR_OK) return st;
-    CullArgs A{};
-    A.x = qq;
-    A.n = m;
-    A.nrhs = 1;
-    A.stride = 1;
-    if ((st = launch_cull_sweep(P.C, A, wc, -1, s)) != LR_OK) return st;
-    WbMergeArgs M{};
-    M.parts = cull_parts(P.C, m, wc);
-    M.v = v;
-    M.d_a = d_v;
-    M.d_b = d_q;
-    wn_cols_merge_kernel<<<(unsigned)(P.C.row_blocks * P.C.R), kCullThreads, 0, s>>>(M);
-    LR_CHECK_CUDA(cudaGetLastError());
-  }
-  return LR_OK;
+  // the two sweeps are independent: the columns run on the side stream, where
+  // their prepare, plan and merge fill what the row sweep's leave idle
+  const bool rows = d_p || d_z || d_lengthscale, cols = d_v || d_q;
+  Fork f{};
+  f.side = s;
+  if (rows && cols && (st = fork_begin(s, &f)) != LR_OK) return st;
+  if (cols) st = windowed_bwd_cols(P, pp, qq, n, m, v, g, wcoef, wreach, d_v, d_q, ws, f.side);
+  if (st == LR_OK && rows)
+    st = windowed_bwd_rows(P, pp, qq, n, v, lengthscale, g, wcoef, wreach, d_p, d_z, d_lengthscale, ws, s);
+  const lr_status sj = fork_end(s, &f);
+  return st != LR_OK ? st : sj;
 }
 
 extern "C" lr_status lr_windowed_pairs_evaluated(const float* p, const float* z, int64_t n, const lr_grid* layout,
