@@ -640,6 +640,13 @@ lr_status lr_vec_axpby(int64_t n, float a, const float* x, float b, const float*
 lr_status lr_vec_mul(int64_t n, const float* a, const float* b, float* out, lr_stream stream);
 /* out[0:nh] = (float)head (FP64), out[nh:nh+nt] = tail. */
 lr_status lr_vec_pack(const double* head, int32_t nh, const float* tail, int64_t nt, float* out, lr_stream stream);
+/* The parameter gradients of gp_kernel_matvec_bwd (FP64; each may be NULL: 0) as
+ * one FP32 array of 12 + 5 n_sub values: out[0:8] = d/d(x0, y0, q, phi, theta_e,
+ * gamma, g1, g2) with 0 for the fixed slope gamma, out[8] = d/d lengthscale,
+ * out[9] = d/d variance, out[10:12] = 0, out[12 + 5h ...] = the subhalo record's
+ * (x_h, y_h, kappa_s | theta_pm, theta_s, tau) with 0 for tau. */
+lr_status lr_param_grads(const double* d_lens, const double* d_lengthscale, const double* d_variance,
+                         const double* d_sub, int32_t n_sub, float* out, lr_stream stream);
 /* *out = sum of the n (<= 16) device doubles *parts[k] (parts: a HOST array
  * of device pointers), in that order. */
 lr_status lr_sum_scalars(const double* const* parts, int32_t n, double* out, lr_stream stream);

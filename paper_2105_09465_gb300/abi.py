@@ -102,6 +102,7 @@ SIGNATURES = {
     "lr_vec_axpby": (ctypes.c_int32, [ctypes.c_int64, ctypes.c_float, _P, ctypes.c_float, _P, _P, _P]),
     "lr_vec_mul": (ctypes.c_int32, [ctypes.c_int64, _P, _P, _P, _P]),
     "lr_vec_pack": (ctypes.c_int32, [_P, ctypes.c_int32, _P, ctypes.c_int64, _P, _P]),
+    "lr_param_grads": (ctypes.c_int32, [_P, _P, _P, _P, ctypes.c_int32, _P, _P]),
     "lr_sum_scalars": (ctypes.c_int32, [ctypes.POINTER(ctypes.c_void_p), ctypes.c_int32, _P, _P]),
     "lens_jacobian": (ctypes.c_int32, [ctypes.POINTER(lr_points), _P, _P, _P]),
     "gp_kernel_matvec": (ctypes.c_int32, [ctypes.POINTER(lr_points), ctypes.POINTER(lr_points), _P, ctypes.c_int32,

@@ -40,9 +40,14 @@ def _require_cuda(t: torch.Tensor | None, name: str, shape_tail=None) -> None:
         raise ValueError(f"{name} must have shape (n, {', '.join(map(str, shape_tail))})")
 
 
-def _stream_handle(stream: torch.cuda.Stream | None) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream_handle(stream: torch.cuda.Stream | None) -> int:
+    # the current stream's handle without building a Stream object (20 us a call on the host)
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
+
+
+_LENS_FIELDS = tuple(name for name, _ in abi.lr_lens._fields_)
 
 
 def to_c_points(p: Points | None):
@@ -64,7 +69,7 @@ def to_c_points(p: Points | None):
         c.n = p.grid.n
     if p.lens is not None or p.lens_record is not None:
         if p.lens is not None:
-            L = abi.lr_lens(*p.lens.astuple())
+            L = abi.lr_lens(*(getattr(p.lens, k) for k in _LENS_FIELDS))
             keep.append(L)
             c.lens = ctypes.pointer(L)
         else:
@@ -150,6 +155,19 @@ def vec_pack(head: torch.Tensor, tail: torch.Tensor, stream=None) -> torch.Tenso
     out = torch.empty(head.numel() + tail.numel(), dtype=torch.float32, device=tail.device)
     abi.check(lib.lr_vec_pack(head.data_ptr(), head.numel(), tail.data_ptr(), tail.numel(), out.data_ptr(),
                               _stream_handle(stream)), "lr_vec_pack")
+    return out
+
+
+def param_grads(grads: dict, n_sub: int, device, stream=None) -> torch.Tensor:
+    """The parameter gradients of gp_kernel_matvec_bwd as one float32 tensor of
+    12 + 5 n_sub values, in one launch: [0:8] the lens (0 for the fixed slope),
+    [8] the length scale, [9] the variance, [12:] the (n_sub, 5) subhalo records
+    (0 for tau); 0 where `grads` lacks one."""
+    lib = abi.load()
+    ptr = lambda k: grads[k].data_ptr() if k in grads else None
+    out = torch.empty(12 + 5 * n_sub, dtype=torch.float32, device=device)
+    abi.check(lib.lr_param_grads(ptr("lens"), ptr("lengthscale"), ptr("variance"), ptr("sub") if n_sub else None,
+                                 n_sub, out.data_ptr(), _stream_handle(stream)), "lr_param_grads")
     return out
 
 

@@ -18,12 +18,23 @@ from . import api
 from .workloads import Grid, Lens
 
 
+def _host_params(lens_params, lengthscale, variance):
+    """(lens values, length scale, variance) on the host: with one copy where
+    the three live on one CUDA device in one type."""
+    ts = (lens_params, lengthscale, variance)
+    if (all(isinstance(t, torch.Tensor) and t.is_cuda and t.device == lens_params.device
+            and t.dtype == lens_params.dtype for t in ts) and lens_params.dim() == 1
+            and lengthscale.numel() == variance.numel() == 1):
+        vals = torch.cat([t.detach().reshape(-1) for t in ts]).tolist()
+        return vals[:-2], vals[-2], vals[-1]
+    return lens_params.detach().cpu().tolist(), float(lengthscale), float(variance)
+
+
 class RaytraceKernelMatvec(torch.autograd.Function):
     @staticmethod
     def forward(ctx, v, lens_params, sub, lengthscale, variance, xgrid: Grid, ygrid: Grid | None, profile: int):
-        lens = Lens(*[float(t) for t in lens_params.detach().cpu().tolist()])
-        ell = float(lengthscale)
-        var = float(variance)
+        vals, ell, var = _host_params(lens_params, lengthscale, variance)
+        lens = Lens(*[float(t) for t in vals])
         q = api.Points(grid=xgrid, lens=lens, sub=sub.detach().contiguous() if sub is not None else None,
                        profile=profile)
         s = api.Points(grid=ygrid) if ygrid is not None else None
@@ -37,6 +48,10 @@ class RaytraceKernelMatvec(torch.autograd.Function):
             mom = torch.empty(0, device=v.device)
         ctx.save_for_backward(v, sub if sub is not None else torch.empty(0), beta, mom)
         ctx.meta = (q, s, ell, var, lens_params.dtype, lens_params.device)
+        # float32 parameters on the points' device take their gradients from one launch
+        ctx.packed = all(not isinstance(t, torch.Tensor) or (t.dtype == torch.float32 and t.device == v.device)
+                         for t in (lens_params, lengthscale, variance)) and lens_params.shape == (8,)
+        ctx.scalar_shapes = tuple(t.shape if isinstance(t, torch.Tensor) else () for t in (lengthscale, variance))
         return out
 
     @staticmethod
@@ -60,6 +75,12 @@ class RaytraceKernelMatvec(torch.autograd.Function):
         G = api.gp_kernel_matvec_bwd(q, s, v.detach().contiguous(), ell, var, grad_out.contiguous().float(),
                                      want=want, beta=beta, moments=mom if mom.numel() else None)
         gv = G.get("v")
+        if ctx.packed:
+            ns = sub.shape[0] if sub.numel() else 0
+            pg = api.param_grads(G, ns if "sub" in G else 0, v.device)
+            return (gv, pg[:8] if "lens" in G else None, pg[12:].view(ns, 5) if "sub" in G else None,
+                    pg[8].reshape(ctx.scalar_shapes[0]) if "lengthscale" in G else None,
+                    pg[9].reshape(ctx.scalar_shapes[1]) if "variance" in G else None, None, None, None)
         gl = None
         if "lens" in G:
             g7 = G["lens"].to(ldev, ldtype)

@@ -17,6 +17,16 @@ lr_status cuda_status(cudaError_t e, const char* what);
 // Device address of the library's fault word on the current device.
 int* fault_ptr();
 
+// kernel_occupancy: resident CTAs of `threads` threads per SM of a kernel (no dynamic shared
+// memory) and the SM count, on the current device. Constants of the kernel and
+// the device, asked of the runtime once per pair and kept: every call plans
+// twice (its workspace size, then itself), at 1 to 3 us a question.
+lr_status kernel_occupancy_of(const void* fn, int threads, int* occ, int* n_sm);
+template <class Fn>
+lr_status kernel_occupancy(Fn* fn, int threads, int* occ, int* n_sm) {
+  return kernel_occupancy_of(reinterpret_cast<const void*>(fn), threads, occ, n_sm);
+}
+
 // Launch timer (lr_kernel_timer_enable): events on stream s before and after
 // one launch of kernel id (an LR_KT_* value). No-ops while the timer is off or
 // s is capturing a graph.
@@ -42,6 +52,12 @@ inline cudaStream_t as_cuda(lr_stream s) { return reinterpret_cast<cudaStream_t>
   do {                                                             \
     cudaError_t _e = (call);                                       \
     if (_e != cudaSuccess) return ::lr::cuda_status(_e, #call);    \
+  } while (0)
+
+#define LR_CHECK(call)                         \
+  do {                                         \
+    const lr_status _s = (call);               \
+    if (_s != LR_OK) return _s;                \
   } while (0)
 
 #define LR_REQUIRE(cond, ...)                                      \

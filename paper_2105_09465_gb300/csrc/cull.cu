@@ -1120,10 +1120,8 @@ lr_status plan_cull(int kind, int nrhs, int64_t n, const lr_grid* qlayout, int64
     P.map.TH = (P.map.H + P.map.th - 1) / P.map.th;
   }
   P.row_blocks = row_block_count(P.map, n, P.rows_per_cta);
-  int dev = 0, n_sm = 1, occ = 1;
-  LR_CHECK_CUDA(cudaGetDevice(&dev));
-  LR_CHECK_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-  LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cull_kernel_ptr(kind, P.nw, layers), kCullThreads, 0));
+  int n_sm = 1, occ = 1;
+  LR_CHECK(kernel_occupancy_of(cull_kernel_ptr(kind, P.nw, layers), kCullThreads, &occ, &n_sm));
   // In parts (cull.cuh) where the row blocks are under kFewWaves waves of the
   // resident CTA slots (above, one CTA per row block keeps its sums in
   // registers, and a band of rows gives the whole problem's bits), and always for windowed points: they differ in reach by orders of

@@ -2,6 +2,10 @@
 // leaves a human-readable message in a thread-local buffer.
 #include <stdarg.h>
 #include <string.h>
+
+#include <mutex>
+#include <vector>
+
 #include "common.cuh"
 #include "tma.cuh"
 
@@ -19,6 +23,31 @@ void set_error(const char* fmt, ...) {
 lr_status cuda_status(cudaError_t e, const char* what) {
   set_error("%s failed: %s (%s)", what, cudaGetErrorName(e), cudaGetErrorString(e));
   return e == cudaErrorMemoryAllocation ? LR_ERR_OUT_OF_MEMORY : LR_ERR_CUDA;
+}
+
+lr_status kernel_occupancy_of(const void* fn, int threads, int* occ, int* n_sm) {
+  struct Known {
+    const void* fn;
+    int threads, dev, occ, n_sm;
+  };
+  static std::mutex mu;
+  static std::vector<Known> known;  // one entry per kernel and device in use
+  int dev = 0;
+  LR_CHECK_CUDA(cudaGetDevice(&dev));
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    for (const Known& k : known)
+      if (k.fn == fn && k.threads == threads && k.dev == dev) {
+        *occ = k.occ;
+        *n_sm = k.n_sm;
+        return LR_OK;
+      }
+  }
+  LR_CHECK_CUDA(cudaDeviceGetAttribute(n_sm, cudaDevAttrMultiProcessorCount, dev));
+  LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, fn, threads, 0));
+  std::lock_guard<std::mutex> lock(mu);
+  known.push_back({fn, threads, dev, *occ, *n_sm});
+  return LR_OK;
 }
 
 }  // namespace lr

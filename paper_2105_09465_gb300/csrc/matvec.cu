@@ -379,10 +379,8 @@ static lr_status plan_matvec(const lr_points* q, const lr_points* s, int32_t nrh
   p.n_tiles = (int32_t)((int64_t)p.segs * s->grid.ny * s->grid.ss);
   p.map = layout ? make_row_map(layout, kRowsPerCta) : RowMap{};
   p.row_blocks = (int32_t)row_block_count(p.map, p.n, kRowsPerCta);
-  int dev = 0, n_sm = 1, occ = 1;
-  LR_CHECK_CUDA(cudaGetDevice(&dev));
-  LR_CHECK_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-  LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, matvec_kernel<true>, kMvThreads, 0));
+  int n_sm = 1, occ = 1;
+  LR_CHECK(kernel_occupancy(&matvec_kernel<true>, kMvThreads, &occ, &n_sm));
   p.chunks = plan_chunks(p.row_blocks, p.n_tiles, occ, n_sm, kSkipWaves);
   p.off_partial = off;
   if (p.chunks > 1) off += align256(sizeof(float) * (size_t)p.chunks * (size_t)p.n);

@@ -1303,27 +1303,23 @@ static lr_status plan_rows(int64_t n, int64_t m, bool grid, const lr_grid* g, bo
   p.map = (grid && qgrid) ? make_row_map(qgrid, p.rows_per_cta) : RowMap{};
   p.row_blocks = (int32_t)row_block_count(p.map, n, p.rows_per_cta);
   p.info_bytes = grid ? row_info_bytes(p.map, n, p.rows_per_cta) : 0;
-  int dev = 0, n_sm = 1, occ = 1;
-  LR_CHECK_CUDA(cudaGetDevice(&dev));
-  LR_CHECK_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+  int n_sm = 1, occ = 1;
   if (self)
-    LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bwd_rows_kernel<false, true, false>, kBwThreads, 0));
+    LR_CHECK(kernel_occupancy(&bwd_rows_kernel<false, true, false>, kBwThreads, &occ, &n_sm));
   else if (dv) {
     // the split and unsplit variants: plan for the lower occupancy of the two
     int occ2 = 1;
-    LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bwd_rows_kernel<true, false, true>, kBwThreads, 0));
-    LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, bwd_rows_kernel<true, false, true, true>,
-                                                                kBwThreads, 0));
+    LR_CHECK(kernel_occupancy(&bwd_rows_kernel<true, false, true>, kBwThreads, &occ, &n_sm));
+    LR_CHECK(kernel_occupancy(&bwd_rows_kernel<true, false, true, true>, kBwThreads, &occ2, &n_sm));
     occ = occ < occ2 ? occ : occ2;
   }
   else if (grid) {
     int occ2 = 1;
-    LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bwd_rows_kernel<true, false, false>, kBwThreads, 0));
-    LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, bwd_rows_kernel<true, false, false, true>,
-                                                                kBwThreads, 0));
+    LR_CHECK(kernel_occupancy(&bwd_rows_kernel<true, false, false>, kBwThreads, &occ, &n_sm));
+    LR_CHECK(kernel_occupancy(&bwd_rows_kernel<true, false, false, true>, kBwThreads, &occ2, &n_sm));
     occ = occ < occ2 ? occ : occ2;
   } else {
-    LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bwd_rows_kernel<false, false, false>, kBwThreads, 0));
+    LR_CHECK(kernel_occupancy(&bwd_rows_kernel<false, false, false>, kBwThreads, &occ, &n_sm));
   }
   const int32_t chunks = plan_chunks(p.row_blocks, p.n_tiles, occ, n_sm, grid ? kSkipWaves : kChunkWaves);
   p.chunks = chunks;
@@ -1523,11 +1519,9 @@ static lr_status plan_dv(int64_t n, const lr_grid* g, const lr_grid* qgrid, RowP
   p.map = qgrid ? make_row_map(qgrid, kDvRows) : RowMap{};
   p.row_blocks = (int32_t)row_block_count(p.map, n, kDvRows);
   p.info_bytes = row_info_bytes(p.map, n, kDvRows);
-  int dev = 0, n_sm = 1, occ = 1, occ2 = 1;
-  LR_CHECK_CUDA(cudaGetDevice(&dev));
-  LR_CHECK_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-  LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dv_rows_kernel<true>, kBwThreads, 0));
-  LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, dv_rows_kernel<false>, kBwThreads, 0));
+  int n_sm = 1, occ = 1, occ2 = 1;
+  LR_CHECK(kernel_occupancy(&dv_rows_kernel<true>, kBwThreads, &occ, &n_sm));
+  LR_CHECK(kernel_occupancy(&dv_rows_kernel<false>, kBwThreads, &occ2, &n_sm));
   p.chunks = plan_chunks(p.row_blocks, p.n_tiles, occ < occ2 ? occ : occ2, n_sm, kSkipWaves);
   const int64_t m = (int64_t)W * g->ny * g->ss;
   p.dv_bytes = align256(sizeof(float) * (size_t)p.row_blocks * (size_t)m);

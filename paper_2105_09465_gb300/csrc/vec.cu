@@ -26,6 +26,28 @@ __global__ void pack_kernel(const double* __restrict__ head, int32_t nh, const f
     out[i] = i < nh ? (float)head[i] : tail[i - nh];
 }
 
+// The parameter gradients of one lens system as float32: [0, 8) the lens with
+// the fixed slope's 0 in place 5, [8] the length scale, [9] the variance,
+// [12, 12 + 5 n_sub) the subhalo records with tau's 0 in place 4. A NULL input
+// leaves zeros.
+__global__ void param_grads_kernel(const double* __restrict__ lens, const double* __restrict__ ell,
+                                   const double* __restrict__ var, const double* __restrict__ sub, int32_t n_sub,
+                                   float* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 12 + 5 * n_sub) return;
+  float r = 0.f;
+  if (i < 8) {
+    if (lens && i != 5) r = (float)lens[i < 5 ? i : i - 1];
+  } else if (i < 12) {
+    if (i == 8 && ell) r = (float)*ell;
+    if (i == 9 && var) r = (float)*var;
+  } else if (sub) {
+    const int h = (i - 12) / 5, k = (i - 12) - 5 * h;
+    if (k < 4) r = (float)sub[4 * h + k];
+  }
+  out[i] = r;
+}
+
 constexpr int kMaxScalars = 16;
 struct ScalarList {
   const double* p[kMaxScalars];
@@ -75,6 +97,20 @@ extern "C" lr_status lr_vec_pack(const double* head, int32_t nh, const float* ta
   LR_REQUIRE((head != nullptr || nh == 0) && (tail != nullptr || nt == 0) && out != nullptr,
              "lr_vec_pack: NULL argument");
   pack_kernel<<<vec_blocks(nh + nt), 256, 0, as_cuda(stream)>>>(head, nh, tail, nt, out);
+  LR_CHECK_CUDA(cudaGetLastError());
+  return LR_OK;
+}
+
+extern "C" lr_status lr_param_grads(const double* d_lens, const double* d_lengthscale, const double* d_variance,
+                                    const double* d_sub, int32_t n_sub, float* out, lr_stream stream) {
+  LR_REQUIRE(n_sub >= 0 && n_sub < (1 << 28), "lr_param_grads: n_sub = %d out of range", n_sub);
+  LR_REQUIRE(out != nullptr, "lr_param_grads: out is NULL");
+  LR_REQUIRE((((uintptr_t)d_lens | (uintptr_t)d_lengthscale | (uintptr_t)d_variance | (uintptr_t)d_sub) & 7u) == 0 &&
+                 ((uintptr_t)out & 3u) == 0,
+             "lr_param_grads: misaligned pointer");
+  const int n = 12 + 5 * n_sub;
+  param_grads_kernel<<<(n + 255) / 256, 256, 0, as_cuda(stream)>>>(d_lens, d_lengthscale, d_variance, d_sub, n_sub,
+                                                                   out);
   LR_CHECK_CUDA(cudaGetLastError());
   return LR_OK;
 }

@@ -251,10 +251,8 @@ static lr_status plan_windowed(int64_t n, const lr_grid* layout, const lr_points
   p.segs = (W + kWnTile - 1) / kWnTile;
   p.n_tiles = (int32_t)((int64_t)p.segs * s->grid.ny * s->grid.ss);
   p.row_blocks = (int32_t)((n + kWnRows - 1) / kWnRows);
-  int dev = 0, n_sm = 1, occ = 1;
-  LR_CHECK_CUDA(cudaGetDevice(&dev));
-  LR_CHECK_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-  LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, windowed_kernel, kWnThreads, 0));
+  int n_sm = 1, occ = 1;
+  LR_CHECK(kernel_occupancy(&windowed_kernel, kWnThreads, &occ, &n_sm));
   p.chunks = plan_chunks(p.row_blocks, p.n_tiles, occ, n_sm);
   p.off_wcoef = p.chunks > 1 ? align256(4 * (size_t)p.chunks * (size_t)n) : 0;
   p.off_wreach = p.off_wcoef + align256(16 * (size_t)n);
