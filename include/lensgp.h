@@ -400,6 +400,10 @@ lr_status gp_pixel_shapes_vjp(const float* p, int32_t W, int32_t H, const float*
  */
 lr_status gp_knn_density(const float* q, int64_t m, int32_t k, float lengthscale, float* r2_out, float* a_out,
                          void* workspace, size_t workspace_bytes, lr_stream stream);
+/* A_i = pi l sqrt(2 r2_i / k) from neighbour radii r2 [m] of gp_knn_density: the
+ * weights of another length scale at the same points, bit for bit its a_out. */
+lr_status gp_transmission_weights(const float* r2, int64_t m, int32_t k, float lengthscale, float* a_out,
+                                  lr_stream stream);
 lr_status lr_knn_workspace_size(int64_t m, size_t* bytes);
 
 /* ------------------------------------------------------------------------ */

@@ -118,6 +118,7 @@ SIGNATURES = {
                                             _P, ctypes.c_float, _P, _P, ctypes.c_size_t, _P]),
     "gp_knn_density": (ctypes.c_int32, [_P, ctypes.c_int64, ctypes.c_int32, ctypes.c_float, _P, _P, _P,
                                         ctypes.c_size_t, _P]),
+    "gp_transmission_weights": (ctypes.c_int32, [_P, ctypes.c_int64, ctypes.c_int32, ctypes.c_float, _P, _P]),
     "lr_knn_workspace_size": (ctypes.c_int32, [ctypes.c_int64, ctypes.POINTER(ctypes.c_size_t)]),
     "gp_kernel_matvec_train": (ctypes.c_int32, [ctypes.POINTER(lr_points), ctypes.POINTER(lr_points), _P,
                                                 ctypes.c_int32, ctypes.c_float, ctypes.c_float, _P, _P, _P, _P,

@@ -365,6 +365,17 @@ def knn_density(q: torch.Tensor, k: int = 20, lengthscale: float | None = None, 
     return r2 if r2 is not None else a
 
 
+def transmission_weights(r2: torch.Tensor, k: int, lengthscale: float, stream=None) -> torch.Tensor:
+    """The transmission weights A = pi l sqrt(2 r2 / k) of neighbour radii r2
+    (knn_density): another layer's weights from the same points' radii."""
+    lib = abi.load()
+    _require_cuda(r2, "r2")
+    a = torch.empty_like(r2)
+    abi.check(lib.gp_transmission_weights(r2.data_ptr(), r2.numel(), int(k), float(lengthscale), a.data_ptr(),
+                                          _stream_handle(stream)), "gp_transmission_weights")
+    return a
+
+
 # ---------------------------------------------------------------- likelihood and ELBO terms
 def _elbo_ws(device) -> torch.Tensor:
     return torch.empty(int(abi.load().lr_elbo_workspace_size()), dtype=torch.uint8, device=device)

@@ -115,9 +115,12 @@ def loss_and_grads(cfg: ModelConfig, guide: Guide, data: torch.Tensor, eps_sp: t
     z = api.pixel_shapes(beta, W, H)
     self_pts = api.Points(xy=beta, grid=cfg.pixels)  # the pixels in their image layout
     a_layers, w_layers = [], []
-    nll = g = None
+    nll = g = r2 = None
     for li, (y, s) in enumerate(zip(ys, cfg.sigma_layers)):
-        a_k = api.knn_density(beta, cfg.knn_k, lengthscale=s, want_r2=False)
+        if r2 is None:  # the neighbour radii of the step's points, once for all layers
+            r2, a_k = api.knn_density(beta, cfg.knn_k, lengthscale=s)
+        else:
+            a_k = api.transmission_weights(r2, cfg.knn_k, s)
         w = api.vec_mul(a_k, y)
         if li + 1 < len(ys):
             api.vec_axpby(1.0, f, 1.0, api.gp_windowed_matvec(beta, z, self_pts, w, s, layout=cfg.pixels), out=f)
