@@ -76,6 +76,7 @@ struct VjSmem {
   float wbox[kVjWarps][4];        // per-warp bounds of the CTA's points
   float box[4];                   // x_lo, y_lo, x_hi, y_hi of the CTA's points
   float2 wm[3][kVjExpTerms];      // the tile's moments for the local expansion (vj_moments): W, W_x, W_y
+  int nexp;                       // subhalos of the tile that the local expansion serves
   float mred[kVjWarps][2 * kVjExpTerms];  // their per-warp sums, in the order of vj_moment_at
 };
 
@@ -86,6 +87,7 @@ struct VjSmem {
 struct VjPlan {
   const int* perm;
   const unsigned short* ord;
+  const int* nexp;  // per tile: how many of them the local expansion serves (they come first)
 };
 
 // One tNFW pair's terms of the four subhalo sums, for two points at once
@@ -581,10 +583,11 @@ __device__ __forceinline__ float vj_cost(int cls, int npts) {
 // (vj_class): those served by the local expansion first, then by the series
 // of degree 3, 4, 5, 7, each class in index order, those that need the
 // closed forms last: ord[rank] = subhalo (shared or global memory). cls:
-// per-subhalo scratch in shared memory. Returns the thread's share of the
-// tile's work per point (sum of vj_cost over its subhalos).
+// per-subhalo scratch in shared memory; *nexp: the expansion's count. Returns
+// the thread's share of the tile's work per point (sum of vj_cost over its
+// subhalos).
 __device__ __forceinline__ float vj_sort(const float* __restrict__ sub, int n_sub, const float* box, bool exp_ok,
-                                         int npts, unsigned char* cls, unsigned short* ord) {
+                                         int npts, unsigned char* cls, unsigned short* ord, int* nexp) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float cost = 0.f;
   for (int h = tid; h < n_sub; h += kVjThreads) {
@@ -621,6 +624,7 @@ __device__ __forceinline__ float vj_sort(const float* __restrict__ sub, int n_su
       tot += wcnt[w][pass];
       if (w < warp) before += wcnt[w][pass];
     }
+    if (pass == 0 && tid == 0) *nexp = tot;
     int pos = nf + before;
     for (int b = h0; b < h1; b += 32) {
       const bool f = b + lane < h1 && vj_cls_key(cls[b + lane]) == want;
@@ -634,6 +638,141 @@ __device__ __forceinline__ float vj_sort(const float* __restrict__ sub, int n_su
   return cost;
 }
 
+// Whether a tile of npts points in one staged chunk takes the local expansion:
+// its cost does not depend on the points, and below 64 of them the direct sums
+// are cheaper.
+__device__ __forceinline__ bool vj_exp_ok(bool one, int npts) { return one && npts >= 64; }
+
+// Phases of the nd direct subhalos of a tile of np point pairs: the power of
+// two P <= 8 (at least 16 pairs a slot) for which the CTA's groups of slots are
+// done soonest: ceil(nd P / threads) rounds of np / P steps and a slot's set-up.
+__device__ __forceinline__ int vj_pick_phases(int nd, int np) {
+  int best = 1, cost = 0x7fffffff;
+#pragma unroll
+  for (int P = 1; P <= kVjMaxPhases; P *= 2) {
+    if (P > 1 && np < 16 * P) break;
+    const int c = (nd * P + kVjThreads - 1) / kVjThreads * ((np + P - 1) / P + 8);
+    if (c < cost) {
+      cost = c;
+      best = P;
+    }
+  }
+  return best;
+}
+
+// The tNFW subhalo sums of a tile whose points are staged in one chunk: the
+// first nexp subhalos of its order by the local expansion, one thread each,
+// then the direct ones in slots (subhalo, phase) with the tile's own phase
+// count; a subhalo's P slots are neighbouring lanes, added by shuffles.
+// Choosing the phases per tile keeps the threads busy when few subhalos are
+// left to the direct sums, and lets any subhalo count take the expansion: with
+// one phase count per launch, 200 subhalos ran in 3 phases and every pair
+// directly (249 us at 640k points).
+__device__ __forceinline__ void vj_tile_sums(const float* __restrict__ sub, int n_sub, int nexp,
+                                             const unsigned short* __restrict__ ord, int cnt, float2 cen, float hd2,
+                                             float* __restrict__ sub_part, int64_t blk, int64_t nblk, VjSmem& sm) {
+  constexpr int PR = LR_PROFILE_TNFW;
+  const int tid = threadIdx.x;
+  for (int e = tid; e < nexp; e += kVjThreads) {
+    const int h = ord[e];
+    const float* rr = sub + 5 * (int64_t)h;
+    const SubRec rec = prep_sub(rr, PR);
+    const SubSer q = prep_series(rec, PR);
+    const int deg = vj_degree_box(rec, q, sm.box);
+    const float4 x = vj_expand(rec, q, __ldg(rr + 2), __ldg(rr + 3), deg, cen, hd2, sm);
+    float* o = sub_part + (int64_t)h * 4 * nblk + blk;  // [value][CTA]
+    o[0] = x.x;
+    o[nblk] = x.y;
+    o[2 * nblk] = x.z;
+    o[3 * nblk] = x.w;
+  }
+  const int nd = n_sub - nexp, np = (cnt + 1) >> 1;
+  const int P = vj_pick_phases(nd, np);
+  for (int base = 0; base < nd * P; base += kVjThreads) {
+    const int slot = base + tid, r = slot & (P - 1);
+    const bool own = slot < nd * P;
+    const int h = own ? (int)ord[nexp + slot / P] : 0;
+    float sc[4] = {0.f, 0.f, 0.f, 0.f}, cc[4] = {0.f, 0.f, 0.f, 0.f};
+    if (own) {
+      const float* rr = sub + 5 * (int64_t)h;
+      const SubRec rec = prep_sub(rr, PR);
+      const SubSer q = prep_series(rec, PR);
+      const int deg = vj_degree_box(rec, q, sm.box);
+      const float tau = __ldg(rr + 4), t2 = tau * tau;
+      const float2 ex = make_float2(4.0f * t2 / ((t2 + 1.0f) * (t2 + 1.0f)), 1.0f / __ldg(rr + 3));
+      switch (deg) {
+        case 3: vj_sweep<PR, 3, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+        case 4: vj_sweep<PR, 4, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+        case 5: vj_sweep<PR, 5, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+        case 7: vj_sweep<PR, 7, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+        default: vj_sweep<PR, 0, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
+      }
+#pragma unroll
+      for (int v = 0; v < 4; ++v) sc[v] = __fmul_rn(sc[v] - cc[v], vj_scale<PR>(rec, ex, v));
+    }
+    for (int o = P >> 1; o > 0; o >>= 1)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) sc[v] += __shfl_xor_sync(0xffffffffu, sc[v], o);
+    if (own && r == 0) {
+      float* o = sub_part + (int64_t)h * 4 * nblk + blk;
+#pragma unroll
+      for (int v = 0; v < 4; ++v) o[v * nblk] = sc[v];
+    }
+  }
+}
+
+// Stages the chunk of cnt points from c0 as packed pairs (sm.pos, sm.grad) and,
+// with lens_terms, adds their lens and shear terms to la.
+__device__ __forceinline__ void vj_stage(const LensConst& L, const LensGradConst& LG, const GridDev& g,
+                                         const float2* __restrict__ xi, const VjMap& mp, bool grid,
+                                         const float2* __restrict__ dbeta, int64_t c0, int cnt, bool lens_terms,
+                                         float (&la)[7], VjSmem& sm) {
+  const int tid = threadIdx.x;
+  for (int k = tid; k < cnt; k += kVjThreads) {
+    const int64_t i = vj_index(g, mp, grid, c0 + k);
+    const float2 p = xi ? xi[i] : grid_point(g, i);
+    const float2 d = dbeta[i];
+    if (lens_terms) {  // each chunk is staged once with them: the point's lens and shear terms
+      float o5[5];
+      sple_vjp(L, LG, p.x, p.y, d.x, d.y, o5);
+#pragma unroll
+      for (int t = 0; t < 5; ++t) la[t] += o5[t];
+      la[5] -= fmaf(d.x, p.x, -d.y * p.y);  // dalpha/dg1 = (x, -y)
+      la[6] -= fmaf(d.x, p.y, d.y * p.x);   // dalpha/dg2 = (y, x)
+    }
+    float* ps = reinterpret_cast<float*>(&sm.pos[k >> 1]);
+    float* gs = reinterpret_cast<float*>(&sm.grad[k >> 1]);
+    const int lane2 = k & 1;
+    ps[lane2] = p.x;
+    ps[2 + lane2] = p.y;
+    gs[lane2] = d.x;
+    gs[2 + lane2] = d.y;
+    if (k == cnt - 1 && lane2 == 0) {  // odd count: a zero-gradient partner at the same position
+      ps[1] = p.x;
+      ps[3] = p.y;
+      gs[1] = 0.f;
+      gs[3] = 0.f;
+    }
+  }
+  __syncthreads();
+}
+
+// The tile's lens terms: warp shuffles then the warps in fixed order, FP64.
+__device__ __forceinline__ void vj_lens_out(const float (&la)[7], double* __restrict__ out, VjSmem& sm) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+  for (int t = 0; t < 7; ++t) {
+    const double v = warp_sum_d((double)la[t]);
+    if (lane == 0) sm.lred[warp][t] = v;
+  }
+  __syncthreads();
+  if (tid < 7) {
+    double v = 0.0;
+    for (int w = 0; w < kVjWarps; ++w) v += sm.lred[w][tid];
+    out[tid] = v;
+  }
+}
+
 template <int PROFILE>
 __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst& LG, const GridDev& g,
                                          const float2* __restrict__ xi, int64_t n, const float* __restrict__ sub,
@@ -641,7 +780,7 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
                                          const float2* __restrict__ dbeta, double* __restrict__ lens_part,
                                          float* __restrict__ sub_part, float* __restrict__ slot_part, int64_t blk,
                                          int64_t nblk, VjSmem& sm) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const bool grid = xi == nullptr;
   // the lens partials are indexed by tile, the subhalo and slot partials by
   // launch position: CTAs that run together write neighbouring words
@@ -649,8 +788,6 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
   const VjMap mp = vj_map(g, grid, n, bands, tile, nblk);
   const int64_t p0 = mp.u0, p1 = mp.u1;
   const int nchunks = (int)((p1 - p0 + kVjChunk - 1) / kVjChunk);
-  const int slots = n_sub * P;
-  const int ngroups = slots > 0 ? (slots + kVjThreads - 1) / kVjThreads : 1;
   float la[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   int staged = -1;
   // tNFW: the subhalos in the order of their classes for the tile's box
@@ -658,15 +795,28 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
   // index order. Each slot finds its subhalo's class itself (vj_class). The
   // local expansion needs one phase and one staged chunk.
   const bool ordered = PROFILE == LR_PROFILE_TNFW && n_sub > 0 && n_sub <= kVjMaxOrd;
-  const bool exp_ok = ordered && P == 1 && nchunks == 1;
+  const bool one = ordered && nchunks == 1;  // one staged chunk: vj_tile_sums takes the subhalos
+  const bool exp_ok = vj_exp_ok(one, (int)(p1 - p0));
   const unsigned short* ord = plan.ord ? plan.ord + tile * n_sub : sm.ord;
   if (PROFILE == LR_PROFILE_TNFW) {
     vj_box(g, xi, mp, sm.wbox, sm.box);
-    if (ordered && !plan.ord) vj_sort(sub, n_sub, sm.box, exp_ok, (int)(p1 - p0), sm.deg, sm.ord);
+    if (ordered && !plan.ord) vj_sort(sub, n_sub, sm.box, exp_ok, (int)(p1 - p0), sm.deg, sm.ord, &sm.nexp);
   }
-  const float2 cen = make_float2(0.5f * (sm.box[0] + sm.box[2]), 0.5f * (sm.box[1] + sm.box[3]));
-  const float hx = 0.5f * (sm.box[2] - sm.box[0]), hy = 0.5f * (sm.box[3] - sm.box[1]);
-  const float hd2 = fmaf(hx, hx, hy * hy);  // the tile's half-diagonal squared
+  if constexpr (PROFILE == LR_PROFILE_TNFW) {
+    if (one) {
+      const int cnt = (int)(p1 - p0);
+      vj_stage(L, LG, g, xi, mp, grid, dbeta, p0, cnt, true, la, sm);
+      vj_lens_out(la, lens_part + tile * 7, sm);  // its barrier also ends the staging
+      const float2 cen = make_float2(0.5f * (sm.box[0] + sm.box[2]), 0.5f * (sm.box[1] + sm.box[3]));
+      const float hx = 0.5f * (sm.box[2] - sm.box[0]), hy = 0.5f * (sm.box[3] - sm.box[1]);
+      const int nexp = plan.nexp ? plan.nexp[tile] : sm.nexp;
+      if (nexp > 0) vj_moments(sm, cnt, cen);  // uniform over the CTA
+      vj_tile_sums(sub, n_sub, nexp, ord, cnt, cen, fmaf(hx, hx, hy * hy), sub_part, blk, nblk, sm);
+      return;
+    }
+  }
+  const int slots = n_sub * P;
+  const int ngroups = slots > 0 ? (slots + kVjThreads - 1) / kVjThreads : 1;
 
   for (int grp = 0; grp < ngroups; ++grp) {
     const int slot = grp * kVjThreads + tid;
@@ -676,14 +826,14 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
     const int h = ordered ? (int)ord[hs] : hs;
     SubRec rec{};
     SubSer q{};
-    int deg = 0;  // class for the tile (vj_class): series degree, 0 the closed forms, | kVjExpFlag
+    int deg = 0;  // class for the tile (vj_class): series degree, 0 the closed forms
     float2 ex = make_float2(0.f, 0.f);  // tNFW: (4T, 1/theta_s); point mass: (0, theta_pm)
     if (own) {
       const float* rr = sub + 5 * (int64_t)h;
       rec = prep_sub(rr, PROFILE);
       if (PROFILE == LR_PROFILE_TNFW) {
         q = prep_series(rec, PROFILE);
-        deg = vj_class(rec, q, sm.box, exp_ok);
+        deg = vj_class(rec, q, sm.box, false);
       }
       if (PROFILE == LR_PROFILE_POINT_MASS) {
         ex = make_float2(0.f, __ldg(rr + 2));
@@ -698,89 +848,24 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
       const int cnt = (int)min((int64_t)kVjChunk, p1 - c0);
       if (ch != staged) {  // uniform over the CTA
         __syncthreads();   // the previous chunk's readers are done
-        for (int k = tid; k < cnt; k += kVjThreads) {
-          const int64_t i = vj_index(g, mp, grid, c0 + k);
-          const float2 p = xi ? xi[i] : grid_point(g, i);
-          const float2 d = dbeta[i];
-          if (grp == 0) {  // each chunk is staged once in group 0: the point's lens and shear terms
-            float o5[5];
-            sple_vjp(L, LG, p.x, p.y, d.x, d.y, o5);
-#pragma unroll
-            for (int t = 0; t < 5; ++t) la[t] += o5[t];
-            la[5] -= fmaf(d.x, p.x, -d.y * p.y);  // dalpha/dg1 = (x, -y)
-            la[6] -= fmaf(d.x, p.y, d.y * p.x);   // dalpha/dg2 = (y, x)
-          }
-          float* ps = reinterpret_cast<float*>(&sm.pos[k >> 1]);
-          float* gs = reinterpret_cast<float*>(&sm.grad[k >> 1]);
-          const int lane2 = k & 1;
-          ps[lane2] = p.x;
-          ps[2 + lane2] = p.y;
-          gs[lane2] = d.x;
-          gs[2 + lane2] = d.y;
-          if (k == cnt - 1 && lane2 == 0) {  // odd count: a zero-gradient partner at the same position
-            ps[1] = p.x;
-            ps[3] = p.y;
-            gs[1] = 0.f;
-            gs[3] = 0.f;
-          }
-        }
-        __syncthreads();
+        vj_stage(L, LG, g, xi, mp, grid, dbeta, c0, cnt, grp == 0, la, sm);
         staged = ch;
-        if (exp_ok && grp == 0) vj_moments(sm, cnt, cen);  // uniform over the CTA
       }
-      if (own && (deg & kVjExpFlag)) {
-        // the local expansion about the tile's centre: the four sums whole
-        const float* rr = sub + 5 * (int64_t)h;
-        const float kap = __ldg(rr + 2), ts = __ldg(rr + 3);
-        const float4 e = vj_expand(rec, q, kap, ts, deg & (kVjExpFlag - 1), cen, hd2, sm);
-        sc[0] = e.x;
-        sc[1] = e.y;
-        sc[2] = e.z;
-        sc[3] = e.w;
-      } else if (own) {
+      if (own) {
         const int np = (cnt + 1) >> 1;
-        if (P == 1) {
-          switch (deg) {
-            case 3:
-              vj_sweep<PROFILE, 3, true>(rec, ex, q, sm.pos, sm.grad, np, r, 1, sc, cc);
-              break;
-            case 4:
-              vj_sweep<PROFILE, 4, true>(rec, ex, q, sm.pos, sm.grad, np, r, 1, sc, cc);
-              break;
-            case 5:
-              vj_sweep<PROFILE, 5, true>(rec, ex, q, sm.pos, sm.grad, np, r, 1, sc, cc);
-              break;
-            case 7:
-              vj_sweep<PROFILE, 7, true>(rec, ex, q, sm.pos, sm.grad, np, r, 1, sc, cc);
-              break;
-            default:
-              vj_sweep<PROFILE, 0, true>(rec, ex, q, sm.pos, sm.grad, np, r, 1, sc, cc);
-          }
-        } else {
-          switch (deg) {
-            case 3:
-              vj_sweep<PROFILE, 3, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
-              break;
-            case 4:
-              vj_sweep<PROFILE, 4, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
-              break;
-            case 5:
-              vj_sweep<PROFILE, 5, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
-              break;
-            case 7:
-              vj_sweep<PROFILE, 7, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
-              break;
-            default:
-              vj_sweep<PROFILE, 0, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
-          }
+        switch (deg) {
+          case 3: vj_sweep<PROFILE, 3, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+          case 4: vj_sweep<PROFILE, 4, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+          case 5: vj_sweep<PROFILE, 5, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+          case 7: vj_sweep<PROFILE, 7, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+          default: vj_sweep<PROFILE, 0, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
         }
       }
     }
     if (own) {
-      const bool expd = (deg & kVjExpFlag) != 0;  // sc holds the expansion's sums, already scaled
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
-        const float x = expd ? sc[v] : __fmul_rn(sc[v] - cc[v], vj_scale<PROFILE>(rec, ex, v));
+        const float x = __fmul_rn(sc[v] - cc[v], vj_scale<PROFILE>(rec, ex, v));
         if (P == 1)
           sub_part[((int64_t)h * 4 + v) * nblk + blk] = x;  // [value][CTA], h the subhalo itself
         else
@@ -802,18 +887,7 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
     }
   }
 
-  // lens terms: warp shuffles then the warps in fixed order, FP64
-#pragma unroll
-  for (int t = 0; t < 7; ++t) {
-    const double v = warp_sum_d((double)la[t]);
-    if (lane == 0) sm.lred[warp][t] = v;
-  }
-  __syncthreads();
-  if (tid < 7) {
-    double v = 0.0;
-    for (int w = 0; w < kVjWarps; ++w) v += sm.lred[w][tid];
-    lens_part[tile * 7 + tid] = v;
-  }
+  vj_lens_out(la, lens_part + tile * 7, sm);
 }
 
 template <int PROFILE>
@@ -852,9 +926,9 @@ __global__ void __launch_bounds__(kVjThreads, 4) raytrace_vjp_rec_kernel(const L
 // (vj_sort) into ord, and writes the tile's work (FP32 lanes over its
 // point-subhalo pairs, the expansion's per tile) to weight.
 __global__ void __launch_bounds__(kVjThreads) vjp_plan_kernel(GridDev g, const float2* __restrict__ xi, int64_t n,
-                                                              const float* __restrict__ sub, int n_sub, int P,
+                                                              const float* __restrict__ sub, int n_sub,
                                                               int bands, int64_t ntiles,
-                                                              unsigned short* __restrict__ ord,
+                                                              unsigned short* __restrict__ ord, int* __restrict__ nexp,
                                                               float* __restrict__ weight) {
   __shared__ float wbox[kVjWarps][4], box[4], wsum[kVjWarps];
   __shared__ unsigned char cls[kVjMaxOrd];
@@ -862,9 +936,9 @@ __global__ void __launch_bounds__(kVjThreads) vjp_plan_kernel(GridDev g, const f
   const VjMap mp = vj_map(g, xi == nullptr, n, bands, tile, ntiles);
   vj_box(g, xi, mp, wbox, box);
   const int npts = (int)(mp.u1 - mp.u0);
-  // the same choice as the sweep's (vjp_body): one phase and one staged chunk
-  const bool exp_ok = P == 1 && npts > 0 && npts <= kVjChunk;
-  float c = vj_sort(sub, n_sub, box, exp_ok, npts, cls, ord + tile * n_sub);
+  // the same choice as the sweep's (vjp_body)
+  const bool exp_ok = vj_exp_ok(npts <= kVjChunk, npts);
+  float c = vj_sort(sub, n_sub, box, exp_ok, npts, cls, ord + tile * n_sub, nexp + tile);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = c;
@@ -1093,13 +1167,14 @@ lr_status make_lens_grad_const(const lr_lens* lens, LensGradConst* out) {
 
 // Workspace: per-tile lens partials [tile][7] (FP64), subhalo partials
 // [4 n_sub][CTA], with P > 1 the slot sums [CTA][n_sub P][4], and where a
-// plan fits (plan_fits) its subhalo orders [tile][n_sub] (16 bit), tile
-// weights and the permutation of the tiles.
+// plan fits (plan_fits) its subhalo orders [tile][n_sub] (16 bit), the
+// expansion's counts, tile weights and the permutation of the tiles.
 struct VjWs {
   double* lens_part;
   float* sub_part;
   float* slot_part;
   unsigned short* ord;
+  int* nexp;
   float* weight;
   int* perm;
   size_t bytes;
@@ -1127,6 +1202,7 @@ static VjWs vjp_ws_layout(void* ws, int64_t n, int32_t n_sub) {
   w.sub_part = reinterpret_cast<float*>(at(b_sub));
   w.slot_part = reinterpret_cast<float*>(at(b_slot));
   w.ord = reinterpret_cast<unsigned short*>(at(b_ord));
+  w.nexp = reinterpret_cast<int*>(at(b_perm));
   w.weight = reinterpret_cast<float*>(at(b_w));
   w.perm = reinterpret_cast<int*>(at(b_perm));
   w.bytes = off;
@@ -1163,13 +1239,13 @@ lr_status launch_raytrace_vjp(const lr_points* p, const float2* dbeta, double* d
   LR_REQUIRE(fault != nullptr, "could not resolve the device fault word");
   VjPlan plan{};
   if (vjp_planned(nblk, p)) {
-    vjp_plan_kernel<<<(unsigned)nblk, kVjThreads, 0, s>>>(g, xi, p->n, p->sub, p->n_sub, P, bands, nblk, w.ord,
-                                                          w.weight);
+    vjp_plan_kernel<<<(unsigned)nblk, kVjThreads, 0, s>>>(g, xi, p->n, p->sub, p->n_sub, bands, nblk, w.ord,
+                                                          w.nexp, w.weight);
     LR_CHECK_CUDA(cudaGetLastError());
     vjp_rank_kernel<<<(unsigned)((nblk + 3) / 4), 128, sizeof(float) * (size_t)nblk, s>>>(w.weight, (int)nblk,
                                                                                           w.perm);
     LR_CHECK_CUDA(cudaGetLastError());
-    plan = VjPlan{w.perm, w.ord};
+    plan = VjPlan{w.perm, w.ord, w.nexp};
   }
   ktimer_begin(LR_KT_RAYTRACE_VJP, s);
   if (rec && p->profile == LR_PROFILE_POINT_MASS)
