@@ -83,6 +83,13 @@ def vj_ser_lanes(k: int) -> float:
 # per tile and subhalo, whatever the tile's point count; its moments add
 # about 31 operations per point and term, once per tile (not counted).
 VJ_EXP_LANES_PER_TERM = 40.0
+# The forward's expansion (grids with rows of 160 points, from 64 subhalos on,
+# 40 + n_sub / 4 of them at least 12.5 half-diagonals away): 24 independent
+# terms of 9 FP32 operations (6 series terms, the scale, 2 sums) and 34 for
+# the powers, per tile and subhalo; the polynomial, 36 terms per point, and
+# the classes of the subhalos are not counted.
+RT_EXP_LANES = 250.0
+RT_EXP_MIN, RT_EXP_WIDTH = 64, 160
 
 
 def _grid_axes(g):
@@ -93,12 +100,13 @@ def _grid_axes(g):
     return w, hgt, xs, ys
 
 
-def _degree_shares(p, boxes, counts, degrees, expand=False) -> dict:
+def _degree_shares(p, boxes, counts, degrees, expand=None) -> dict:
     """Share of the point-subhalo pairs by the series degree that serves a
     CTA's whole box (x_lo, y_lo, x_hi, y_hi) of `counts` points; 0: the
-    closed forms. With `expand`, the pairs of a far subhalo whose distance
-    from the box's centre is at least 12.5 half-diagonals go to the key
-    "expansion" (the ray-trace backward's local expansion)."""
+    closed forms. With `expand` ("forward" or "backward"), the pairs of a far
+    subhalo (x^2 >= 64 max(tau^2, 4)) whose distance from the box's centre is
+    at least 12.5 half-diagonals go to the key "expansion" (that kernel's
+    local expansion)."""
     sub = p.sub.astype(np.float64)
     its2 = 1.0 / sub[:, 3] ** 2
     m = np.maximum(sub[:, 4] ** 2, 4.0)
@@ -117,12 +125,18 @@ def _degree_shares(p, boxes, counts, degrees, expand=False) -> dict:
             cx = 0.5 * (bx[:, 0] + bx[:, 2])[:, None] - sub[None, :, 0]
             cy = 0.5 * (bx[:, 1] + bx[:, 3])[:, None] - sub[None, :, 1]
             c2 = cx * cx + cy * cy
-            hit = (x2 >= degrees[-1][1]) & (hd2[:, None] <= 0.0064 * c2) & (cn[:, None] <= 2048)
+            hit = (x2 >= 64.0) & (hd2[:, None] <= 0.0064 * c2)
+            if expand == "forward":
+                far = (hd2[:, None] <= 0.0064 * c2).sum(1, keepdims=True)
+                hit &= (hd2[:, None] > 0) & (far >= 40 + len(sub) // 4)
+            else:
+                hit &= (cn[:, None] <= 2048) & (cn[:, None] >= 64)
             tot["expansion"] += float((hit.sum(1) * cn).sum())
             # terms of the expansion's order: 15, 21, 28 or 36 for (half-diagonal / |c|) up to 0.01, 0.03, 0.05, 0.08
             r2 = hd2[:, None] / c2
             terms = np.where(r2 <= 1e-4, 15, np.where(r2 <= 9e-4, 21, np.where(r2 <= 2.5e-3, 28, 36)))
-            exp_lanes += float(np.sum(np.where(hit, VJ_EXP_LANES_PER_TERM * terms + 30.0, 0.0)))
+            lanes = RT_EXP_LANES if expand == "forward" else VJ_EXP_LANES_PER_TERM * terms + 30.0
+            exp_lanes += float(np.sum(np.where(hit, lanes, 0.0)))
             left &= ~hit
         for k, r2 in degrees:
             hit = left & (x2 >= r2)
@@ -139,16 +153,18 @@ def raytrace_cost(p):
     """(MUFU, FP32 lanes) per point-subhalo pair of the forward ray-trace on
     a pixel grid, and the pairs' shares by series degree: a CTA takes a
     16 x 16 tile of pixels, a subhalo takes the series of the degree that
-    serves the whole tile, the others the far-side closed form."""
+    serves the whole tile, the others the far-side closed form; from
+    RT_EXP_MIN subhalos on, the far ones take the local expansion."""
     w, hgt, xs, ys = _grid_axes(p.xgrid)
     tw, th = (w + 15) // 16, (hgt + 15) // 16
     ty, tx = np.divmod(np.arange(tw * th), tw)
     r0, c0 = ty * 16, tx * 16
     r1, c1 = np.minimum(r0 + 16, hgt) - 1, np.minimum(c0 + 16, w) - 1
     boxes = np.stack([xs[c0], ys[r0], xs[c1], ys[r1]], 1)
-    sh = _degree_shares(p, boxes, (r1 - r0 + 1) * (c1 - c0 + 1), RT_DEGREES)
-    mufu = sh[0] * RT_MUFU + (1 - sh[0]) * SER_MUFU
-    lanes = sh[0] * RT_LANES + sum(sh[k] * rt_ser_lanes(k) for k, _ in RT_DEGREES)
+    sh = _degree_shares(p, boxes, (r1 - r0 + 1) * (c1 - c0 + 1), RT_DEGREES,
+                        expand="forward" if len(p.sub) >= RT_EXP_MIN and w >= RT_EXP_WIDTH else None)
+    mufu = sh[0] * RT_MUFU + sum(sh[k] for k, _ in RT_DEGREES) * SER_MUFU
+    lanes = sh[0] * RT_LANES + sum(sh[k] * rt_ser_lanes(k) for k, _ in RT_DEGREES) + sh["expansion_lanes"]
     return mufu, lanes, sh
 
 
@@ -167,10 +183,11 @@ def vjp_bands(nblk: int, w: int, hgt: int) -> int:
 
 
 def vjp_phases(n: int, nblk: int, n_sub: int) -> int:
-    """Slots per subhalo of the ray-trace backward: 1 when n_sub slots waste
-    at most 5 % of the last 128 threads, else the P in [1, 8] whose n_sub P
-    wastes the fewest of them, keeping 128 points per slot (the local
-    expansion needs P = 1)."""
+    """Slots per subhalo of the ray-trace backward's tiles that take no
+    expansion (more than 4096 subhalos, or more points than one staged
+    chunk): 1 when n_sub slots waste at most 5 % of the last 128 threads, else
+    the P in [1, 8] whose n_sub P wastes the fewest of them, keeping 128
+    points per slot."""
     per = -(-n // nblk)
     if -(-n_sub // 128) * 128 <= 1.05 * n_sub:
         return 1
@@ -204,7 +221,7 @@ def vjp_cost(p, nblk: int):
     rlo = np.where(one, u0 % rows, 0)
     rhi = np.where(one, (u1 - 1) % rows, rows - 1)
     boxes = np.stack([xs[col0], ys[row0 + rlo], xs[col1], ys[row0 + rhi]], 1)
-    sh = _degree_shares(p, boxes, u1 - u0, VJ_DEGREES, expand=vjp_phases(p.n, nblk, len(p.sub)) == 1)
+    sh = _degree_shares(p, boxes, u1 - u0, VJ_DEGREES, expand="backward" if len(p.sub) <= 4096 else None)
     mufu = sh[0] * VJ_MUFU + sum(sh[k] for k, _ in VJ_DEGREES) * SER_MUFU
     lanes = (sh[0] * VJ_LANES + sum(sh[k] * vj_ser_lanes(k) for k, _ in VJ_DEGREES) + sh["expansion_lanes"])
     return mufu, lanes, sh

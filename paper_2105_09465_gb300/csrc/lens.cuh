@@ -367,6 +367,21 @@ __device__ __forceinline__ float2 c2mul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
+// After it, lane i holds the warp's total of v[i] (fixed order).
+__device__ __forceinline__ float warp_scatter32(float (&v)[32], int lane) {
+#pragma unroll
+  for (int h = 16; h >= 1; h >>= 1) {
+    const bool upper = (lane & h) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float send = upper ? v[i] : v[i + h];
+      const float keep = upper ? v[i + h] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+    }
+  }
+  return v[0];
+}
+
 // The truncation order of an expansion for (tile half-diagonal / |c|)^2 =
 // hd2 / r2: 4 up to a ratio of 0.01, 5 up to 0.03, 6 up to 0.05, 7 up to
 // 0.08 (the largest served). Each keeps the truncation below 5e-9 of the

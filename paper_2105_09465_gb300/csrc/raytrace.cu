@@ -8,7 +8,9 @@
 // point of the CTA. Each chunk is sorted by the degree of the far-field
 // series that serves the whole tile (rt_degree, fewest terms first), and each
 // degree's run is swept without per-pair tests; the rest take a per-pair
-// choice of series, far-side closed form or general form. Stores are
+// choice of series, far-side closed form or general form. Where many subhalos
+// are far from a grid tile (rt_expands), those are summed as one local
+// expansion about its centre and only the others are staged. Stores are
 // coalesced float2 writes.
 #include <math.h>
 
@@ -25,6 +27,13 @@ constexpr int kRtPoints = kRtThreads * kRtPts;   // points per CTA
 constexpr int kRtTile = 16;  // grid input: a CTA takes a kRtTile x kRtTile tile of pixels
 static_assert(kRtTile * kRtTile == kRtPoints, "the CTA's points are one tile");
 constexpr int kSubChunk = 256;  // subhalos staged per chunk (multiple of 4)
+constexpr int kRtWin = 2048;     // subhalos per window of the local expansion (16-bit places)
+// The local expansion may serve grids from 64 subhalos and rows of 160 points
+// on (a tile's half-diagonal is 10.6 spacings, so a subhalo is far from 133 on;
+// by the width alone, so that a band of rows takes what the whole image takes);
+// the tiles then decide (rt_expands). Other launches take a kernel without it.
+constexpr int kRtExpMin = 64, kRtExpSide = 160;
+constexpr int kRtExpFloats = 44;  // floats of the expansion's independent coefficients (rt_exp_at)
 
 __global__ void grid_points_kernel(GridDev g, int64_t n, float2* out) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -58,6 +67,10 @@ struct RtSmem {
   float box[4];          // the CTA's points: x_lo, y_lo, x_hi, y_hi
   int nfar;
   uint64_t bar;
+  unsigned short list[kRtWin];        // the window's subhalos that the expansion does not serve, in index order
+  int lcnt[2][kRtThreads / 32];       // per warp: how many of them this round of threads holds
+  float mred[kRtThreads / 32][kRtExpFloats];  // per-warp sums of the expansion's independent coefficients
+  float2 coef[(kExpN + 1) * (kExpN + 2) / 2];  // the tile's coefficients: by l, then k (rt_coef_at)
 };
 
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
@@ -105,15 +118,25 @@ __device__ __forceinline__ int rt_degree(float x2min, float m) {
                                 : 0;
 }
 
-// Stages subhalos [h0, h0 + cnt). Subhalos whose centre is beyond the series
+// Stages subhalos [h0, h0 + cnt), of the window's list where one is given (sub
+// then points at the window). Subhalos whose centre is beyond the series
 // radius from the whole box of the CTA's points (every pair of them takes the
 // series) come first, ordered by the degree that serves the whole box
 // (rt_degree, fewest terms first), each degree in index order; sm.ndeg
 // counts them by degree and sm.nfar in all. Returns false (all threads) if
 // the bulk-copy wait timed out.
 __device__ __forceinline__ bool stage_rt(const float* __restrict__ sub, int h0, int cnt, int profile, RtSmem& sm,
-                                         uint32_t& phase, bool bulk_ok, int* fault) {
-  if (!stage_raw(sub, h0, cnt, sm.raw, &sm.bar, phase, bulk_ok, fault)) return false;
+                                         uint32_t& phase, bool bulk_ok, int* fault,
+                                         const unsigned short* list = nullptr) {
+  if (list) {
+    for (int w = threadIdx.x; w < 5 * cnt; w += kRtThreads) {
+      const int t = w / 5;
+      sm.raw[w] = __ldg(sub + 5 * (int64_t)list[h0 + t] + (w - 5 * t));
+    }
+    __syncthreads();
+  } else if (!stage_raw(sub, h0, cnt, sm.raw, &sm.bar, phase, bulk_ok, fault)) {
+    return false;
+  }
   for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
     const SubRec h = prep_sub(sm.raw + 5 * t, profile);
     const SubSer q = prep_series(h, profile);
@@ -385,7 +408,220 @@ __device__ __forceinline__ void add_subs(const RtSmem& sm, int cnt, const float 
   }
 }
 
-template <int PROFILE>
+// ---------------------------------------------------------------------------
+// Local expansion of the far subhalos about a tile's centre (grid tiles).
+//
+// The deflection of a subhalo whose series of degree 7 serves the whole tile
+// and whose distance |c| from the tile's centre is at least 12.5 half-
+// diagonals h is (lens.cuh, with u = 1/c and delta in units of h)
+//   alpha = (A theta_s^2 / h) sum_{k+l<=7} c_kl (h u)^k (h conj(u))^(l+1) delta^k conj(delta)^l,
+//   c_kl = sum_j q_j (theta_s / |c|)^j C(-j/2, k) C(-(j+2)/2, l).
+// The coefficients of all such subhalos add, so the tile sums them once, a
+// subhalo to a thread, and each point evaluates one polynomial of 36 terms:
+// about 250 FP32 lanes per subhalo and tile instead of 13.5 per subhalo and
+// point, of which a tile has 256. 2.56M points x 2000 subhalos: 2.59 -> 0.57
+// ms. alpha is the gradient of a real potential, so k c_kl = (l + 1)
+// c_(l+1)(k-1): only the 24 terms with m = l + 1 - k >= 0 are summed,
+// (h u)^k (h conj(u))^(l+1) = (h |u|)^2k (h conj(u))^m, those of m = 0 real.
+// The truncation is below 5e-9 of the sum of absolute terms.
+
+// First float of the term (m, k): m = 0 holds k = 1..4, m > 0 holds k = 0 ..
+// (8 - m) / 2 as complex values.
+__device__ constexpr int rt_exp_at(int m, int k) {
+  if (m == 0) return k - 1;
+  int at = 4;
+  for (int i = 1; i < m; ++i) at += 2 * ((kExpN + 1 - i) / 2 + 1);
+  return at + 2 * k;
+}
+static_assert(rt_exp_at(kExpN + 1, 0) + 2 == kRtExpFloats, "the last term ends the floats");
+
+// Place of the coefficient of delta^k conj(delta)^l: by l, then k.
+__device__ constexpr int rt_coef_at(int k, int l) { return l * (2 * kExpN + 3 - l) / 2 + k; }
+
+struct RtExpBin {
+  float ab[kExpN + 2][kExpN / 2 + 2][8];  // C(-j/2, k) C(-(j+2)/2, k + m - 1) of (m, k, j)
+};
+constexpr RtExpBin rt_make_bin() {
+  RtExpBin t{};
+  const ExpBin b = exp_make_bin();
+  for (int m = 0; m <= kExpN + 1; ++m)
+    for (int k = m == 0 ? 1 : 0; k <= (kExpN + 1 - m) / 2; ++k)
+      for (int j = 0; j < 8; ++j) t.ab[m][k][j] = b.a[j][k] * b.b[j][k + m - 1];
+  return t;
+}
+static __constant__ RtExpBin kRtBin = rt_make_bin();
+
+// Adds one subhalo's coefficients (c: the tile's centre less the subhalo's,
+// r2 = |c|^2).
+__device__ __forceinline__ void rt_exp_add(const SubRec& rec, const SubSer& q, float ts, float2 c, float r2, float h,
+                                           float (&acc)[kRtExpFloats]) {
+  const float ir2 = 1.0f / r2, yc = ts * sqrtf(ir2);
+  float qy[8], yj = rec.A * ts * ts / h;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    qy[j] = q.q[j] * yj;  // q1 = 0
+    yj *= yc;
+  }
+  const float hr = h * ir2, rho2 = h * hr;
+  const float2 ub = make_float2(c.x * hr, c.y * hr);  // h conj(u)
+  float rk[kExpN / 2 + 2];
+  rk[0] = 1.f;
+#pragma unroll
+  for (int k = 1; k < kExpN / 2 + 2; ++k) rk[k] = rk[k - 1] * rho2;
+  float2 um = make_float2(1.f, 0.f);
+#pragma unroll
+  for (int m = 0; m <= kExpN + 1; ++m) {
+    if (m > 0) um = m == 1 ? ub : c2mul(um, ub);
+#pragma unroll
+    for (int k = m == 0 ? 1 : 0; k <= (kExpN + 1 - m) / 2; ++k) {
+      float s = k == 0 ? qy[0] * kRtBin.ab[m][k][0] : 0.f;  // C(0, k) = 0 for k > 0
+#pragma unroll
+      for (int j = 2; j < 8; ++j) s = fmaf(qy[j], kRtBin.ab[m][k][j], s);
+      const int at = rt_exp_at(m, k);
+      if (m == 0) {
+        acc[at] = fmaf(s, rk[k], acc[at]);
+      } else {
+        if (k > 0) s *= rk[k];
+        acc[at] = fmaf(s, um.x, acc[at]);
+        acc[at + 1] = fmaf(s, um.y, acc[at + 1]);
+      }
+    }
+  }
+}
+
+// Whether the tile takes the expansion: where at least 40 + n_sub / 4 subhalos
+// are 12.5 half-diagonals from its centre. A far subhalo saves about 15 issue
+// slots per thread (two points); the expansion costs some 600 once and 500 per
+// 128 subhalos, far or not. 640k points: 200 subhalos 90 -> 59 us, 500 197 ->
+// 87 us; 16k points, 128 subhalos, few of them far, 24.5 us without and 26.9
+// with it.
+__device__ __forceinline__ bool rt_expands(const float* __restrict__ sub, int n_sub, float2 cen, float hd2,
+                                           RtSmem& sm) {
+  int far = 0;
+  for (int h = threadIdx.x; h < n_sub; h += kRtThreads) {
+    const float dx = cen.x - __ldg(sub + 5 * (int64_t)h), dy = cen.y - __ldg(sub + 5 * (int64_t)h + 1);
+    far += hd2 <= kExpRatio2 * fmaf(dx, dx, dy * dy);
+  }
+  far = __reduce_add_sync(0xffffffffu, far);
+  if ((threadIdx.x & 31) == 0) sm.lcnt[1][threadIdx.x >> 5] = far;  // rt_expand_window starts with the other half
+  __syncthreads();
+  far = 0;
+  for (int w = 0; w < kRtThreads / 32; ++w) far += sm.lcnt[1][w];
+  return far >= 40 + n_sub / 4;
+}
+
+// The window's wn subhalos at sub: those far enough from the tile are summed
+// into sm.coef (added where add), the others listed in sm.list in index
+// order. Returns the list's length. All threads of the CTA take part.
+__device__ __forceinline__ int rt_expand_window(const float* __restrict__ sub, int wn, bool add, float2 cen, float hd2,
+                                                RtSmem& sm) {
+  constexpr int kW = kRtThreads / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float h = sqrtf(hd2);
+  float acc[kRtExpFloats];
+#pragma unroll
+  for (int i = 0; i < kRtExpFloats; ++i) acc[i] = 0.f;
+  int nl = 0;
+  for (int base = 0, it = 0; base < wn; base += kRtThreads, it ^= 1) {
+    const int t = base + tid;
+    bool direct = t < wn;
+    if (direct) {
+      float r[5];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) r[i] = __ldg(sub + 5 * t + i);
+      const SubRec rec = prep_sub(r, LR_PROFILE_TNFW);
+      const SubSer q = prep_series(rec, LR_PROFILE_TNFW);
+      const float dx = fmaxf(fmaxf(sm.box[0] - rec.xh, rec.xh - sm.box[2]), 0.f);
+      const float dy = fmaxf(fmaxf(sm.box[1] - rec.yh, rec.yh - sm.box[3]), 0.f);
+      const float2 c = make_float2(cen.x - rec.xh, cen.y - rec.yh);
+      const float r2 = fmaf(c.x, c.x, c.y * c.y);
+      if (!isinf(q.xT2) && fmaf(dx, dx, dy * dy) * rec.its2 >= 64.0f * fmaxf(rec.tau2, 4.0f) &&
+          hd2 <= kExpRatio2 * r2) {
+        direct = false;
+        rt_exp_add(rec, q, r[3], c, r2, h, acc);
+      }
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, direct);
+    if (lane == 0) sm.lcnt[it][warp] = __popc(m);
+    __syncthreads();  // the other half of lcnt is written before the next one
+    int before = nl;
+#pragma unroll
+    for (int w = 0; w < kW; ++w) {
+      const int x = sm.lcnt[it][w];
+      before += w < warp ? x : 0;
+      nl += x;
+    }
+    if (direct) sm.list[before + __popc(m & ((1u << lane) - 1u))] = (unsigned short)t;
+  }
+#pragma unroll
+  for (int b = 0; b < kRtExpFloats; b += 32) {
+    float v[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = b + i < kRtExpFloats ? acc[b + i < kRtExpFloats ? b + i : 0] : 0.f;
+    const float t = warp_scatter32(v, lane);
+    if (b + lane < kRtExpFloats) sm.mred[warp][b + lane] = t;
+  }
+  __syncthreads();
+  if (tid < (kExpN + 1) * (kExpN + 2) / 2) {
+    int l = 0;
+    while (rt_coef_at(0, l + 1) <= tid) ++l;
+    const int k = tid - rt_coef_at(0, l);
+    // k <= l + 1: summed itself; else (l + 1) / k of the conjugate of (l + 1, k - 1)
+    const bool own = k <= l + 1;
+    const int m = own ? l + 1 - k : k - l - 1, at = rt_exp_at(m, own ? k : l + 1);
+    float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < kW; ++w) {
+      v.x += sm.mred[w][at];
+      if (m > 0) v.y += sm.mred[w][at + 1];
+    }
+    if (!own) {
+      const float f = (float)(l + 1) / (float)k;
+      v = make_float2(v.x * f, -v.y * f);
+    }
+    if (add) v = make_float2(v.x + sm.coef[tid].x, v.y + sm.coef[tid].y);
+    sm.coef[tid] = v;
+  }
+  __syncthreads();
+  return nl;
+}
+
+// The expansion at the thread's points, added to their Kahan sums: Horner in
+// delta, then in conj(delta), both points packed.
+__device__ __forceinline__ void rt_expand_eval(const RtSmem& sm, float2 cen, float ih, const float (&x)[kRtPts],
+                                               const float (&y)[kRtPts], float (&sx)[kRtPts], float (&cx)[kRtPts],
+                                               float (&sy)[kRtPts], float (&cy)[kRtPts]) {
+  static_assert(kRtPts == 2, "the thread's points are the two lanes");
+  const float2 X = make_float2((x[0] - cen.x) * ih, (x[1] - cen.x) * ih);
+  const float2 Y = make_float2((y[0] - cen.y) * ih, (y[1] - cen.y) * ih), nY = make_float2(-Y.x, -Y.y);
+  float2 ar = f2(0.f), ai = f2(0.f);
+#pragma unroll
+  for (int l = kExpN; l >= 0; --l) {
+    float2 pr = f2(0.f), pi = f2(0.f);
+#pragma unroll
+    for (int k = kExpN - l; k >= 0; --k) {
+      const float2 c = sm.coef[rt_coef_at(k, l)];
+      const float2 r = __ffma2_rn(pr, X, __ffma2_rn(pi, nY, f2(c.x)));
+      pi = __ffma2_rn(pr, Y, __ffma2_rn(pi, X, f2(c.y)));
+      pr = r;
+    }
+    const float2 r = __ffma2_rn(ar, X, __ffma2_rn(ai, Y, pr));
+    ai = __ffma2_rn(ai, X, __ffma2_rn(ar, nY, pi));
+    ar = r;
+  }
+  kahan(sx[0], cx[0], ar.x);
+  kahan(sx[1], cx[1], ar.y);
+  kahan(sy[0], cy[0], ai.x);
+  kahan(sy[1], cy[1], ai.y);
+}
+
+__host__ __device__ __forceinline__ bool rt_may_expand(bool explicit_points, const GridDev& g, int profile,
+                                                       int n_sub) {
+  return !explicit_points && profile == LR_PROFILE_TNFW && n_sub >= kRtExpMin && g.W >= kRtExpSide;
+}
+
+// EXP: grid tiles may take the local expansion.
+template <int PROFILE, bool EXP>
 __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev& g, const float2* __restrict__ xi,
                                               int64_t n, const float* __restrict__ sub, int n_sub, int bulk_ok,
                                               float2* __restrict__ beta, float2* __restrict__ alpha_out, int* fault,
@@ -465,7 +701,27 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
     float sx[kRtPts], cx[kRtPts], sy[kRtPts], cy[kRtPts];
 #pragma unroll
     for (int j = 0; j < kRtPts; ++j) sx[j] = cx[j] = sy[j] = cy[j] = 0.f;
-    for (int h0 = 0; h0 < n_sub; h0 += kSubChunk) {
+    bool expand = false;
+    if constexpr (EXP && PROFILE == LR_PROFILE_TNFW) {
+      const float2 cen = make_float2(0.5f * (sm.box[0] + sm.box[2]), 0.5f * (sm.box[1] + sm.box[3]));
+      const float hx = 0.5f * (sm.box[2] - sm.box[0]), hy = 0.5f * (sm.box[3] - sm.box[1]);
+      const float hd2 = fmaf(hx, hx, hy * hy);  // the tile's half-diagonal squared (0: a single point)
+      expand = hd2 > 0.f && rt_expands(sub, n_sub, cen, hd2, sm);
+      if (expand) {
+        for (int w0 = 0; w0 < n_sub; w0 += kRtWin) {
+          const float* win = sub + 5 * (int64_t)w0;
+          const int nl = rt_expand_window(win, min(kRtWin, n_sub - w0), w0 > 0, cen, hd2, sm);
+          for (int h0 = 0; h0 < nl; h0 += kSubChunk) {
+            const int cnt = min(kSubChunk, nl - h0);
+            stage_rt(win, h0, cnt, PROFILE, sm, phase, false, fault, sm.list);
+            add_subs<PROFILE>(sm, cnt, px, py, sx, cx, sy, cy);
+            __syncthreads();
+          }
+        }
+        rt_expand_eval(sm, cen, 1.0f / sqrtf(hd2), px, py, sx, cx, sy, cy);
+      }
+    }
+    for (int h0 = 0; h0 < n_sub && !expand; h0 += kSubChunk) {
       const int cnt = min(kSubChunk, n_sub - h0);
       if (!stage_rt(sub, h0, cnt, PROFILE, sm, phase, bulk_ok != 0, fault)) return;
       add_subs<PROFILE>(sm, cnt, px, py, sx, cx, sy, cy);
@@ -486,19 +742,19 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
   }
 }
 
-template <int PROFILE>
+template <int PROFILE, bool EXP>
 __global__ void __launch_bounds__(kRtThreads, 5) raytrace_kernel(const __grid_constant__ LensConst L, GridDev g,
                                                               const float2* __restrict__ xi, int64_t n,
                                                               const float* __restrict__ sub, int n_sub, int bulk_ok,
                                                               float2* __restrict__ beta,
                                                               float2* __restrict__ alpha_out, int* fault) {
   __shared__ __align__(16) RtSmem sm;
-  raytrace_body<PROFILE>(L, g, xi, n, sub, n_sub, bulk_ok, beta, alpha_out, fault, blockIdx.x, sm);
+  raytrace_body<PROFILE, EXP>(L, g, xi, n, sub, n_sub, bulk_ok, beta, alpha_out, fault, blockIdx.x, sm);
 }
 
 // The same with the lens read from a device record (lr_lens_prepare); an
 // invalid record is reported in the fault word.
-template <int PROFILE>
+template <int PROFILE, bool EXP>
 __global__ void __launch_bounds__(kRtThreads, 5) raytrace_rec_kernel(const LensRecord* __restrict__ rec, GridDev g,
                                                                   const float2* __restrict__ xi, int64_t n,
                                                                   const float* __restrict__ sub, int n_sub,
@@ -506,7 +762,7 @@ __global__ void __launch_bounds__(kRtThreads, 5) raytrace_rec_kernel(const LensR
                                                                   float2* __restrict__ alpha_out, int* fault) {
   __shared__ __align__(16) RtSmem sm;
   if (rec->status != 0 && blockIdx.x == 0 && threadIdx.x == 0) atomicExch(fault, kFaultBadLens);
-  raytrace_body<PROFILE>(rec->L, g, xi, n, sub, n_sub, bulk_ok, beta, alpha_out, fault, blockIdx.x, sm);
+  raytrace_body<PROFILE, EXP>(rec->L, g, xi, n, sub, n_sub, bulk_ok, beta, alpha_out, fault, blockIdx.x, sm);
 }
 
 __global__ void lens_prepare_kernel(const float* __restrict__ theta7, float gamma, LensRecord* __restrict__ rec) {
@@ -535,11 +791,14 @@ __global__ void __launch_bounds__(kRtThreads, 5) raytrace_batched_kernel(const _
   const RtP& P = B.p[k];
   const int64_t blk = blockIdx.x - B.start[k];
   if (P.profile == LR_PROFILE_POINT_MASS)
-    raytrace_body<LR_PROFILE_POINT_MASS>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault,
+    raytrace_body<LR_PROFILE_POINT_MASS, false>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault,
+                                         blk, sm);
+  else if (rt_may_expand(P.xi != nullptr, P.g, P.profile, P.n_sub))
+    raytrace_body<LR_PROFILE_TNFW, true>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault,
                                          blk, sm);
   else
-    raytrace_body<LR_PROFILE_TNFW>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault, blk,
-                                   sm);
+    raytrace_body<LR_PROFILE_TNFW, false>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault,
+                                          blk, sm);
 }
 
 // CTAs of the ray-trace: kRtPoints points each, or one per grid tile.
@@ -641,18 +900,16 @@ lr_status launch_raytrace(const lr_points* p, float2* beta, float2* alpha, cudaS
   const float2* xi = reinterpret_cast<const float2*>(p->xy);
   const int ns = p->n_sub;
   ktimer_begin(LR_KT_RAYTRACE, s);
-  if (rec && p->profile == LR_PROFILE_POINT_MASS)
-    raytrace_rec_kernel<LR_PROFILE_POINT_MASS><<<blocks, kRtThreads, 0, s>>>(rec, g, xi, p->n, p->sub, ns, bulk_ok,
-                                                                             beta, alpha, fault);
-  else if (rec)
-    raytrace_rec_kernel<LR_PROFILE_TNFW><<<blocks, kRtThreads, 0, s>>>(rec, g, xi, p->n, p->sub, ns, bulk_ok, beta,
-                                                                       alpha, fault);
-  else if (p->profile == LR_PROFILE_POINT_MASS)
-    raytrace_kernel<LR_PROFILE_POINT_MASS><<<blocks, kRtThreads, 0, s>>>(L, g, xi, p->n, p->sub, ns, bulk_ok, beta,
-                                                                         alpha, fault);
-  else
-    raytrace_kernel<LR_PROFILE_TNFW><<<blocks, kRtThreads, 0, s>>>(L, g, xi, p->n, p->sub, ns, bulk_ok, beta, alpha,
-                                                                   fault);
+  const bool pm = p->profile == LR_PROFILE_POINT_MASS, ex = rt_may_expand(p->xy != nullptr, g, p->profile, ns);
+  if (rec) {
+    const auto k = pm ? raytrace_rec_kernel<LR_PROFILE_POINT_MASS, false>
+                   : ex ? raytrace_rec_kernel<LR_PROFILE_TNFW, true> : raytrace_rec_kernel<LR_PROFILE_TNFW, false>;
+    k<<<blocks, kRtThreads, 0, s>>>(rec, g, xi, p->n, p->sub, ns, bulk_ok, beta, alpha, fault);
+  } else {
+    const auto k = pm ? raytrace_kernel<LR_PROFILE_POINT_MASS, false>
+                   : ex ? raytrace_kernel<LR_PROFILE_TNFW, true> : raytrace_kernel<LR_PROFILE_TNFW, false>;
+    k<<<blocks, kRtThreads, 0, s>>>(L, g, xi, p->n, p->sub, ns, bulk_ok, beta, alpha, fault);
+  }
   LR_CHECK_CUDA(cudaGetLastError());
   ktimer_end(LR_KT_RAYTRACE, s);
   return LR_OK;

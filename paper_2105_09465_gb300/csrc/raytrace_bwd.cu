@@ -342,21 +342,6 @@ __device__ __forceinline__ int vj_class(const SubRec& h, const SubSer& q, const 
 // then k.
 __device__ constexpr int vj_moment_at(int k, int l) { return l * (2 * kVjExpN + 3 - l) / 2 + k; }
 
-// After it, lane i holds the warp's total of v[i] (fixed order).
-__device__ __forceinline__ float warp_scatter32(float (&v)[32], int lane) {
-#pragma unroll
-  for (int h = 16; h >= 1; h >>= 1) {
-    const bool upper = (lane & h) != 0;
-#pragma unroll
-    for (int i = 0; i < h; ++i) {
-      const float send = upper ? v[i] : v[i + h];
-      const float keep = upper ? v[i + h] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
-    }
-  }
-  return v[0];
-}
-
 // The moments of l in [L0, L1) over the thread's points, summed over the warp
 // into sm.mred: at most 7 complex products per point for the powers of delta
 // and conj(delta), then one per moment.
