@@ -76,13 +76,13 @@ def vj_ser_lanes(k: int) -> float:
     return 20.3 + 2 * (k - 2)
 
 
-# The backward's local expansion of a far subhalo about a tile's centre: 15
-# to 36 terms (by the tile's size against its distance) of 40 FP32
-# operations each (7 series terms of the coefficient, 4 real parts of
-# products with the tile's moments, the next power of u) and 30 to set up,
-# per tile and subhalo, whatever the tile's point count; its moments add
-# about 31 operations per point and term, once per tile (not counted).
-VJ_EXP_LANES_PER_TERM = 40.0
+# The backward's local expansion of a far subhalo about a tile's centre: 24
+# terms of 24 FP32 operations (6 series terms each of the coefficient and of
+# its theta_s derivative, their scale, 3 real parts of products with the tile's
+# moments, 4 sums) and 50 to set up, per tile and subhalo, whatever the tile's
+# point count; its moments add about 200 operations per point, once per tile
+# (not counted).
+VJ_EXP_LANES = 24 * 24.0 + 50.0
 # The forward's expansion (grids with rows of 160 points, from 64 subhalos on,
 # 40 + n_sub / 4 of them at least 12.5 half-diagonals away): 24 independent
 # terms of 9 FP32 operations (6 series terms, the scale, 2 sums) and 34 for
@@ -132,11 +132,7 @@ def _degree_shares(p, boxes, counts, degrees, expand=None) -> dict:
             else:
                 hit &= (cn[:, None] <= 2048) & (cn[:, None] >= 64)
             tot["expansion"] += float((hit.sum(1) * cn).sum())
-            # terms of the expansion's order: 15, 21, 28 or 36 for (half-diagonal / |c|) up to 0.01, 0.03, 0.05, 0.08
-            r2 = hd2[:, None] / c2
-            terms = np.where(r2 <= 1e-4, 15, np.where(r2 <= 9e-4, 21, np.where(r2 <= 2.5e-3, 28, 36)))
-            lanes = RT_EXP_LANES if expand == "forward" else VJ_EXP_LANES_PER_TERM * terms + 30.0
-            exp_lanes += float(np.sum(np.where(hit, lanes, 0.0)))
+            exp_lanes += float(hit.sum()) * (RT_EXP_LANES if expand == "forward" else VJ_EXP_LANES)
             left &= ~hit
         for k, r2 in degrees:
             hit = left & (x2 >= r2)

@@ -361,7 +361,23 @@ constexpr ExpBin exp_make_bin() {
   return t;
 }
 
-static __constant__ ExpBin kExpBin = exp_make_bin();
+// The deflection is the gradient of a real potential, so its coefficients
+// c_kl = sum_j q_j (theta_s / |c|)^j C(-j/2, k) C(-(j+2)/2, l) satisfy
+// k c_kl = (l + 1) c_(l+1)(k-1): the terms with m = l + 1 - k >= 0 stand for
+// all. They are taken by m, then k (from 1 for m = 0, whose terms are their own
+// partners), up to k = (kExpN + 1 - m) / 2: 24 of them.
+struct ExpPairBin {
+  float ab[kExpN + 2][kExpN / 2 + 2][8];  // C(-j/2, k) C(-(j+2)/2, k + m - 1) of (m, k, j)
+};
+constexpr ExpPairBin exp_make_pair_bin() {
+  ExpPairBin t{};
+  const ExpBin b = exp_make_bin();
+  for (int m = 0; m <= kExpN + 1; ++m)
+    for (int k = m == 0 ? 1 : 0; k <= (kExpN + 1 - m) / 2; ++k)
+      for (int j = 0; j < 8; ++j) t.ab[m][k][j] = b.a[j][k] * b.b[j][k + m - 1];
+  return t;
+}
+static __constant__ ExpPairBin kExpBin = exp_make_pair_bin();
 
 __device__ __forceinline__ float2 c2mul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
@@ -382,14 +398,9 @@ __device__ __forceinline__ float warp_scatter32(float (&v)[32], int lane) {
   return v[0];
 }
 
-// The truncation order of an expansion for (tile half-diagonal / |c|)^2 =
-// hd2 / r2: 4 up to a ratio of 0.01, 5 up to 0.03, 6 up to 0.05, 7 up to
-// 0.08 (the largest served). Each keeps the truncation below 5e-9 of the
-// sums of absolute terms.
+// (tile half-diagonal / |c|)^2 up to which an expansion serves (0.08^2): the
+// truncation stays below 5e-9 of the sums of absolute terms.
 constexpr float kExpRatio2 = 0.0064f;
-__device__ __forceinline__ int exp_order(float hd2, float r2) {
-  return hd2 <= 1e-4f * r2 ? 4 : hd2 <= 9e-4f * r2 ? 5 : hd2 <= 2.5e-3f * r2 ? 6 : kExpN;
-}
 
 // Converts a raw subhalo record (5 floats) into the prepared form.
 __device__ __forceinline__ SubRec prep_sub(const float* r, int profile) {

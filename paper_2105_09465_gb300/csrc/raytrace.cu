@@ -438,19 +438,6 @@ static_assert(rt_exp_at(kExpN + 1, 0) + 2 == kRtExpFloats, "the last term ends t
 // Place of the coefficient of delta^k conj(delta)^l: by l, then k.
 __device__ constexpr int rt_coef_at(int k, int l) { return l * (2 * kExpN + 3 - l) / 2 + k; }
 
-struct RtExpBin {
-  float ab[kExpN + 2][kExpN / 2 + 2][8];  // C(-j/2, k) C(-(j+2)/2, k + m - 1) of (m, k, j)
-};
-constexpr RtExpBin rt_make_bin() {
-  RtExpBin t{};
-  const ExpBin b = exp_make_bin();
-  for (int m = 0; m <= kExpN + 1; ++m)
-    for (int k = m == 0 ? 1 : 0; k <= (kExpN + 1 - m) / 2; ++k)
-      for (int j = 0; j < 8; ++j) t.ab[m][k][j] = b.a[j][k] * b.b[j][k + m - 1];
-  return t;
-}
-static __constant__ RtExpBin kRtBin = rt_make_bin();
-
 // Adds one subhalo's coefficients (c: the tile's centre less the subhalo's,
 // r2 = |c|^2).
 __device__ __forceinline__ void rt_exp_add(const SubRec& rec, const SubSer& q, float ts, float2 c, float r2, float h,
@@ -474,9 +461,9 @@ __device__ __forceinline__ void rt_exp_add(const SubRec& rec, const SubSer& q, f
     if (m > 0) um = m == 1 ? ub : c2mul(um, ub);
 #pragma unroll
     for (int k = m == 0 ? 1 : 0; k <= (kExpN + 1 - m) / 2; ++k) {
-      float s = k == 0 ? qy[0] * kRtBin.ab[m][k][0] : 0.f;  // C(0, k) = 0 for k > 0
+      float s = k == 0 ? qy[0] * kExpBin.ab[m][k][0] : 0.f;  // C(0, k) = 0 for k > 0
 #pragma unroll
-      for (int j = 2; j < 8; ++j) s = fmaf(qy[j], kRtBin.ab[m][k][j], s);
+      for (int j = 2; j < 8; ++j) s = fmaf(qy[j], kExpBin.ab[m][k][j], s);
       const int at = rt_exp_at(m, k);
       if (m == 0) {
         acc[at] = fmaf(s, rk[k], acc[at]);

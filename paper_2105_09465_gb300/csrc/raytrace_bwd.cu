@@ -35,7 +35,7 @@
 // diagonal within 0.08 of it) and a tile is swept in one phase, the same
 // series is summed by its local expansion about the tile's centre
 // (vj_expand): the tile's gradient moments are formed once (vj_moments), and
-// each such subhalo costs a fixed 36 terms instead of a pass over the points.
+// each such subhalo costs a fixed 24 terms instead of a pass over the points.
 // The others take the far-side closed form per pair and the general form for
 // the rare near pairs. The subhalos of a tile are ordered by that choice,
 // the expansion first and the closed forms last (vj_sort, by the plan or by
@@ -58,6 +58,7 @@ constexpr int kVjWaves = 8;       // large inputs: tiles per resident CTA slot
 constexpr int kVjTilePts = 512;   // ... while every tile keeps at least this many points
 constexpr int kVjExpN = kExpN;     // local expansion: terms delta^k conj(delta)^l with k + l <= kVjExpN
 constexpr int kVjExpTerms = (kVjExpN + 1) * (kVjExpN + 2) / 2;
+constexpr int kVjPairTerms = 24;  // of them with coefficients of their own (lens.cuh)
 constexpr float kVjExpRatio2 = kExpRatio2;  // (tile half-diagonal / distance)^2 up to which it serves (0.08^2)
 constexpr int kVjExpFlag = 16;           // class code: series degree | flag, the expansion serves the tile
 
@@ -76,6 +77,8 @@ struct VjSmem {
   float wbox[kVjWarps][4];        // per-warp bounds of the CTA's points
   float box[4];                   // x_lo, y_lo, x_hi, y_hi of the CTA's points
   float2 wm[3][kVjExpTerms];      // the tile's moments for the local expansion (vj_moments): W, W_x, W_y
+  float4 vm[kVjPairTerms];        // combined over the terms that share a coefficient: W, W_x
+  float2 vmy[kVjPairTerms];       // W_y
   int nexp;                       // subhalos of the tile that the local expansion serves
   float mred[kVjWarps][2 * kVjExpTerms];  // their per-warp sums, in the order of vj_moment_at
 };
@@ -318,11 +321,9 @@ __device__ __forceinline__ int vj_degree_box(const SubRec& h, const SubSer& q, c
 //   sum_i G_i . alpha_i = Re sum_kl M_kl W_kl, with M_kl the coefficients,
 //   and d/dxi_x, d/dxi_y of delta^k conj(delta)^l give the moments
 //   W_x = k W_(k-1,l) + l W_(k,l-1), W_y = i (k W_(k-1,l) - l W_(k,l-1)).
-// The order of the truncation follows the ratio of the tile's half-diagonal
-// to |c|: 4 up to 0.01, 5 up to 0.03, 6 up to 0.05, 7 (kVjExpN) up to 0.08.
-// Each keeps the truncation below 5e-9 of the sums of absolute terms
-// (checked against the analytic FP64 gradients for theta_s from 0.015 to
-// 0.2 arcsec and series degrees 3 to 7).
+// The truncation at order 7 (kVjExpN) stays below 5e-9 of the sums of absolute
+// terms up to a half-diagonal of 0.08 |c| (checked against the analytic FP64
+// gradients for theta_s from 0.015 to 0.2 arcsec).
 
 // Term index of delta^k conj(delta)^l: by total order s = k + l, then k.
 __device__ __forceinline__ int vj_term(int k, int l) { return (k + l) * (k + l + 1) / 2 + k; }
@@ -341,6 +342,16 @@ __device__ __forceinline__ int vj_class(const SubRec& h, const SubSer& q, const 
 // Position of the moment W_kl in the order in which the warps sum them: by l,
 // then k.
 __device__ constexpr int vj_moment_at(int k, int l) { return l * (2 * kVjExpN + 3 - l) / 2 + k; }
+
+// Place of the term (m, k) among those with coefficients of their own: by m,
+// then k; m = 0 starts at k = 1, so its "k = 0" is place -1.
+__device__ constexpr int vj_pair_at(int m, int k) {
+  if (m == 0) return k - 1;
+  int at = (kExpN + 1) / 2;
+  for (int i = 1; i < m; ++i) at += (kExpN + 1 - i) / 2 + 1;
+  return at + k;
+}
+static_assert(vj_pair_at(kExpN + 1, 0) + 1 == kVjPairTerms, "the last term ends them");
 
 // The moments of l in [L0, L1) over the thread's points, summed over the warp
 // into sm.mred: at most 7 complex products per point for the powers of delta
@@ -427,56 +438,81 @@ __device__ __forceinline__ void vj_moments(VjSmem& sm, int cnt, float2 cen) {
     sm.wm[2][t] = make_float2(-fmaf(fk, wa.y, -fl * wb.y), fmaf(fk, wa.x, -fl * wb.x));
   }
   __syncthreads();
+  // The coefficient of (l + 1, k - 1) is k / (l + 1) times the conjugate of
+  // that of (k, l): its moment joins the latter's, conjugated.
+  if (t < kVjPairTerms) {
+    int m = 0;
+    while (m <= kVjExpN && vj_pair_at(m + 1, 0) <= t) ++m;
+    const int k = t - vj_pair_at(m, 0), l = k + m - 1;
+    const float f = m > 0 && k > 0 ? (float)k / (float)(l + 1) : 0.f;
+    float2 v[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      v[i] = sm.wm[i][vj_term(k, l)];
+      if (f > 0.f) {
+        const float2 p = sm.wm[i][vj_term(l + 1, k - 1)];
+        v[i] = make_float2(fmaf(f, p.x, v[i].x), fmaf(-f, p.y, v[i].y));
+      }
+    }
+    sm.vm[t] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+    sm.vmy[t] = v[2];
+  }
+  __syncthreads();
 }
 
 // The tile's four subhalo sums by the local expansion: dL/d(x_h, y_h,
-// kappa_s, theta_s) of one tNFW subhalo (K: its series degree for the tile),
-// from the tile's moments about cen. The term loops stay rolled: unrolled
-// inside the sweep's kernel they spill, and a separate (not inlined) unrolled
-// function measured slower.
-__device__ __forceinline__ float4 vj_expand(const SubRec& rec, const SubSer& q, float kappa, float ts, int K,
-                                            float2 cen, float hd2, const VjSmem& sm) {
+// kappa_s, theta_s) of one tNFW subhalo, from the tile's combined moments
+// (vj_moments): 24 terms of 24 FP32 operations (the six series terms of the
+// coefficient and of its theta_s derivative, their scale, three real parts of
+// products with the moments, four sums), all unrolled. With the 36 plain
+// moments, 40 operations each in rolled loops of 15 to 36 terms, the VJP took
+// 1.23 ms at 2.56M points x 2000 subhalos, now 0.90.
+__device__ __forceinline__ float4 vj_expand(const SubRec& rec, const SubSer& q, float kappa, float ts, float2 cen,
+                                            const VjSmem& sm) {
   const float2 c = make_float2(cen.x - rec.xh, cen.y - rec.yh);
-  const float r2 = fmaf(c.x, c.x, c.y * c.y), ir2 = 1.0f / r2;
-  // the truncation order for (half-diagonal / |c|)^2 = hd2 / r2
-  const int nmax = exp_order(hd2, r2);
-  const float2 u = make_float2(c.x * ir2, -c.y * ir2), ub = make_float2(u.x, -u.y);
+  const float ir2 = 1.0f / fmaf(c.x, c.x, c.y * c.y);
+  const float2 ub = make_float2(c.x * ir2, c.y * ir2);  // conj(u)
   const float yc = ts * sqrtf(ir2);
-  float qy[8];
+  float qy[8], qt[8];
   float yj = 1.f;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    qy[j] = (j == 1 || j > K) ? 0.f : q.q[j] * yj;
+    qy[j] = q.q[j] * yj;  // q1 = 0
+    qt[j] = (float)(j + 2) * qy[j];
     yj *= yc;
   }
-  // Q = u^k conj(u)^(l+1) for the terms of total order s = k + l: from
-  // conj(u)^(s+1) at k = 0, each step in k times u / conj(u) = conj(c)^2 / |c|^2
-  const float2 rot = make_float2((c.x * c.x - c.y * c.y) * ir2, -2.0f * c.x * c.y * ir2);
-  float2 us = ub;  // conj(u)^(s+1)
-  float L = 0.f, Lt = 0.f, X = 0.f, Y = 0.f;
-#pragma unroll 1
-  for (int s = 0; s <= nmax; ++s) {
-    float2 Q = us;
-#pragma unroll 1
-    for (int k = 0; k <= s; ++k) {
-      const int l = s - k, m = s * (s + 1) / 2 + k;
-      float ckl = 0.f, ctl = 0.f;
+  float rk[kExpN / 2 + 2];  // |u|^2k
+  rk[0] = 1.f;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (j == 1) continue;
-        const float w = qy[j] * (kExpBin.a[j][k] * kExpBin.b[j][l]);
-        ckl += w;
-        ctl = fmaf(w, (float)(j + 2), ctl);
+  for (int k = 1; k < kExpN / 2 + 2; ++k) rk[k] = rk[k - 1] * ir2;
+  float2 um = make_float2(1.f, 0.f);  // conj(u)^m
+  float L = 0.f, Lt = 0.f, X = 0.f, Y = 0.f;
+#pragma unroll
+  for (int m = 0; m <= kExpN + 1; ++m) {
+    if (m > 0) um = m == 1 ? ub : c2mul(um, ub);
+#pragma unroll
+    for (int k = m == 0 ? 1 : 0; k <= (kExpN + 1 - m) / 2; ++k) {
+      float s = k == 0 ? qy[0] * kExpBin.ab[m][k][0] : 0.f;  // C(0, k) = 0 for k > 0
+      float t = k == 0 ? qt[0] * kExpBin.ab[m][k][0] : 0.f;
+#pragma unroll
+      for (int j = 2; j < 8; ++j) {
+        s = fmaf(qy[j], kExpBin.ab[m][k][j], s);
+        t = fmaf(qt[j], kExpBin.ab[m][k][j], t);
       }
-      const float2 W = sm.wm[0][m], Wx = sm.wm[1][m], Wy = sm.wm[2][m];
-      const float rw = fmaf(Q.x, W.x, -Q.y * W.y);
-      L = fmaf(ckl, rw, L);
-      Lt = fmaf(ctl, rw, Lt);
-      X = fmaf(ckl, fmaf(Q.x, Wx.x, -Q.y * Wx.y), X);
-      Y = fmaf(ckl, fmaf(Q.x, Wy.x, -Q.y * Wy.y), Y);
-      Q = c2mul(Q, rot);
+      if (k > 0) {
+        s *= rk[k];
+        t *= rk[k];
+      }
+      const float4 W = sm.vm[vj_pair_at(m, k)];   // W, W_x
+      const float2 V = sm.vmy[vj_pair_at(m, k)];  // W_y
+      const float rw = m == 0 ? W.x : fmaf(um.x, W.x, -um.y * W.y);
+      const float rx = m == 0 ? W.z : fmaf(um.x, W.z, -um.y * W.w);
+      const float ry = m == 0 ? V.x : fmaf(um.x, V.x, -um.y * V.y);
+      L = fmaf(s, rw, L);
+      Lt = fmaf(t, rw, Lt);
+      X = fmaf(s, rx, X);
+      Y = fmaf(s, ry, Y);
     }
-    us = c2mul(us, ub);
   }
   const float sc = rec.A * ts * ts;
   return make_float4(sc * X, sc * Y, -sc * L / kappa, -sc * Lt / ts);
@@ -557,10 +593,10 @@ __device__ __forceinline__ int vj_cls_key(int c) { return (c & kVjExpFlag) ? kVj
 
 // FP32 lanes per point of a subhalo's sums for a tile of npts points, by its
 // class (vj_class): the series of degree K, the closed forms (0), or the
-// local expansion (up to about 1,600 lanes per tile): the weight of a tile's
+// local expansion (about 650 lanes per tile): the weight of a tile's
 // work.
 __device__ __forceinline__ float vj_cost(int cls, int npts) {
-  if (cls & kVjExpFlag) return 1600.0f / (float)max(npts, 1);
+  if (cls & kVjExpFlag) return 650.0f / (float)max(npts, 1);
   return cls ? 20.3f + 2.0f * (float)(cls - 2) : 50.3f;
 }
 
@@ -654,7 +690,7 @@ __device__ __forceinline__ int vj_pick_phases(int nd, int np) {
 // one phase count per launch, 200 subhalos ran in 3 phases and every pair
 // directly (249 us at 640k points).
 __device__ __forceinline__ void vj_tile_sums(const float* __restrict__ sub, int n_sub, int nexp,
-                                             const unsigned short* __restrict__ ord, int cnt, float2 cen, float hd2,
+                                             const unsigned short* __restrict__ ord, int cnt, float2 cen,
                                              float* __restrict__ sub_part, int64_t blk, int64_t nblk, VjSmem& sm) {
   constexpr int PR = LR_PROFILE_TNFW;
   const int tid = threadIdx.x;
@@ -663,8 +699,7 @@ __device__ __forceinline__ void vj_tile_sums(const float* __restrict__ sub, int 
     const float* rr = sub + 5 * (int64_t)h;
     const SubRec rec = prep_sub(rr, PR);
     const SubSer q = prep_series(rec, PR);
-    const int deg = vj_degree_box(rec, q, sm.box);
-    const float4 x = vj_expand(rec, q, __ldg(rr + 2), __ldg(rr + 3), deg, cen, hd2, sm);
+    const float4 x = vj_expand(rec, q, __ldg(rr + 2), __ldg(rr + 3), cen, sm);
     float* o = sub_part + (int64_t)h * 4 * nblk + blk;  // [value][CTA]
     o[0] = x.x;
     o[nblk] = x.y;
@@ -793,10 +828,9 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
       vj_stage(L, LG, g, xi, mp, grid, dbeta, p0, cnt, true, la, sm);
       vj_lens_out(la, lens_part + tile * 7, sm);  // its barrier also ends the staging
       const float2 cen = make_float2(0.5f * (sm.box[0] + sm.box[2]), 0.5f * (sm.box[1] + sm.box[3]));
-      const float hx = 0.5f * (sm.box[2] - sm.box[0]), hy = 0.5f * (sm.box[3] - sm.box[1]);
       const int nexp = plan.nexp ? plan.nexp[tile] : sm.nexp;
       if (nexp > 0) vj_moments(sm, cnt, cen);  // uniform over the CTA
-      vj_tile_sums(sub, n_sub, nexp, ord, cnt, cen, fmaf(hx, hx, hy * hy), sub_part, blk, nblk, sm);
+      vj_tile_sums(sub, n_sub, nexp, ord, cnt, cen, sub_part, blk, nblk, sm);
       return;
     }
   }
