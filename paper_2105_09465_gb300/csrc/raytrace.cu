@@ -22,6 +22,13 @@
 namespace lr {
 
 constexpr int kRtThreads = 128;
+// Launches that fit the GPU at this many CTAs of 256 threads per SM take one
+// point per thread: twice the warps over the same points, staged records and
+// order of the sums (the same bits). Fewer CTAs of 128 threads leave the SMs'
+// latency uncovered: a list of 20k points x 500 subhalos 73 -> 50 us, 105k (a
+// 412-CTA wave) 89 -> 77 us, 64 x 64 at 2 x 2 x 500 53 -> 40 us; past one wave
+// the two are level (130k points: 95 us).
+constexpr int kRtSmallPerSm = 3;
 constexpr int kRtPts = 2;                        // points per thread
 constexpr int kRtPoints = kRtThreads * kRtPts;   // points per CTA
 constexpr int kRtTile = 16;  // grid input: a CTA takes a kRtTile x kRtTile tile of pixels
@@ -63,7 +70,7 @@ struct RtSmem {
   int order[kSubChunk];  // staged position -> subhalo of the chunk
   unsigned char deg[kSubChunk];  // series degree for the CTA's points of each subhalo of the chunk (0: none)
   int ndeg[5];                   // staged subhalos served by the series to y^3, y^4, y^5, y^7, y^9
-  int wcnt[kRtThreads / 32][6];  // per warp's quarter of the chunk: subhalos by degree class
+  int wcnt[kRtPoints / 32][6];   // per warp's part of the chunk: subhalos by degree class
   float box[4];          // the CTA's points: x_lo, y_lo, x_hi, y_hi
   int nfar;
   uint64_t bar;
@@ -125,11 +132,12 @@ __device__ __forceinline__ int rt_degree(float x2min, float m) {
 // (rt_degree, fewest terms first), each degree in index order; sm.ndeg
 // counts them by degree and sm.nfar in all. Returns false (all threads) if
 // the bulk-copy wait timed out.
+template <int NT>
 __device__ __forceinline__ bool stage_rt(const float* __restrict__ sub, int h0, int cnt, int profile, RtSmem& sm,
                                          uint32_t& phase, bool bulk_ok, int* fault,
                                          const unsigned short* list = nullptr) {
   if (list) {
-    for (int w = threadIdx.x; w < 5 * cnt; w += kRtThreads) {
+    for (int w = threadIdx.x; w < 5 * cnt; w += NT) {
       const int t = w / 5;
       sm.raw[w] = __ldg(sub + 5 * (int64_t)list[h0 + t] + (w - 5 * t));
     }
@@ -150,7 +158,7 @@ __device__ __forceinline__ bool stage_rt(const float* __restrict__ sub, int h0, 
   // w takes the chunk's positions [w q, (w + 1) q), q = kSubChunk / warps:
   // it counts its subhalos per class, then scatters them after the classes
   // before theirs and the warps before it.
-  constexpr int kW = kRtThreads / 32, kQ = kSubChunk / kW;
+  constexpr int kW = NT / 32, kQ = kSubChunk / kW;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll 1
   for (int pass = 0; pass < 6; ++pass) {
@@ -227,10 +235,10 @@ __device__ __forceinline__ void rt_coeffs(const float4* hot, float2 (&q)[kSerTer
 // Staged pairs kp and kp + 1 (four subhalos, all far from every point of the
 // CTA) by the series to y^K: four independent chains per thread, added in
 // order.
-template <int K>
-__device__ __forceinline__ void rt_far4(const RtSmem& sm, int kp, const float2 (&X)[kRtPts],
-                                        const float2 (&Y)[kRtPts], float2 (&ax)[kRtPts], float2 (&ay)[kRtPts]) {
-  float2 m[2][kRtPts], dxs[2][kRtPts], dys[2][kRtPts];
+template <int K, int NP>
+__device__ __forceinline__ void rt_far4(const RtSmem& sm, int kp, const float2 (&X)[NP],
+                                        const float2 (&Y)[NP], float2 (&ax)[NP], float2 (&ay)[NP]) {
+  float2 m[2][NP], dxs[2][NP], dys[2][NP];
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const float4* hot = sm.hot[kp + u];
@@ -238,7 +246,7 @@ __device__ __forceinline__ void rt_far4(const RtSmem& sm, int kp, const float2 (
     float2 q[kSerTerms];
     rt_coeffs<K>(hot, q);
 #pragma unroll
-    for (int j = 0; j < kRtPts; ++j) {
+    for (int j = 0; j < NP; ++j) {
       dxs[u][j] = sub2(X[j], make_float2(w0.x, w0.y));
       dys[u][j] = sub2(Y[j], make_float2(w0.z, w0.w));
       const float2 R2 = __ffma2_rn(dxs[u][j], dxs[u][j], __fmul2_rn(dys[u][j], dys[u][j]));
@@ -248,7 +256,7 @@ __device__ __forceinline__ void rt_far4(const RtSmem& sm, int kp, const float2 (
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
 #pragma unroll
-    for (int j = 0; j < kRtPts; ++j) {
+    for (int j = 0; j < NP; ++j) {
       ax[j] = __ffma2_rn(m[u][j], dxs[u][j], ax[j]);
       ay[j] = __ffma2_rn(m[u][j], dys[u][j], ay[j]);
     }
@@ -257,15 +265,15 @@ __device__ __forceinline__ void rt_far4(const RtSmem& sm, int kp, const float2 (
 
 // Staged pair kp (both subhalos far from every point of the CTA) by the
 // series to y^K.
-template <int K>
-__device__ __forceinline__ void rt_far2(const RtSmem& sm, int kp, const float2 (&X)[kRtPts],
-                                        const float2 (&Y)[kRtPts], float2 (&ax)[kRtPts], float2 (&ay)[kRtPts]) {
+template <int K, int NP>
+__device__ __forceinline__ void rt_far2(const RtSmem& sm, int kp, const float2 (&X)[NP],
+                                        const float2 (&Y)[NP], float2 (&ax)[NP], float2 (&ay)[NP]) {
   const float4* hot = sm.hot[kp];
   const float4 w0 = hot[0], w1 = hot[1], w2 = hot[2];
   float2 q[kSerTerms];
   rt_coeffs<K>(hot, q);
 #pragma unroll
-  for (int j = 0; j < kRtPts; ++j) {
+  for (int j = 0; j < NP; ++j) {
     const float2 dx = sub2(X[j], make_float2(w0.x, w0.y)), dy = sub2(Y[j], make_float2(w0.z, w0.w));
     const float2 R2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
     const float2 m = rt_series2<K>(hi2(w1), hi2(w2), q, __fmul2_rn(R2, lo2(w1)));
@@ -274,10 +282,11 @@ __device__ __forceinline__ void rt_far2(const RtSmem& sm, int kp, const float2 (
   }
 }
 
-__device__ __forceinline__ void fold(const float2 (&ax)[kRtPts], const float2 (&ay)[kRtPts], float (&sx)[kRtPts],
-                                     float (&cx)[kRtPts], float (&sy)[kRtPts], float (&cy)[kRtPts]) {
+template <int NP>
+__device__ __forceinline__ void fold(const float2 (&ax)[NP], const float2 (&ay)[NP], float (&sx)[NP],
+                                     float (&cx)[NP], float (&sy)[NP], float (&cy)[NP]) {
 #pragma unroll
-  for (int j = 0; j < kRtPts; ++j) {
+  for (int j = 0; j < NP; ++j) {
     kahan(sx[j], cx[j], __fadd_rn(ax[j].x, ax[j].y));
     kahan(sy[j], cy[j], __fadd_rn(ay[j].x, ay[j].y));
   }
@@ -286,15 +295,15 @@ __device__ __forceinline__ void fold(const float2 (&ax)[kRtPts], const float2 (&
 // Staged pairs [ka, kb), every subhalo of them far from the whole CTA and
 // served by the series to y^K (a pair that straddles two degrees takes the
 // larger): two pairs per step, kRtFoldPairs pairs summed plainly per fold.
-template <int K>
-__device__ __forceinline__ void rt_far_run(const RtSmem& sm, int ka, int kb, const float2 (&X)[kRtPts],
-                                           const float2 (&Y)[kRtPts], float (&sx)[kRtPts], float (&cx)[kRtPts],
-                                           float (&sy)[kRtPts], float (&cy)[kRtPts]) {
+template <int K, int NP>
+__device__ __forceinline__ void rt_far_run(const RtSmem& sm, int ka, int kb, const float2 (&X)[NP],
+                                           const float2 (&Y)[NP], float (&sx)[NP], float (&cx)[NP],
+                                           float (&sy)[NP], float (&cy)[NP]) {
   for (int k = ka; k < kb;) {
     const int kend = min(kb, k + kRtFoldPairs);
-    float2 ax[kRtPts], ay[kRtPts];
+    float2 ax[NP], ay[NP];
 #pragma unroll
-    for (int j = 0; j < kRtPts; ++j) ax[j] = ay[j] = f2(0.f);
+    for (int j = 0; j < NP; ++j) ax[j] = ay[j] = f2(0.f);
     for (; k + 1 < kend; k += 2) rt_far4<K>(sm, k, X, Y, ax, ay);
     if (k < kend) {
       rt_far2<K>(sm, k, X, Y, ax, ay);
@@ -304,20 +313,20 @@ __device__ __forceinline__ void rt_far_run(const RtSmem& sm, int ka, int kb, con
   }
 }
 
-// Deflection of the staged subhalos at the thread's kRtPts points (x[j],
+// Deflection of the staged subhalos at the thread's NP points (x[j],
 // y[j]), added to the Kahan sums (sx, cx), (sy, cy) of each point. The
 // subhalos far from the whole CTA come first, in runs of one series degree
 // (rt_far_run); the rest in blocks of kRtFold subhalos. Each block is summed
 // plainly in two packed lanes and folded into the Kahan sums; the order is
 // fixed, so a point's bits do not depend on the other points of its thread.
 // Each staged record is read once for all of the thread's points.
-template <int PROFILE>
-__device__ __forceinline__ void add_subs(const RtSmem& sm, int cnt, const float (&x)[kRtPts],
-                                         const float (&y)[kRtPts], float (&sx)[kRtPts], float (&cx)[kRtPts],
-                                         float (&sy)[kRtPts], float (&cy)[kRtPts]) {
-  float2 X[kRtPts], Y[kRtPts];
+template <int PROFILE, int NP>
+__device__ __forceinline__ void add_subs(const RtSmem& sm, int cnt, const float (&x)[NP],
+                                         const float (&y)[NP], float (&sx)[NP], float (&cx)[NP],
+                                         float (&sy)[NP], float (&cy)[NP]) {
+  float2 X[NP], Y[NP];
 #pragma unroll
-  for (int j = 0; j < kRtPts; ++j) {
+  for (int j = 0; j < NP; ++j) {
     X[j] = f2(x[j]);
     Y[j] = f2(y[j]);
   }
@@ -343,9 +352,9 @@ __device__ __forceinline__ void add_subs(const RtSmem& sm, int cnt, const float 
   }
   for (int t0 = tfar; t0 < cnt; t0 += kRtFold) {
     const int t1 = min(cnt, t0 + kRtFold);
-    float2 ax[kRtPts], ay[kRtPts];
+    float2 ax[NP], ay[NP];
 #pragma unroll
-    for (int j = 0; j < kRtPts; ++j) ax[j] = ay[j] = f2(0.f);
+    for (int j = 0; j < NP; ++j) ax[j] = ay[j] = f2(0.f);
     int t = t0;
     if (PROFILE == LR_PROFILE_TNFW) {
       for (; t + 1 < t1; t += 2) {
@@ -359,7 +368,7 @@ __device__ __forceinline__ void add_subs(const RtSmem& sm, int cnt, const float 
           // gives the same bits for far pairs)
           const SubRec2 H = rec_from(hot, sm.cold[t >> 1]);
 #pragma unroll
-          for (int j = 0; j < kRtPts; ++j) {
+          for (int j = 0; j < NP; ++j) {
             const float2 dx = sub2(X[j], make_float2(w0.x, w0.y)), dy = sub2(Y[j], make_float2(w0.z, w0.w));
             const float2 R2 = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
             const float2 x2 = __fmul2_rn(R2, lo2(w1));
@@ -386,7 +395,7 @@ __device__ __forceinline__ void add_subs(const RtSmem& sm, int cnt, const float 
       const float4* hot = sm.hot[t >> 1];
       const SubRec h = sub_lane(rec_from(hot, sm.cold[t >> 1]), t & 1);
 #pragma unroll
-      for (int j = 0; j < kRtPts; ++j) {
+      for (int j = 0; j < NP; ++j) {
         const float dx = __fsub_rn(x[j], h.xh), dy = __fsub_rn(y[j], h.yh);
         const float R2 = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
         const float m = (PROFILE == LR_PROFILE_POINT_MASS) ? pointmass_m(h, R2)
@@ -401,7 +410,7 @@ __device__ __forceinline__ void add_subs(const RtSmem& sm, int cnt, const float 
       }
     }
 #pragma unroll
-    for (int j = 0; j < kRtPts; ++j) {
+    for (int j = 0; j < NP; ++j) {
       kahan(sx[j], cx[j], __fadd_rn(ax[j].x, ax[j].y));
       kahan(sy[j], cy[j], __fadd_rn(ay[j].x, ay[j].y));
     }
@@ -608,20 +617,22 @@ __host__ __device__ __forceinline__ bool rt_may_expand(bool explicit_points, con
 }
 
 // EXP: grid tiles may take the local expansion.
-template <int PROFILE, bool EXP>
+template <int PROFILE, bool EXP, int NP>
 __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev& g, const float2* __restrict__ xi,
                                               int64_t n, const float* __restrict__ sub, int n_sub, int bulk_ok,
                                               float2* __restrict__ beta, float2* __restrict__ alpha_out, int* fault,
                                               int64_t blk, RtSmem& sm) {
+  constexpr int NT = kRtPoints / NP;  // threads of the CTA
+  static_assert(!EXP || NP == kRtPts, "the expansion is summed by kRtThreads threads");
   // explicit points: kRtPoints consecutive ones; grid: a 2-D tile, so that
   // the CTA's points are compact (padding points repeat an edge point).
-  // Thread t takes the CTA's points t + j kRtThreads (j < kRtPts).
-  int64_t i[kRtPts];
-  bool valid[kRtPts];
-  float px[kRtPts], py[kRtPts], ax[kRtPts], ay[kRtPts];
+  // Thread t takes the CTA's points t + j NT (j < NP).
+  int64_t i[NP];
+  bool valid[NP];
+  float px[NP], py[NP], ax[NP], ay[NP];
 #pragma unroll
-  for (int j = 0; j < kRtPts; ++j) {
-    const int w = (int)threadIdx.x + j * kRtThreads;
+  for (int j = 0; j < NP; ++j) {
+    const int w = (int)threadIdx.x + j * NT;
     int64_t ii;
     if (xi) {
       i[j] = blk * kRtPoints + w;
@@ -648,7 +659,7 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
     // the box of the CTA's points (the padding points repeat an edge point)
     float b0 = px[0], b1 = py[0], b2 = px[0], b3 = py[0];
 #pragma unroll
-    for (int j = 1; j < kRtPts; ++j) {
+    for (int j = 1; j < NP; ++j) {
       b0 = fminf(b0, px[j]);
       b1 = fminf(b1, py[j]);
       b2 = fmaxf(b2, px[j]);
@@ -672,7 +683,7 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
     __syncthreads();
     if (threadIdx.x == 0) {
       float c0 = sm.raw[0], c1 = sm.raw[1], c2 = sm.raw[2], c3 = sm.raw[3];
-      for (int w = 1; w < kRtThreads / 32; ++w) {
+      for (int w = 1; w < NT / 32; ++w) {
         c0 = fminf(c0, sm.raw[4 * w]);
         c1 = fminf(c1, sm.raw[4 * w + 1]);
         c2 = fmaxf(c2, sm.raw[4 * w + 2]);
@@ -685,9 +696,9 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
     }
     __syncthreads();
     uint32_t phase = 0;
-    float sx[kRtPts], cx[kRtPts], sy[kRtPts], cy[kRtPts];
+    float sx[NP], cx[NP], sy[NP], cy[NP];
 #pragma unroll
-    for (int j = 0; j < kRtPts; ++j) sx[j] = cx[j] = sy[j] = cy[j] = 0.f;
+    for (int j = 0; j < NP; ++j) sx[j] = cx[j] = sy[j] = cy[j] = 0.f;
     bool expand = false;
     if constexpr (EXP && PROFILE == LR_PROFILE_TNFW) {
       const float2 cen = make_float2(0.5f * (sm.box[0] + sm.box[2]), 0.5f * (sm.box[1] + sm.box[3]));
@@ -700,8 +711,8 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
           const int nl = rt_expand_window(win, min(kRtWin, n_sub - w0), w0 > 0, cen, hd2, sm);
           for (int h0 = 0; h0 < nl; h0 += kSubChunk) {
             const int cnt = min(kSubChunk, nl - h0);
-            stage_rt(win, h0, cnt, PROFILE, sm, phase, false, fault, sm.list);
-            add_subs<PROFILE>(sm, cnt, px, py, sx, cx, sy, cy);
+            stage_rt<NT>(win, h0, cnt, PROFILE, sm, phase, false, fault, sm.list);
+            add_subs<PROFILE, NP>(sm, cnt, px, py, sx, cx, sy, cy);
             __syncthreads();
           }
         }
@@ -710,18 +721,18 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
     }
     for (int h0 = 0; h0 < n_sub && !expand; h0 += kSubChunk) {
       const int cnt = min(kSubChunk, n_sub - h0);
-      if (!stage_rt(sub, h0, cnt, PROFILE, sm, phase, bulk_ok != 0, fault)) return;
-      add_subs<PROFILE>(sm, cnt, px, py, sx, cx, sy, cy);
+      if (!stage_rt<NT>(sub, h0, cnt, PROFILE, sm, phase, bulk_ok != 0, fault)) return;
+      add_subs<PROFILE, NP>(sm, cnt, px, py, sx, cx, sy, cy);
       __syncthreads();
     }
 #pragma unroll
-    for (int j = 0; j < kRtPts; ++j) {
+    for (int j = 0; j < NP; ++j) {
       ax[j] += sx[j] - cx[j];
       ay[j] += sy[j] - cy[j];
     }
   }
 #pragma unroll
-  for (int j = 0; j < kRtPts; ++j) {
+  for (int j = 0; j < NP; ++j) {
     if (valid[j]) {
       beta[i[j]] = make_float2(px[j] - ax[j], py[j] - ay[j]);
       if (alpha_out) alpha_out[i[j]] = make_float2(ax[j], ay[j]);
@@ -729,27 +740,29 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
   }
 }
 
-template <int PROFILE, bool EXP>
-__global__ void __launch_bounds__(kRtThreads, 5) raytrace_kernel(const __grid_constant__ LensConst L, GridDev g,
+constexpr int rt_min_blocks(int np) { return np == kRtPts ? 5 : kRtSmallPerSm; }
+
+template <int PROFILE, bool EXP, int NP>
+__global__ void __launch_bounds__(kRtPoints / NP, rt_min_blocks(NP)) raytrace_kernel(const __grid_constant__ LensConst L, GridDev g,
                                                               const float2* __restrict__ xi, int64_t n,
                                                               const float* __restrict__ sub, int n_sub, int bulk_ok,
                                                               float2* __restrict__ beta,
                                                               float2* __restrict__ alpha_out, int* fault) {
   __shared__ __align__(16) RtSmem sm;
-  raytrace_body<PROFILE, EXP>(L, g, xi, n, sub, n_sub, bulk_ok, beta, alpha_out, fault, blockIdx.x, sm);
+  raytrace_body<PROFILE, EXP, NP>(L, g, xi, n, sub, n_sub, bulk_ok, beta, alpha_out, fault, blockIdx.x, sm);
 }
 
 // The same with the lens read from a device record (lr_lens_prepare); an
 // invalid record is reported in the fault word.
-template <int PROFILE, bool EXP>
-__global__ void __launch_bounds__(kRtThreads, 5) raytrace_rec_kernel(const LensRecord* __restrict__ rec, GridDev g,
+template <int PROFILE, bool EXP, int NP>
+__global__ void __launch_bounds__(kRtPoints / NP, rt_min_blocks(NP)) raytrace_rec_kernel(const LensRecord* __restrict__ rec, GridDev g,
                                                                   const float2* __restrict__ xi, int64_t n,
                                                                   const float* __restrict__ sub, int n_sub,
                                                                   int bulk_ok, float2* __restrict__ beta,
                                                                   float2* __restrict__ alpha_out, int* fault) {
   __shared__ __align__(16) RtSmem sm;
   if (rec->status != 0 && blockIdx.x == 0 && threadIdx.x == 0) atomicExch(fault, kFaultBadLens);
-  raytrace_body<PROFILE, EXP>(rec->L, g, xi, n, sub, n_sub, bulk_ok, beta, alpha_out, fault, blockIdx.x, sm);
+  raytrace_body<PROFILE, EXP, NP>(rec->L, g, xi, n, sub, n_sub, bulk_ok, beta, alpha_out, fault, blockIdx.x, sm);
 }
 
 __global__ void lens_prepare_kernel(const float* __restrict__ theta7, float gamma, LensRecord* __restrict__ rec) {
@@ -778,13 +791,13 @@ __global__ void __launch_bounds__(kRtThreads, 5) raytrace_batched_kernel(const _
   const RtP& P = B.p[k];
   const int64_t blk = blockIdx.x - B.start[k];
   if (P.profile == LR_PROFILE_POINT_MASS)
-    raytrace_body<LR_PROFILE_POINT_MASS, false>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault,
+    raytrace_body<LR_PROFILE_POINT_MASS, false, kRtPts>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault,
                                          blk, sm);
   else if (rt_may_expand(P.xi != nullptr, P.g, P.profile, P.n_sub))
-    raytrace_body<LR_PROFILE_TNFW, true>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault,
+    raytrace_body<LR_PROFILE_TNFW, true, kRtPts>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault,
                                          blk, sm);
   else
-    raytrace_body<LR_PROFILE_TNFW, false>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault,
+    raytrace_body<LR_PROFILE_TNFW, false, kRtPts>(P.L, P.g, P.xi, P.n, P.sub, P.n_sub, P.bulk_ok, P.beta, P.alpha, fault,
                                           blk, sm);
 }
 
@@ -888,14 +901,25 @@ lr_status launch_raytrace(const lr_points* p, float2* beta, float2* alpha, cudaS
   const int ns = p->n_sub;
   ktimer_begin(LR_KT_RAYTRACE, s);
   const bool pm = p->profile == LR_PROFILE_POINT_MASS, ex = rt_may_expand(p->xy != nullptr, g, p->profile, ns);
+  constexpr int PM = LR_PROFILE_POINT_MASS, TN = LR_PROFILE_TNFW;
+  bool small = false;
+  if (!ex && ns > 0) {
+    int occ = 0, n_sm = 0;
+    LR_CHECK(kernel_occupancy(raytrace_kernel<TN, false, 1>, kRtPoints, &occ, &n_sm));
+    small = blocks <= (unsigned)(occ * n_sm);
+  }
   if (rec) {
-    const auto k = pm ? raytrace_rec_kernel<LR_PROFILE_POINT_MASS, false>
-                   : ex ? raytrace_rec_kernel<LR_PROFILE_TNFW, true> : raytrace_rec_kernel<LR_PROFILE_TNFW, false>;
-    k<<<blocks, kRtThreads, 0, s>>>(rec, g, xi, p->n, p->sub, ns, bulk_ok, beta, alpha, fault);
+    const auto k = small ? (pm ? raytrace_rec_kernel<PM, false, 1> : raytrace_rec_kernel<TN, false, 1>)
+                   : pm  ? raytrace_rec_kernel<PM, false, kRtPts>
+                   : ex  ? raytrace_rec_kernel<TN, true, kRtPts>
+                         : raytrace_rec_kernel<TN, false, kRtPts>;
+    k<<<blocks, small ? kRtPoints : kRtThreads, 0, s>>>(rec, g, xi, p->n, p->sub, ns, bulk_ok, beta, alpha, fault);
   } else {
-    const auto k = pm ? raytrace_kernel<LR_PROFILE_POINT_MASS, false>
-                   : ex ? raytrace_kernel<LR_PROFILE_TNFW, true> : raytrace_kernel<LR_PROFILE_TNFW, false>;
-    k<<<blocks, kRtThreads, 0, s>>>(L, g, xi, p->n, p->sub, ns, bulk_ok, beta, alpha, fault);
+    const auto k = small ? (pm ? raytrace_kernel<PM, false, 1> : raytrace_kernel<TN, false, 1>)
+                   : pm  ? raytrace_kernel<PM, false, kRtPts>
+                   : ex  ? raytrace_kernel<TN, true, kRtPts>
+                         : raytrace_kernel<TN, false, kRtPts>;
+    k<<<blocks, small ? kRtPoints : kRtThreads, 0, s>>>(L, g, xi, p->n, p->sub, ns, bulk_ok, beta, alpha, fault);
   }
   LR_CHECK_CUDA(cudaGetLastError());
   ktimer_end(LR_KT_RAYTRACE, s);
