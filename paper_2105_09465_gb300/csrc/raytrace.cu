@@ -1,6 +1,7 @@
 // Pixel-grid generation and the lens ray-trace beta = xi - alpha(xi).
 //
-// Two image-plane points per thread; a CTA takes a 16 x 16 tile of a pixel
+// Two image-plane points per thread (one where a launch fits one wave of
+// larger CTAs); a CTA takes a 16 x 16 tile of a pixel
 // grid (or 256 consecutive explicit points). The SPLE and shear terms are
 // evaluated in registers from per-lens constants passed as a kernel
 // parameter; the subhalo records are staged into shared memory in chunks by a
