@@ -21,8 +21,9 @@
 // once the points are staged, a thread sweeps without block barriers. Points
 // are staged as packed pairs (2k, 2k + 1), so a slot evaluates two points per
 // step in f32x2 arithmetic; slot (h, r) takes the point pairs k = r (mod P).
-// P is chosen on the host so that n_sub * P fills the CTA's threads nearly
-// evenly. At the end the CTA adds each subhalo's P slot sums in phase order.
+// A tile in one staged chunk chooses its own P for the subhalos it sums directly
+// (vj_pick_phases); the others take the launch's P (vjp_phases), and at the end
+// the CTA adds each subhalo's P slot sums in phase order.
 // Per-tile partials (FP64 lens terms, Kahan-compensated FP32 slot sums) are
 // added in fixed order (the lens terms by tile, the subhalo sums by launch
 // position) by a final kernel, so results are deterministic.
@@ -32,8 +33,8 @@
 // x dG/dx (1 rsqrt and two short polynomials per pair) with no per-pair
 // test, with as few terms as the box's distance allows (vj_degree). Where
 // the tile is also small against its distance from the subhalo (half-
-// diagonal within 0.08 of it) and a tile is swept in one phase, the same
-// series is summed by its local expansion about the tile's centre
+// diagonal within 0.08 of it) and has 64 points or more in one staged chunk, the
+// same series is summed by its local expansion about the tile's centre
 // (vj_expand): the tile's gradient moments are formed once (vj_moments), and
 // each such subhalo costs a fixed 24 terms instead of a pass over the points.
 // The others take the far-side closed form per pair and the general form for
@@ -197,13 +198,12 @@ __device__ __forceinline__ void vj_series2(const VjSer<K>& c, float2 x2, float2&
 
 // K > 0: every staged point of the CTA is at or beyond the radius of the
 // gradient's series of degree K (tNFW only), so that series serves every
-// pair without a test; K = 0: the closed forms. P1: one phase (P = 1), so
-// that consecutive steps read neighbouring point pairs.
-template <int PROFILE, int K, bool P1>
+// pair without a test; K = 0: the closed forms. P: the slot's stride over the
+// point pairs.
+template <int PROFILE, int K>
 __device__ __forceinline__ void vj_sweep(const SubRec& rec, float2 ex, const SubSer& q,
                                          const float4* __restrict__ pos, const float4* __restrict__ grad, int npairs,
-                                         int r, int Pr, float* s, float* c) {
-  const int P = P1 ? 1 : Pr;  // the slot's stride over the point pairs
+                                         int r, int P, float* s, float* c) {
   const SubRec2 H = sub_pair(rec, rec);
   constexpr bool kSeries = PROFILE == LR_PROFILE_TNFW && K > 0;
   const VjSer<kSeries ? K : 3> ser = vj_series_coeffs<kSeries ? K : 3>(q);
@@ -721,11 +721,11 @@ __device__ __forceinline__ void vj_tile_sums(const float* __restrict__ sub, int 
       const float tau = __ldg(rr + 4), t2 = tau * tau;
       const float2 ex = make_float2(4.0f * t2 / ((t2 + 1.0f) * (t2 + 1.0f)), 1.0f / __ldg(rr + 3));
       switch (deg) {
-        case 3: vj_sweep<PR, 3, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
-        case 4: vj_sweep<PR, 4, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
-        case 5: vj_sweep<PR, 5, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
-        case 7: vj_sweep<PR, 7, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
-        default: vj_sweep<PR, 0, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
+        case 3: vj_sweep<PR, 3>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+        case 4: vj_sweep<PR, 4>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+        case 5: vj_sweep<PR, 5>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+        case 7: vj_sweep<PR, 7>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+        default: vj_sweep<PR, 0>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
       }
 #pragma unroll
       for (int v = 0; v < 4; ++v) sc[v] = __fmul_rn(sc[v] - cc[v], vj_scale<PR>(rec, ex, v));
@@ -813,7 +813,7 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
   // tNFW: the subhalos in the order of their classes for the tile's box
   // (vj_sort), from the plan or sorted here; more than kVjMaxOrd subhalos:
   // index order. Each slot finds its subhalo's class itself (vj_class). The
-  // local expansion needs one phase and one staged chunk.
+  // local expansion needs one staged chunk.
   const bool ordered = PROFILE == LR_PROFILE_TNFW && n_sub > 0 && n_sub <= kVjMaxOrd;
   const bool one = ordered && nchunks == 1;  // one staged chunk: vj_tile_sums takes the subhalos
   const bool exp_ok = vj_exp_ok(one, (int)(p1 - p0));
@@ -873,11 +873,11 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
       if (own) {
         const int np = (cnt + 1) >> 1;
         switch (deg) {
-          case 3: vj_sweep<PROFILE, 3, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
-          case 4: vj_sweep<PROFILE, 4, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
-          case 5: vj_sweep<PROFILE, 5, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
-          case 7: vj_sweep<PROFILE, 7, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
-          default: vj_sweep<PROFILE, 0, false>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
+          case 3: vj_sweep<PROFILE, 3>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+          case 4: vj_sweep<PROFILE, 4>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+          case 5: vj_sweep<PROFILE, 5>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+          case 7: vj_sweep<PROFILE, 7>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
+          default: vj_sweep<PROFILE, 0>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
         }
       }
     }
@@ -1048,11 +1048,10 @@ static bool vjp_planned(int64_t ntiles, const lr_points* p) {
   return p->profile == LR_PROFILE_TNFW && plan_fits(ntiles, p->n_sub);
 }
 
-// Phases P of the subhalo sums: 1 when n_sub slots waste at most 5 % of the
-// last group of kVjThreads (one phase sweeps with a constant stride and
-// allows the local expansion), else the P in [1, kVjMaxPhases] whose slot
-// count n_sub P wastes the fewest threads of the last group (the smallest
-// such P), keeping at least 128 points per slot.
+// Phases P of the subhalo sums of tiles that do not choose their own: 1 when
+// n_sub slots waste at most 5 % of the last group of kVjThreads, else the P in
+// [1, kVjMaxPhases] whose slot count n_sub P wastes the fewest threads of the
+// last group (the smallest such P), keeping at least 128 points per slot.
 int vjp_phases(int64_t n, int32_t n_sub) {
   if (n_sub <= 0 || n <= 0) return 1;
   const int64_t per_cta = (n + vjp_tiles(n) - 1) / vjp_tiles(n);
