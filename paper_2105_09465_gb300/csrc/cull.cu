@@ -1131,8 +1131,8 @@ lr_status plan_cull(int kind, int nrhs, int64_t n, const lr_grid* qlayout, int64
   const bool windowed = kind == kCullWin || kind == kCullWinRows || kind == kCullWinCols;
   P.R = cull_rows_per_thread(kind, P.nw, layers);
   P.extra = (int32_t)(kPartWaves * slots);
-  P.parts = P.row_blocks > 0 && P.L.n_groups > 0 &&
-            (windowed || (allow_parts && m > kPartSources && P.row_blocks < kFewWaves * slots));
+  // (with no sources too: the windowed kinds have no other kernel, and their merge writes the outputs)
+  P.parts = P.row_blocks > 0 && (windowed || (allow_parts && m > kPartSources && P.row_blocks < kFewWaves * slots));
   P.K = cull_k(kind, P.nw, layers);
   size_t off = 0;
   P.off_rec = off;
@@ -1192,8 +1192,11 @@ static lr_status launch_prep_kernels(const CullPlan& P, CullPrepP& Q, char* ws, 
   Q.rec = ws + P.off_rec;
   Q.cbox = reinterpret_cast<float4*>(ws + P.off_cbox);
   Q.gbox = reinterpret_cast<float4*>(ws + P.off_gbox);
-  if (P.L.n_chunks == 0) return LR_OK;
   if (P.parts) Q.ticket = plan_ticket(P, ws);
+  if (P.L.n_chunks == 0) {  // no sources: the plan kernel still counts its CTAs
+    if (Q.ticket) LR_CHECK_CUDA(cudaMemsetAsync(Q.ticket, 0, 2 * sizeof(unsigned long long), s));
+    return LR_OK;
+  }
   cull_prep_kernel<<<(unsigned)P.L.n_groups, kPrepThreads, 0, s>>>(Q);
   LR_CHECK_CUDA(cudaGetLastError());
   return LR_OK;
