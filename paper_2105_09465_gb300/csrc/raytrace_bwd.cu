@@ -115,6 +115,12 @@ __device__ __forceinline__ void vj_accum2(float2 dx, float2 dy, float2 gx, float
   a3 = __ffma2_rn(hg, dg, a3);
 }
 
+// A tNFW record's (4T, 1 / theta_s), T = tau^2 / (tau^2 + 1)^2.
+__device__ __forceinline__ float2 vj_tnfw_ex(float ts, float tau) {
+  const float t2 = tau * tau;
+  return make_float2(4.0f * t2 / ((t2 + 1.0f) * (t2 + 1.0f)), 1.0f / ts);
+}
+
 // The constant factors of a tNFW slot's four sums (1 for a point mass, whose
 // terms are accumulated whole).
 template <int PROFILE>
@@ -467,7 +473,7 @@ __device__ __forceinline__ void vj_moments(VjSmem& sm, int cnt, float2 cen) {
 // products with the moments, four sums), all unrolled. With the 36 plain
 // moments, 40 operations each in rolled loops of 15 to 36 terms, the VJP took
 // 1.23 ms at 2.56M points x 2000 subhalos, now 0.90.
-__device__ __forceinline__ float4 vj_expand(const SubRec& rec, const SubSer& q, float kappa, float ts, float2 cen,
+__device__ __forceinline__ float4 vj_expand(const SubRec& rec, const SubSer& q, float ts, float2 ex, float2 cen,
                                             const VjSmem& sm) {
   const float2 c = make_float2(cen.x - rec.xh, cen.y - rec.yh);
   const float ir2 = 1.0f / fmaf(c.x, c.x, c.y * c.y);
@@ -514,8 +520,9 @@ __device__ __forceinline__ float4 vj_expand(const SubRec& rec, const SubSer& q, 
       Y = fmaf(s, ry, Y);
     }
   }
-  const float sc = rec.A * ts * ts;
-  return make_float4(sc * X, sc * Y, -sc * L / kappa, -sc * Lt / ts);
+  // the direct sums' factors (vj_scale): no division by kappa_s, which may be 0
+  const float t2 = ts * ts, sc = rec.A * t2;
+  return make_float4(sc * X, sc * Y, -ex.x * t2 * L, -rec.A * ts * Lt);
 }
 
 // The CTA's points: u in [u0, u1) indexes explicit points directly; on a
@@ -699,7 +706,8 @@ __device__ __forceinline__ void vj_tile_sums(const float* __restrict__ sub, int 
     const float* rr = sub + 5 * (int64_t)h;
     const SubRec rec = prep_sub(rr, PR);
     const SubSer q = prep_series(rec, PR);
-    const float4 x = vj_expand(rec, q, __ldg(rr + 2), __ldg(rr + 3), cen, sm);
+    const float ts = __ldg(rr + 3);
+    const float4 x = vj_expand(rec, q, ts, vj_tnfw_ex(ts, __ldg(rr + 4)), cen, sm);
     float* o = sub_part + (int64_t)h * 4 * nblk + blk;  // [value][CTA]
     o[0] = x.x;
     o[nblk] = x.y;
@@ -718,8 +726,7 @@ __device__ __forceinline__ void vj_tile_sums(const float* __restrict__ sub, int 
       const SubRec rec = prep_sub(rr, PR);
       const SubSer q = prep_series(rec, PR);
       const int deg = vj_degree_box(rec, q, sm.box);
-      const float tau = __ldg(rr + 4), t2 = tau * tau;
-      const float2 ex = make_float2(4.0f * t2 / ((t2 + 1.0f) * (t2 + 1.0f)), 1.0f / __ldg(rr + 3));
+      const float2 ex = vj_tnfw_ex(__ldg(rr + 3), __ldg(rr + 4));
       switch (deg) {
         case 3: vj_sweep<PR, 3>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
         case 4: vj_sweep<PR, 4>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc); break;
@@ -857,8 +864,7 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
       if (PROFILE == LR_PROFILE_POINT_MASS) {
         ex = make_float2(0.f, __ldg(rr + 2));
       } else {
-        const float tau = __ldg(rr + 4), t2 = tau * tau;
-        ex = make_float2(4.0f * t2 / ((t2 + 1.0f) * (t2 + 1.0f)), 1.0f / __ldg(rr + 3));
+        ex = vj_tnfw_ex(__ldg(rr + 3), __ldg(rr + 4));
       }
     }
     float sc[4] = {0.f, 0.f, 0.f, 0.f}, cc[4] = {0.f, 0.f, 0.f, 0.f};

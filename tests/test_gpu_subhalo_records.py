@@ -1,0 +1,47 @@
+"""Subhalo records at the edges of what a fit or a padded list holds, where
+tiles take the local expansion: zero mass (kappa_s = 0: the deflection is 0 but
+its derivative by kappa_s is not). Against the FP64 oracle within 2e-5 of the
+sum of absolute terms (the repository's gradient tolerance)."""
+import numpy as np
+import pytest
+
+from paper_2105_09465_gb300 import api, workloads as W
+from tests.gpu_util import GRAD_REL, assert_close_tol, dev, host, need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    need_gpu()
+
+
+def check_vjp(orc, g, lens, sub, seed, ref_sub=None, sign=1.0):
+    """Subhalo gradients of the grid g against the oracle's for ref_sub, its
+    theta_s column times sign."""
+    xi = orc.grid_points(*g.astuple())
+    d = np.random.default_rng(seed).standard_normal((g.n, 2)).astype(np.float32)
+    _, ds = api.lens_raytrace_vjp(api.Points(grid=g, lens=lens, sub=dev(sub)), dev(d))
+    _, rs, _, asub = orc.raytrace_vjp(xi.astype(np.float64), lens.astuple(), sub if ref_sub is None else ref_sub,
+                                      d.astype(np.float64), with_abs=True)
+    rs[:, 3] *= sign
+    assert np.isfinite(host(ds)).all()
+    assert_close_tol(host(ds), rs, GRAD_REL * asub, what="subhalos")
+
+
+def population(rng, n_sub):
+    """Near and far subhalos of a field of about 4 arcsec."""
+    return np.column_stack([rng.uniform(-9, 9, (n_sub, 2)), rng.uniform(0.01, 0.1, n_sub),
+                            rng.uniform(0.02, 0.1, n_sub), rng.uniform(1, 15, n_sub)]).astype(np.float32)
+
+
+# 640k points x 200: more than one wave of tiles, ordered by the plan
+@pytest.mark.parametrize("n_sub,side,which", [(1, 32, "all"), (17, 32, "one"), (17, 32, "all"), (200, 32, "one"),
+                                              (200, 32, "half"), (200, 32, "all"), (257, 60, "half"),
+                                              (200, 400, "half")])
+def test_zero_mass(orc, n_sub, side, which):
+    rng = np.random.default_rng(n_sub + side)
+    g = W.Grid(side, side, 2, 4.0 / side)
+    sub = population(rng, n_sub)
+    sub[{"one": slice(0, 1), "half": slice(n_sub // 2, None), "all": slice(None)}[which], 2] = 0.0
+    check_vjp(orc, g, W.draw_lens(rng), sub, n_sub)
