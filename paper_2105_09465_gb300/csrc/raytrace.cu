@@ -452,7 +452,7 @@ __device__ constexpr int rt_coef_at(int k, int l) { return l * (2 * kExpN + 3 - 
 // r2 = |c|^2).
 __device__ __forceinline__ void rt_exp_add(const SubRec& rec, const SubSer& q, float ts, float2 c, float r2, float h,
                                            float (&acc)[kRtExpFloats]) {
-  const float ir2 = 1.0f / r2, yc = ts * sqrtf(ir2);
+  const float ir2 = 1.0f / r2, yc = fabsf(ts) * sqrtf(ir2);  // theta_s by its modulus, as in the direct sums (its2)
   float qy[8], yj = rec.A * ts * ts / h;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {

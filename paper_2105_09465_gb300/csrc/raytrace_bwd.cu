@@ -478,7 +478,7 @@ __device__ __forceinline__ float4 vj_expand(const SubRec& rec, const SubSer& q, 
   const float2 c = make_float2(cen.x - rec.xh, cen.y - rec.yh);
   const float ir2 = 1.0f / fmaf(c.x, c.x, c.y * c.y);
   const float2 ub = make_float2(c.x * ir2, c.y * ir2);  // conj(u)
-  const float yc = ts * sqrtf(ir2);
+  const float yc = fabsf(ts) * sqrtf(ir2);  // theta_s / |c|, by its modulus as in the direct sums (its2)
   float qy[8], qt[8];
   float yj = 1.f;
 #pragma unroll

@@ -1,12 +1,14 @@
 """Subhalo records at the edges of what a fit or a padded list holds, where
 tiles take the local expansion: zero mass (kappa_s = 0: the deflection is 0 but
-its derivative by kappa_s is not). Against the FP64 oracle within 2e-5 of the
-sum of absolute terms (the repository's gradient tolerance)."""
+its derivative by kappa_s is not), and a negative scale radius (only its square and
+its modulus enter). Against the FP64 oracle: gradients within 2e-5 of the sum of
+absolute terms (the repository's gradient tolerance), deflections within 1e-6
+arcsec."""
 import numpy as np
 import pytest
 
 from paper_2105_09465_gb300 import api, workloads as W
-from tests.gpu_util import GRAD_REL, assert_close_tol, dev, host, need_gpu
+from tests.gpu_util import ALPHA_TOL, GRAD_REL, assert_close_tol, dev, host, need_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -16,11 +18,10 @@ def _gpu():
     need_gpu()
 
 
-def check_vjp(orc, g, lens, sub, seed, ref_sub=None, sign=1.0):
+def check_vjp(orc, g, lens, sub, d, ref_sub=None, sign=1.0):
     """Subhalo gradients of the grid g against the oracle's for ref_sub, its
     theta_s column times sign."""
     xi = orc.grid_points(*g.astuple())
-    d = np.random.default_rng(seed).standard_normal((g.n, 2)).astype(np.float32)
     _, ds = api.lens_raytrace_vjp(api.Points(grid=g, lens=lens, sub=dev(sub)), dev(d))
     _, rs, _, asub = orc.raytrace_vjp(xi.astype(np.float64), lens.astuple(), sub if ref_sub is None else ref_sub,
                                       d.astype(np.float64), with_abs=True)
@@ -44,4 +45,33 @@ def test_zero_mass(orc, n_sub, side, which):
     g = W.Grid(side, side, 2, 4.0 / side)
     sub = population(rng, n_sub)
     sub[{"one": slice(0, 1), "half": slice(n_sub // 2, None), "all": slice(None)}[which], 2] = 0.0
-    check_vjp(orc, g, W.draw_lens(rng), sub, n_sub)
+    check_vjp(orc, g, W.draw_lens(rng), sub, rng.standard_normal((g.n, 2)).astype(np.float32))
+
+
+@pytest.mark.parametrize("n_sub", [17, 200])
+def test_negative_scale_radius_backward(orc, n_sub):
+    rng = np.random.default_rng(n_sub)
+    ref = population(rng, n_sub)
+    ref[:, :2] /= 3.0
+    ref[:, 3:] = (0.1, 1.0)  # the series' odd terms: 7e-4 of the sums at 1.6 arcsec
+    sub = ref.copy()
+    sub[:, 3] *= -1.0
+    g = W.Grid(40, 40, 2, 0.02)  # 50 tiles of 8 x 16 points
+    # one gradient at every point: the sums are of the size of their absolute terms
+    check_vjp(orc, g, W.draw_lens(rng), sub, np.tile(np.float32([0.8, -0.6]), (g.n, 1)), ref, -1.0)
+
+
+@pytest.mark.parametrize("n_sub", [64, 300])
+def test_negative_scale_radius_forward(orc, n_sub):
+    g = W.Grid(90, 33, 2, 0.01)
+    lens = W.Lens(0.0, 0.0, 0.9, 0.2, 1e-9, 2.0, 0.0, 0.0)
+    rng = np.random.default_rng(n_sub)
+    ref = population(rng, n_sub)
+    ref[:, 2:] = (6.0 / n_sub, 0.1, 1.0)
+    t = rng.uniform(0, 2 * np.pi, n_sub)  # the odd terms are 3e-4 of the deflection, 0.03 arcsec
+    ref[:, 0], ref[:, 1] = 2.15 + 0.05 * np.cos(t), 0.05 * np.sin(t)
+    sub = ref.copy()
+    sub[:, 3] *= -1.0
+    _, alpha = api.lens_raytrace(api.Points(grid=g, lens=lens, sub=dev(sub)), want_alpha=True)
+    want, _ = orc.raytrace(orc.grid_points(*g.astuple()), lens.astuple(), ref, 0)
+    assert np.abs(host(alpha) - want).max() <= ALPHA_TOL
