@@ -321,7 +321,8 @@ __device__ __forceinline__ int vj_degree_box(const SubRec& h, const SubSer& q, c
 // give alpha as a polynomial in delta and conj(delta) whose coefficients
 // depend on the subhalo alone:
 //   alpha(c + delta) = A theta_s^2 sum_{k,l} c_kl u^k conj(u)^(l+1) delta^k conj(delta)^l,
-//   c_kl = sum_j q_j (theta_s / |c|)^j C(-j/2, k) C(-(j+2)/2, l), u = 1/c.
+//   c_kl = sum_j q_j (theta_s / |c|)^j C(-j/2, k) C(-(j+2)/2, l), u = 1/c
+// (formed with delta and c in units of about the tile's size, vj_unit).
 // The four gradient sums over the tile's points then need only the tile's
 // moments W_kl = sum_i conj(G_i) delta_i^k conj(delta_i)^l (vj_moments):
 //   sum_i G_i . alpha_i = Re sum_kl M_kl W_kl, with M_kl the coefficients,
@@ -363,7 +364,7 @@ static_assert(vj_pair_at(kExpN + 1, 0) + 1 == kVjPairTerms, "the last term ends 
 // into sm.mred: at most 7 complex products per point for the powers of delta
 // and conj(delta), then one per moment.
 template <int L0, int L1>
-__device__ __forceinline__ void vj_moment_pass(VjSmem& sm, int cnt, float2 cen) {
+__device__ __forceinline__ void vj_moment_pass(VjSmem& sm, int cnt, float2 cen, float ih) {
   constexpr int F = 2 * vj_moment_at(0, L0), N = 2 * vj_moment_at(0, L1) - F;  // first float, floats
   constexpr int NR = (N + 31) / 32 * 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -373,7 +374,7 @@ __device__ __forceinline__ void vj_moment_pass(VjSmem& sm, int cnt, float2 cen) 
   for (int i = threadIdx.x; i < cnt; i += kVjThreads) {
     const float4 P = sm.pos[i >> 1], D = sm.grad[i >> 1];
     const bool b = i & 1;
-    const float2 d = make_float2((b ? P.y : P.x) - cen.x, (b ? P.w : P.z) - cen.y);
+    const float2 d = make_float2(((b ? P.y : P.x) - cen.x) * ih, ((b ? P.w : P.z) - cen.y) * ih);
     float2 pw[kVjExpN + 1 - L0];  // delta^k
     pw[0] = make_float2(1.f, 0.f);
 #pragma unroll
@@ -407,17 +408,28 @@ __device__ __forceinline__ void vj_moment_pass(VjSmem& sm, int cnt, float2 cen) 
   }
 }
 
-// The tile's moments about cen over its staged points (one chunk of cnt
-// points): W into sm.wm[0], W_x into sm.wm[1], W_y into sm.wm[2]. Every thread
+// The unit of length of a tile's expansion: the power of two at or below its
+// half-diagonal (1 for a single point). In units of it the eighth powers of
+// delta and 1 / c stay within FP32 whatever the coordinates' own unit, and the
+// scaling rounds nothing.
+__device__ __forceinline__ float vj_unit(const float* box) {
+  const float hx = 0.5f * (box[2] - box[0]), hy = 0.5f * (box[3] - box[1]);
+  const float hd2 = fmaf(hx, hx, hy * hy);
+  return hd2 > 0.f ? scalbnf(1.0f, ilogbf(hd2) >> 1) : 1.0f;
+}
+
+// The tile's moments about cen, in units of h, over its staged points (one chunk
+// of cnt points): W into sm.wm[0], W_x into sm.wm[1], W_y into sm.wm[2]. Every thread
 // sums all 36 moments over its own points, in two passes that fit the
 // registers, and the warps' sums are added in order; bound by the 36 complex
 // products per point. With three threads per moment, each forming its powers
 // from scratch for every point, this took 0.83 of the kernel's 2.29 ms at
 // 2.56M points x 2000 subhalos.
-__device__ __forceinline__ void vj_moments(VjSmem& sm, int cnt, float2 cen) {
+__device__ __forceinline__ void vj_moments(VjSmem& sm, int cnt, float2 cen, float h) {
   const int t = threadIdx.x;
-  vj_moment_pass<0, 2>(sm, cnt, cen);
-  vj_moment_pass<2, kVjExpN + 1>(sm, cnt, cen);
+  const float ih = 1.0f / h;
+  vj_moment_pass<0, 2>(sm, cnt, cen, ih);
+  vj_moment_pass<2, kVjExpN + 1>(sm, cnt, cen, ih);
   __syncthreads();
   if (t < kVjExpTerms) {
     int s = 0;
@@ -474,10 +486,11 @@ __device__ __forceinline__ void vj_moments(VjSmem& sm, int cnt, float2 cen) {
 // moments, 40 operations each in rolled loops of 15 to 36 terms, the VJP took
 // 1.23 ms at 2.56M points x 2000 subhalos, now 0.90.
 __device__ __forceinline__ float4 vj_expand(const SubRec& rec, const SubSer& q, float ts, float2 ex, float2 cen,
-                                            const VjSmem& sm) {
+                                            float h, const VjSmem& sm) {
   const float2 c = make_float2(cen.x - rec.xh, cen.y - rec.yh);
   const float ir2 = 1.0f / fmaf(c.x, c.x, c.y * c.y);
-  const float2 ub = make_float2(c.x * ir2, c.y * ir2);  // conj(u)
+  const float hr = h * ir2, rho2 = h * hr;
+  const float2 ub = make_float2(c.x * hr, c.y * hr);  // h conj(u)
   const float yc = fabsf(ts) * sqrtf(ir2);  // theta_s / |c|, by its modulus as in the direct sums (its2)
   float qy[8], qt[8];
   float yj = 1.f;
@@ -487,11 +500,11 @@ __device__ __forceinline__ float4 vj_expand(const SubRec& rec, const SubSer& q, 
     qt[j] = (float)(j + 2) * qy[j];
     yj *= yc;
   }
-  float rk[kExpN / 2 + 2];  // |u|^2k
+  float rk[kExpN / 2 + 2];  // (h |u|)^2k
   rk[0] = 1.f;
 #pragma unroll
-  for (int k = 1; k < kExpN / 2 + 2; ++k) rk[k] = rk[k - 1] * ir2;
-  float2 um = make_float2(1.f, 0.f);  // conj(u)^m
+  for (int k = 1; k < kExpN / 2 + 2; ++k) rk[k] = rk[k - 1] * rho2;
+  float2 um = make_float2(1.f, 0.f);  // (h conj(u))^m
   float L = 0.f, Lt = 0.f, X = 0.f, Y = 0.f;
 #pragma unroll
   for (int m = 0; m <= kExpN + 1; ++m) {
@@ -521,8 +534,8 @@ __device__ __forceinline__ float4 vj_expand(const SubRec& rec, const SubSer& q, 
     }
   }
   // the direct sums' factors (vj_scale): no division by kappa_s, which may be 0
-  const float t2 = ts * ts, sc = rec.A * t2;
-  return make_float4(sc * X, sc * Y, -ex.x * t2 * L, -rec.A * ts * Lt);
+  const float th = ts / h, t2 = ts * th, sc = rec.A * th * th;
+  return make_float4(sc * X, sc * Y, -ex.x * t2 * L, -rec.A * th * Lt);
 }
 
 // The CTA's points: u in [u0, u1) indexes explicit points directly; on a
@@ -697,7 +710,7 @@ __device__ __forceinline__ int vj_pick_phases(int nd, int np) {
 // one phase count per launch, 200 subhalos ran in 3 phases and every pair
 // directly (249 us at 640k points).
 __device__ __forceinline__ void vj_tile_sums(const float* __restrict__ sub, int n_sub, int nexp,
-                                             const unsigned short* __restrict__ ord, int cnt, float2 cen,
+                                             const unsigned short* __restrict__ ord, int cnt, float2 cen, float unit,
                                              float* __restrict__ sub_part, int64_t blk, int64_t nblk, VjSmem& sm) {
   constexpr int PR = LR_PROFILE_TNFW;
   const int tid = threadIdx.x;
@@ -707,7 +720,7 @@ __device__ __forceinline__ void vj_tile_sums(const float* __restrict__ sub, int 
     const SubRec rec = prep_sub(rr, PR);
     const SubSer q = prep_series(rec, PR);
     const float ts = __ldg(rr + 3);
-    const float4 x = vj_expand(rec, q, ts, vj_tnfw_ex(ts, __ldg(rr + 4)), cen, sm);
+    const float4 x = vj_expand(rec, q, ts, vj_tnfw_ex(ts, __ldg(rr + 4)), cen, unit, sm);
     float* o = sub_part + (int64_t)h * 4 * nblk + blk;  // [value][CTA]
     o[0] = x.x;
     o[nblk] = x.y;
@@ -836,8 +849,9 @@ __device__ __forceinline__ void vjp_body(const LensConst& L, const LensGradConst
       vj_lens_out(la, lens_part + tile * 7, sm);  // its barrier also ends the staging
       const float2 cen = make_float2(0.5f * (sm.box[0] + sm.box[2]), 0.5f * (sm.box[1] + sm.box[3]));
       const int nexp = plan.nexp ? plan.nexp[tile] : sm.nexp;
-      if (nexp > 0) vj_moments(sm, cnt, cen);  // uniform over the CTA
-      vj_tile_sums(sub, n_sub, nexp, ord, cnt, cen, sub_part, blk, nblk, sm);
+      const float unit = vj_unit(sm.box);
+      if (nexp > 0) vj_moments(sm, cnt, cen, unit);  // uniform over the CTA
+      vj_tile_sums(sub, n_sub, nexp, ord, cnt, cen, unit, sub_part, blk, nblk, sm);
       return;
     }
   }

@@ -1,9 +1,10 @@
 """Subhalo records at the edges of what a fit or a padded list holds, where
 tiles take the local expansion: zero mass (kappa_s = 0: the deflection is 0 but
-its derivative by kappa_s is not), and a negative scale radius (only its square and
-its modulus enter). Against the FP64 oracle: gradients within 2e-5 of the sum of
-absolute terms (the repository's gradient tolerance), deflections within 1e-6
-arcsec."""
+its derivative by kappa_s is not), a negative scale radius (only its square and
+its modulus enter), and coordinates far from the size of an arcsecond. Values
+against the FP64 oracle: gradients within 2e-5 of the sum of absolute terms
+(the repository's gradient tolerance), deflections within 1e-6 of the scale of
+the coordinates."""
 import numpy as np
 import pytest
 
@@ -75,3 +76,17 @@ def test_negative_scale_radius_forward(orc, n_sub):
     _, alpha = api.lens_raytrace(api.Points(grid=g, lens=lens, sub=dev(sub)), want_alpha=True)
     want, _ = orc.raytrace(orc.grid_points(*g.astuple()), lens.astuple(), ref, 0)
     assert np.abs(host(alpha) - want).max() <= ALPHA_TOL
+
+
+@pytest.mark.parametrize("scale", [2.0**-18, 2.0**18])
+@pytest.mark.parametrize("n_sub", [17, 200])
+def test_scale_of_the_coordinates(orc, n_sub, scale):
+    rng = np.random.default_rng(n_sub)
+    g = W.Grid(90, 33, 2, 0.05 * scale)
+    lens = W.Lens(0.0, 0.0, 0.9, 0.2, 1e-9 * scale, 2.0, 0.0, 0.0)
+    sub = population(rng, n_sub)
+    sub[:, [0, 1, 3]] *= np.float32(scale)
+    check_vjp(orc, g, lens, sub, rng.standard_normal((g.n, 2)).astype(np.float32))
+    _, alpha = api.lens_raytrace(api.Points(grid=g, lens=lens, sub=dev(sub)), want_alpha=True)
+    want, _ = orc.raytrace(orc.grid_points(*g.astuple()), lens.astuple(), sub, 0)
+    assert np.abs(host(alpha) - want).max() <= ALPHA_TOL * scale
