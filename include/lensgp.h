@@ -278,6 +278,10 @@ lr_status gp_kernel_matvec(const lr_points* query, const lr_points* source, cons
  * float[L]; v is device float[L][m][nrhs] (layer-major), out device
  * float[n][nrhs]. Sources may be explicit or a grid, or NULL for a
  * self-kernel (the paper's image-plane GP); they may not carry a lens.
+ * Pairs whose kernel value is exactly 0 are left out, but every row's sum
+ * takes in every source: a weight that is not finite, or a source coordinate
+ * that is not a number, makes every row of its right-hand side (of all of
+ * them, for a coordinate) not a number, however far the source (0 * inf).
  * Other arguments as gp_kernel_matvec; workspace of
  * lr_matvec_layers_workspace_size() bytes.
  */

@@ -53,6 +53,7 @@ __device__ __forceinline__ float4 warp_box(float4 b) {
 }
 
 constexpr float4 kEmptyBox = {INFINITY, INFINITY, -INFINITY, -INFINITY};
+constexpr float4 kEveryBox = {-INFINITY, -INFINITY, INFINITY, INFINITY};  // within reach of any box
 
 // ---------------------------------------------------------------------------
 // Prepare: one CTA per group, one warp per chunk at a time (lane = slot). Writes
@@ -60,21 +61,40 @@ constexpr float4 kEmptyBox = {INFINITY, INFINITY, -INFINITY, -INFINITY};
 // reach scale. Bound by the records' writes; one launch for chunks and groups.
 constexpr int kPrepThreads = 1024;
 
+// kCullLay: writes the slot's weights, and says whether a weight of the chunk is
+// not finite or a point of it not a number. Its product with a kernel value of 0
+// is not 0 then, so no row leaves the chunk out.
+__device__ __forceinline__ bool lay_weights(const CullPrepP& P, int64_t i, bool valid, float2 pv, float* w) {
+  bool bad = valid && (isnan(pv.x) || isnan(pv.y));
+  const int nr = P.nw / P.layers;
+  for (int l = 0; l < P.layers; ++l) {
+    const float* al = P.a + ((int64_t)P.lay_src[l] * P.L.n + i) * nr;
+    for (int k = 0; k < nr; ++k) {
+      const float x = valid ? P.lay_var[l] * al[k] : 0.f;
+      w[(l * nr + k) * kChunkPts] = x;
+      bad = bad || !isfinite(x);
+    }
+  }
+  return __any_sync(0xffffffffu, bad);
+}
+
 __device__ __forceinline__ void prep_chunk(const CullPrepP& P, int c, int lane, float4& obox, float& oreach) {
   const int64_t i = chunk_point(P.L, c, lane);
   const bool valid = i >= 0;
   const float2 pv = valid ? (P.pts ? P.pts[i] : grid_point(P.grid, i)) : f2(0.f, 0.f);
-  const float4 box = warp_box(valid ? make_float4(pv.x, pv.y, pv.x, pv.y) : kEmptyBox);
+  float4 box = warp_box(valid ? make_float4(pv.x, pv.y, pv.x, pv.y) : kEmptyBox);
   // an empty slot sits at its chunk's box corner with weight 0
   const float2 p = valid ? pv : f2(box.x, box.y);
   const int RB = rec_bytes(P.nw);
   char* rec = P.rec + (int64_t)c * RB;
+  float* w = reinterpret_cast<float*>(rec + kRecHead + kRecXY);  // [nw][32], pairs consecutive
+  if (P.kind == kCullLay && lay_weights(P, i, valid, pv, w + lane)) box = kEveryBox;
   obox = box;
   oreach = INFINITY;
   if (lane == 0) P.cbox[c] = box;
   if (!(box.x <= box.z)) {  // an empty chunk: never within reach
-    float* w = reinterpret_cast<float*>(rec);
-    for (int k = lane; k < RB / 4; k += 32) w[k] = 0.f;
+    float* z = reinterpret_cast<float*>(rec);
+    for (int k = lane; k < RB / 4; k += 32) z[k] = 0.f;
     __syncwarp();
     if (lane == 0) {
       *reinterpret_cast<float4*>(rec) = box;
@@ -107,15 +127,9 @@ __device__ __forceinline__ void prep_chunk(const CullPrepP& P, int c, int lane, 
   const int pr = lane >> 1, half = lane & 1;
   xy[4 * pr + half] = p.x;
   xy[4 * pr + 2 + half] = p.y;
-  float* w = reinterpret_cast<float*>(rec + kRecHead + kRecXY);  // [nw][32], pairs consecutive
   if (P.kind == kCullOut) {
     for (int k = 0; k < P.nw; ++k) w[k * kChunkPts + lane] = valid ? P.a[i * P.stride + k] : 0.f;
-  } else if (P.kind == kCullLay) {
-    const int nr = P.nw / P.layers;
-    for (int l = 0; l < P.layers; ++l) {
-      const float* al = P.a + ((int64_t)P.lay_src[l] * P.L.n + i) * nr;
-      for (int k = 0; k < nr; ++k) w[(l * nr + k) * kChunkPts + lane] = valid ? P.lay_var[l] * al[k] : 0.f;
-    }
+  } else if (P.kind == kCullLay) {  // written above
   } else if (P.kind == kCullWin || P.kind == kCullWinRows) {
     w[lane] = valid ? P.a[i] : 0.f;
   } else if (P.kind == kCullWinCols) {
