@@ -33,14 +33,15 @@ lr_status kernel_occupancy(Fn* fn, int threads, int* occ, int* n_sm) {
 void ktimer_begin(int id, cudaStream_t s);
 void ktimer_end(int id, cudaStream_t s);
 
-// Fork and join: fork_begin makes a per-device side stream wait for the work
-// enqueued on s so far (f->side is s itself when no side stream exists);
+// Fork and join: fork_begin makes a side stream wait for the work enqueued on s
+// so far (f->side is s itself when no side stream is free);
 // fork_end makes s wait for the side stream's work since. Under stream
 // capture the two become graph edges. Every fork_begin that returned LR_OK
 // must be followed by fork_end, also on error paths.
 struct Fork {
   cudaStream_t side;
   cudaEvent_t join;
+  void* slot;  // the side stream's place in the library's table
 };
 lr_status fork_begin(cudaStream_t s, Fork* f);
 lr_status fork_end(cudaStream_t s, Fork* f);

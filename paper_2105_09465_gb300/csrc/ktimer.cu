@@ -121,34 +121,104 @@ extern "C" lr_status lr_kernel_timer_read(int32_t kernel, int64_t* launches, dou
 
 // ---------------------------------------------------------------------------
 // Fork and join of a second stream for independent branches of one entry
-// point (see common.cuh). The side stream is per device and non-blocking;
-// the events are per call, so concurrent callers never share one.
+// point (see common.cuh). Side streams are non-blocking and kept, at most
+// kSides a device, each used by one fork at a time. A fork takes the one that
+// last served its own stream, so that callers on different streams do not queue
+// behind one another, and never one that another capture has drawn in: a side
+// stream stays in the capture that forked onto it until that capture ends, and
+// anything else put on it would fail or end up in that graph. The events are
+// per call.
 namespace lr {
+namespace {
 
-cudaStream_t side_stream() {
-  static std::mutex mu;
-  static cudaStream_t streams[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-  std::lock_guard<std::mutex> lk(mu);
-  if (!streams[dev] && cudaStreamCreateWithFlags(&streams[dev], cudaStreamNonBlocking) != cudaSuccess)
-    streams[dev] = nullptr;
-  return streams[dev];
+constexpr int kSides = 16, kSideDevs = 64;
+struct Side {
+  cudaStream_t stream, origin;  // the side stream, and the stream whose forks it last served
+  bool busy;                    // between fork_begin and fork_end
+  uint64_t used;
+};
+std::mutex g_side_mu;
+Side g_sides[kSideDevs][kSides];  // in use from the front
+uint64_t g_side_clock = 0;
+
+// The capture a stream is part of (0: none); false: it cannot be told, or the
+// capture is broken.
+bool capture_of(cudaStream_t s, unsigned long long* id) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  *id = 0;
+  if (cudaStreamGetCaptureInfo(s, &cs, id) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (cs == cudaStreamCaptureStatusNone) *id = 0;
+  return cs != cudaStreamCaptureStatusInvalidated;
 }
+
+cudaStream_t create_side() {
+  cudaStream_t t = nullptr;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // creating a stream disturbs no capture
+  const bool swapped = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+  if (cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    t = nullptr;
+  }
+  if (swapped) cudaThreadExchangeStreamCaptureMode(&mode);
+  return t;
+}
+
+// Takes a side stream of the current device for stream s, or nullptr (none
+// free: the branch runs on s).
+Side* take_side(cudaStream_t s) {
+  int dev = 0;
+  unsigned long long cap = 0, of = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kSideDevs || !capture_of(s, &cap)) return nullptr;
+  std::lock_guard<std::mutex> lk(g_side_mu);
+  Side* best = nullptr;
+  for (Side& e : g_sides[dev]) {
+    if (!e.stream) {
+      // a new one for a stream without its own
+      if ((!best || best->origin != s) && (e.stream = create_side()) != nullptr) best = &e;
+      break;
+    }
+    if (e.busy || !capture_of(e.stream, &of) || (of != 0 && of != cap)) continue;
+    const bool own = e.origin == s;
+    if (!best || (own && best->origin != s) || (own == (best->origin == s) && e.used < best->used)) best = &e;
+  }
+  if (best) {
+    best->busy = true;
+    best->origin = s;
+    best->used = ++g_side_clock;
+  }
+  return best;
+}
+
+void give_side(Side* e) {
+  std::lock_guard<std::mutex> lk(g_side_mu);
+  e->busy = false;
+}
+
+}  // namespace
 
 lr_status fork_begin(cudaStream_t s, Fork* f) {
   f->side = s;
   f->join = nullptr;
-  cudaStream_t side = side_stream();
-  if (!side) return LR_OK;  // no second stream: the branch runs on s
-  cudaEvent_t e = nullptr;
-  LR_CHECK_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  cudaError_t r = cudaEventRecord(e, s);
-  if (r == cudaSuccess) r = cudaStreamWaitEvent(side, e, 0);
-  cudaEventDestroy(e);
-  if (r != cudaSuccess) return cuda_status(r, "fork_begin");
-  LR_CHECK_CUDA(cudaEventCreateWithFlags(&f->join, cudaEventDisableTiming));
-  f->side = side;
+  f->slot = nullptr;
+  Side* e = take_side(s);
+  if (!e) return LR_OK;  // no second stream: the branch runs on s
+  cudaEvent_t ev = nullptr;
+  cudaError_t r = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+  if (r == cudaSuccess) {
+    r = cudaEventRecord(ev, s);
+    if (r == cudaSuccess) r = cudaStreamWaitEvent(e->stream, ev, 0);
+    cudaEventDestroy(ev);
+  }
+  if (r == cudaSuccess) r = cudaEventCreateWithFlags(&f->join, cudaEventDisableTiming);
+  if (r != cudaSuccess) {
+    give_side(e);
+    return cuda_status(r, "fork_begin");
+  }
+  f->side = e->stream;
+  f->slot = e;
   return LR_OK;
 }
 
@@ -157,7 +227,9 @@ lr_status fork_end(cudaStream_t s, Fork* f) {
   cudaError_t r = cudaEventRecord(f->join, f->side);
   if (r == cudaSuccess) r = cudaStreamWaitEvent(s, f->join, 0);
   cudaEventDestroy(f->join);
+  give_side(static_cast<Side*>(f->slot));
   f->join = nullptr;
+  f->slot = nullptr;
   f->side = s;
   return r == cudaSuccess ? LR_OK : cuda_status(r, "fork_end");
 }
