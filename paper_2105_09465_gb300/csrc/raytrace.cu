@@ -78,7 +78,9 @@ struct RtSmem {
   unsigned short list[kRtWin];        // the window's subhalos that the expansion does not serve, in index order
   int lcnt[2][kRtThreads / 32];       // per warp: how many of them this round of threads holds
   float mred[kRtThreads / 32][kRtExpFloats];  // per-warp sums of the expansion's independent coefficients
-  float2 coef[(kExpN + 1) * (kExpN + 2) / 2];  // the tile's coefficients: by l, then k (rt_coef_at)
+  float2 coef[(kExpN + 1) * (kExpN + 2) / 2];  // the tile's coefficients: by l, then k (rt_coef_at); 0 for c_00
+  float4 exp;                                  // rt_exp_frame
+  float4 c00w[kRtThreads / 32], c00;           // c_00 by warp and in all: (re, im) and what they are short by
 };
 
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
@@ -434,6 +436,18 @@ __device__ __forceinline__ void add_subs(const RtSmem& sm, int cnt, const float 
 // c_(l+1)(k-1): only the 24 terms with m = l + 1 - k >= 0 are summed,
 // (h u)^k (h conj(u))^(l+1) = (h |u|)^2k (h conj(u))^m, those of m = 0 real.
 // The truncation is below 5e-9 of the sum of absolute terms.
+//
+// The constant term c_00 carries the deflection at the tile's centre; the other
+// terms are below 0.08 of it per subhalo, and so are their roundings. So c_00's
+// sums over groups of 8 threads, the warps and the windows are compensated, it
+// joins the other terms and each point's direct sums by two-sums (rt_two_sum;
+// Kahan's step would lose a small sum under a larger addend), and the centre lies
+// on a lattice coarse enough for its distance from a far subhalo to be exact: a
+// rounding there is the same for all of them. With the far subhalos all to one
+// side their deflection's error then spreads by 0.33 to 0.53 ulp rms over the
+// points (direct sums 0.37 to 0.76; with plain sums and an unrounded centre 0.6
+// to 1.0), at 1 to 3 % of the kernel's time (640k points: 200 subhalos 59.0 ->
+// 60.6 us, 2.56M x 2000 557 -> 565).
 
 // First float of the term (m, k): m = 0 holds k = 1..4, m > 0 holds k = 0 ..
 // (8 - m) / 2 as complex values.
@@ -486,14 +500,43 @@ __device__ __forceinline__ void rt_exp_add(const SubRec& rec, const SubSer& q, f
   }
 }
 
+// The frame of a tile's expansion: the centre of its box, on a lattice of 1/8192
+// to 1/4096 of the half-diagonal, the half-diagonal squared (0: a single point)
+// and its inverse.
+__device__ __forceinline__ float4 rt_exp_frame(const float* box) {
+  const float hx = 0.5f * (box[2] - box[0]), hy = 0.5f * (box[3] - box[1]);
+  const float hd2 = fmaf(hx, hx, hy * hy), h = sqrtf(hd2);
+  const float cell = __uint_as_float(__float_as_uint(h) & 0x7f800000u) * (1.0f / 4096.0f);  // a power of two
+  const float ic = 1.0f / cell;
+  return make_float4(rintf(0.5f * (box[0] + box[2]) * ic) * cell, rintf(0.5f * (box[1] + box[3]) * ic) * cell, hd2,
+                     1.0f / h);
+}
+
+// a + b rounded, and in e what it is short by.
+__device__ __forceinline__ float2 rt_two_sum(float2 a, float2 b, float2& e) {
+  const float2 t = __fadd2_rn(a, b), bb = sub2(t, a);
+  e = __fadd2_rn(sub2(a, sub2(t, bb)), sub2(b, bb));
+  return t;
+}
+
+// a + b of two sums (re, im, what re is short by, what im is short by): the
+// rounding of each addition (two-sum) joins what they are short by.
+__device__ __forceinline__ float4 rt_pair_add(float4 a, float4 b) {
+  float2 e;
+  const float2 t = rt_two_sum(make_float2(a.x, a.y), make_float2(b.x, b.y), e);
+  e = __fadd2_rn(__fadd2_rn(make_float2(a.z, a.w), make_float2(b.z, b.w)), e);
+  return make_float4(t.x, t.y, e.x, e.y);
+}
+
 // Whether the tile takes the expansion: where at least 40 + n_sub / 4 subhalos
 // are 12.5 half-diagonals from its centre. A far subhalo saves about 15 issue
 // slots per thread (two points); the expansion costs some 600 once and 500 per
 // 128 subhalos, far or not. 640k points: 200 subhalos 90 -> 59 us, 500 197 ->
 // 87 us; 16k points, 128 subhalos, few of them far, 24.5 us without and 26.9
 // with it.
-__device__ __forceinline__ bool rt_expands(const float* __restrict__ sub, int n_sub, float2 cen, float hd2,
-                                           RtSmem& sm) {
+__device__ __forceinline__ bool rt_expands(const float* __restrict__ sub, int n_sub, RtSmem& sm) {
+  const float2 cen = make_float2(sm.exp.x, sm.exp.y);
+  const float hd2 = sm.exp.z;
   int far = 0;
   for (int h = threadIdx.x; h < n_sub; h += kRtThreads) {
     const float dx = cen.x - __ldg(sub + 5 * (int64_t)h), dy = cen.y - __ldg(sub + 5 * (int64_t)h + 1);
@@ -510,11 +553,11 @@ __device__ __forceinline__ bool rt_expands(const float* __restrict__ sub, int n_
 // The window's wn subhalos at sub: those far enough from the tile are summed
 // into sm.coef (added where add), the others listed in sm.list in index
 // order. Returns the list's length. All threads of the CTA take part.
-__device__ __forceinline__ int rt_expand_window(const float* __restrict__ sub, int wn, bool add, float2 cen, float hd2,
-                                                RtSmem& sm) {
+__device__ __forceinline__ int rt_expand_window(const float* __restrict__ sub, int wn, bool add, RtSmem& sm) {
   constexpr int kW = kRtThreads / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float h = sqrtf(hd2);
+  const float2 cen = make_float2(sm.exp.x, sm.exp.y);
+  const float hd2 = sm.exp.z, h = sqrtf(hd2);
   float acc[kRtExpFloats];
 #pragma unroll
   for (int i = 0; i < kRtExpFloats; ++i) acc[i] = 0.f;
@@ -550,6 +593,9 @@ __device__ __forceinline__ int rt_expand_window(const float* __restrict__ sub, i
     }
     if (direct) sm.list[before + __popc(m & ((1u << lane) - 1u))] = (unsigned short)t;
   }
+  constexpr int k00 = rt_exp_at(1, 0);
+  float4 z = make_float4(acc[k00], acc[k00 + 1], 0.f, 0.f);
+  acc[k00] = acc[k00 + 1] = 0.f;
 #pragma unroll
   for (int b = 0; b < kRtExpFloats; b += 32) {
     float v[32];
@@ -558,7 +604,21 @@ __device__ __forceinline__ int rt_expand_window(const float* __restrict__ sub, i
     const float t = warp_scatter32(v, lane);
     if (b + lane < kRtExpFloats) sm.mred[warp][b + lane] = t;
   }
+  for (int o = 16; o > 2; o >>= 1) {
+    z.x += __shfl_xor_sync(0xffffffffu, z.x, o);
+    z.y += __shfl_xor_sync(0xffffffffu, z.y, o);
+  }
+#pragma unroll
+  for (int o = 2; o > 0; o >>= 1)
+    z = rt_pair_add(z, make_float4(__shfl_xor_sync(0xffffffffu, z.x, o), __shfl_xor_sync(0xffffffffu, z.y, o),
+                                   __shfl_xor_sync(0xffffffffu, z.z, o), __shfl_xor_sync(0xffffffffu, z.w, o)));
+  if (lane == 0) sm.c00w[warp] = z;
   __syncthreads();
+  if (tid == kRtThreads - 1) {  // its warp has no coefficients below
+    z = add ? rt_pair_add(sm.c00, sm.c00w[0]) : sm.c00w[0];
+    for (int w = 1; w < kW; ++w) z = rt_pair_add(z, sm.c00w[w]);
+    sm.c00 = z;
+  }
   if (tid < (kExpN + 1) * (kExpN + 2) / 2) {
     int l = 0;
     while (rt_coef_at(0, l + 1) <= tid) ++l;
@@ -585,10 +645,12 @@ __device__ __forceinline__ int rt_expand_window(const float* __restrict__ sub, i
 
 // The expansion at the thread's points, added to their Kahan sums: Horner in
 // delta, then in conj(delta), both points packed.
-__device__ __forceinline__ void rt_expand_eval(const RtSmem& sm, float2 cen, float ih, const float (&x)[kRtPts],
+__device__ __forceinline__ void rt_expand_eval(const RtSmem& sm, const float (&x)[kRtPts],
                                                const float (&y)[kRtPts], float (&sx)[kRtPts], float (&cx)[kRtPts],
                                                float (&sy)[kRtPts], float (&cy)[kRtPts]) {
   static_assert(kRtPts == 2, "the thread's points are the two lanes");
+  const float2 cen = make_float2(sm.exp.x, sm.exp.y);
+  const float ih = sm.exp.w;
   const float2 X = make_float2((x[0] - cen.x) * ih, (x[1] - cen.x) * ih);
   const float2 Y = make_float2((y[0] - cen.y) * ih, (y[1] - cen.y) * ih), nY = make_float2(-Y.x, -Y.y);
   float2 ar = f2(0.f), ai = f2(0.f);
@@ -606,10 +668,21 @@ __device__ __forceinline__ void rt_expand_eval(const RtSmem& sm, float2 cen, flo
     ai = __ffma2_rn(ai, X, __ffma2_rn(ar, nY, pi));
     ar = r;
   }
-  kahan(sx[0], cx[0], ar.x);
-  kahan(sx[1], cx[1], ar.y);
-  kahan(sy[0], cy[0], ai.x);
-  kahan(sy[1], cy[1], ai.y);
+  // two-sums: the addends may be larger than the direct sums
+  const float4 z = sm.c00;
+  float2 ex, ey, fx, fy;
+  const float2 tx = rt_two_sum(f2(z.x), ar, ex), ty = rt_two_sum(f2(z.y), ai, ey);
+  const float2 ux = rt_two_sum(make_float2(sx[0], sx[1]), tx, fx), uy = rt_two_sum(make_float2(sy[0], sy[1]), ty, fy);
+  ex = __fadd2_rn(__fadd2_rn(ex, f2(z.z)), fx);
+  ey = __fadd2_rn(__fadd2_rn(ey, f2(z.w)), fy);
+  sx[0] = ux.x;
+  sx[1] = ux.y;
+  sy[0] = uy.x;
+  sy[1] = uy.y;
+  cx[0] -= ex.x;
+  cx[1] -= ex.y;
+  cy[0] -= ey.x;
+  cy[1] -= ey.y;
 }
 
 __host__ __device__ __forceinline__ bool rt_may_expand(bool explicit_points, const GridDev& g, int profile,
@@ -694,6 +767,7 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
       sm.box[1] = c1;
       sm.box[2] = c2;
       sm.box[3] = c3;
+      if constexpr (EXP) sm.exp = rt_exp_frame(sm.box);
     }
     __syncthreads();
     uint32_t phase = 0;
@@ -702,14 +776,11 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
     for (int j = 0; j < NP; ++j) sx[j] = cx[j] = sy[j] = cy[j] = 0.f;
     bool expand = false;
     if constexpr (EXP && PROFILE == LR_PROFILE_TNFW) {
-      const float2 cen = make_float2(0.5f * (sm.box[0] + sm.box[2]), 0.5f * (sm.box[1] + sm.box[3]));
-      const float hx = 0.5f * (sm.box[2] - sm.box[0]), hy = 0.5f * (sm.box[3] - sm.box[1]);
-      const float hd2 = fmaf(hx, hx, hy * hy);  // the tile's half-diagonal squared (0: a single point)
-      expand = hd2 > 0.f && rt_expands(sub, n_sub, cen, hd2, sm);
+      expand = sm.exp.z > 0.f && rt_expands(sub, n_sub, sm);
       if (expand) {
         for (int w0 = 0; w0 < n_sub; w0 += kRtWin) {
           const float* win = sub + 5 * (int64_t)w0;
-          const int nl = rt_expand_window(win, min(kRtWin, n_sub - w0), w0 > 0, cen, hd2, sm);
+          const int nl = rt_expand_window(win, min(kRtWin, n_sub - w0), w0 > 0, sm);
           for (int h0 = 0; h0 < nl; h0 += kSubChunk) {
             const int cnt = min(kSubChunk, nl - h0);
             stage_rt<NT>(win, h0, cnt, PROFILE, sm, phase, false, fault, sm.list);
@@ -717,7 +788,7 @@ __device__ __forceinline__ void raytrace_body(const LensConst& L, const GridDev&
             __syncthreads();
           }
         }
-        rt_expand_eval(sm, cen, 1.0f / sqrtf(hd2), px, py, sx, cx, sy, cy);
+        rt_expand_eval(sm, px, py, sx, cx, sy, cy);
       }
     }
     for (int h0 = 0; h0 < n_sub && !expand; h0 += kSubChunk) {
