@@ -704,7 +704,7 @@ __device__ __forceinline__ int vj_pick_phases(int nd, int np) {
 // The tNFW subhalo sums of a tile whose points are staged in one chunk: the
 // first nexp subhalos of its order by the local expansion, one thread each,
 // then the direct ones in slots (subhalo, phase) with the tile's own phase
-// count; a subhalo's P slots are neighbouring lanes, added by shuffles.
+// count; a subhalo's P slots are neighbouring lanes, added by shuffles (two-sums).
 // Choosing the phases per tile keeps the threads busy when few subhalos are
 // left to the direct sums, and lets any subhalo count take the expansion: with
 // one phase count per launch, 200 subhalos ran in 3 phases and every pair
@@ -734,6 +734,7 @@ __device__ __forceinline__ void vj_tile_sums(const float* __restrict__ sub, int 
     const bool own = slot < nd * P;
     const int h = own ? (int)ord[nexp + slot / P] : 0;
     float sc[4] = {0.f, 0.f, 0.f, 0.f}, cc[4] = {0.f, 0.f, 0.f, 0.f};
+    float scale[4] = {0.f, 0.f, 0.f, 0.f};
     if (own) {
       const float* rr = sub + 5 * (int64_t)h;
       const SubRec rec = prep_sub(rr, PR);
@@ -748,15 +749,22 @@ __device__ __forceinline__ void vj_tile_sums(const float* __restrict__ sub, int 
         default: vj_sweep<PR, 0>(rec, ex, q, sm.pos, sm.grad, np, r, P, sc, cc);
       }
 #pragma unroll
-      for (int v = 0; v < 4; ++v) sc[v] = __fmul_rn(sc[v] - cc[v], vj_scale<PR>(rec, ex, v));
+      for (int v = 0; v < 4; ++v) scale[v] = vj_scale<PR>(rec, ex, v);
     }
+    // the phases' sums with their compensation, by two-sums
     for (int o = P >> 1; o > 0; o >>= 1)
 #pragma unroll
-      for (int v = 0; v < 4; ++v) sc[v] += __shfl_xor_sync(0xffffffffu, sc[v], o);
+      for (int v = 0; v < 4; ++v) {
+        const float b = __shfl_xor_sync(0xffffffffu, sc[v], o), bc = __shfl_xor_sync(0xffffffffu, cc[v], o);
+        const float t = __fadd_rn(sc[v], b), bb = __fsub_rn(t, sc[v]);
+        const float e = __fadd_rn(__fsub_rn(sc[v], __fsub_rn(t, bb)), __fsub_rn(b, bb));
+        cc[v] = __fsub_rn(__fadd_rn(cc[v], bc), e);
+        sc[v] = t;
+      }
     if (own && r == 0) {
       float* o = sub_part + (int64_t)h * 4 * nblk + blk;
 #pragma unroll
-      for (int v = 0; v < 4; ++v) o[v * nblk] = sc[v];
+      for (int v = 0; v < 4; ++v) o[v * nblk] = __fmul_rn(sc[v] - cc[v], scale[v]);
     }
   }
 }
