@@ -750,8 +750,12 @@ lr_status solve_session_destroy(lr_session* s);
  * reduction, with the same arguments minus the workspace.
  *  - Scratch is a static device array of lr_static_scratch_bytes() bytes
  *    (48 MiB) that every GPU loading this library holds until the process
- *    exits. Problems whose workspace requirement (lr_matvec_workspace_size)
- *    exceeds it are rejected with LR_ERR_INVALID_ARG; nothing else is
+ *    exits. A problem whose workspace requirement (lr_matvec_workspace_size)
+ *    exceeds it runs without the partial sums of a sweep in parts, one CTA per
+ *    block of rows, where it fits like that (each row is then one compensated
+ *    sum instead of a sum of parts, so the bits may differ from
+ *    gp_kernel_matvec's; at or below the size they are the same). What does
+ *    not fit even so is rejected with LR_ERR_INVALID_ARG; nothing else is
  *    allocated (no cudaMalloc, cudaFree or allocating library call).
  *  - Every call resolves the array's device address in the current
  *    device's context (cudaGetSymbolAddress, with that device current); the
