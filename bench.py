@@ -1015,8 +1015,8 @@ def run_realistic(args, dev, rates, clk) -> dict:
         "pairs": {"logical_per_step": p.pairs, "evaluated_training_forward": ev[512],
                   "evaluated_dv_sweep": ev[1024],
                   "note": "value counts every logical (i, j) pair; the grid kernels leave out the pairs whose "
-                          "FP32 exp2 flushes to exactly 0 (scaled distance^2 > 127), so results are identical to "
-                          "evaluating all of them; the roofline counts evaluated pairs"},
+                          "FP32 exp2 flushes to 0 (scaled distance^2 > 127), terms below 2^-126 |v| (exactly 0 in "
+                          "the unsplit form); the roofline counts evaluated pairs"},
         "roofline": {"bound": "alu", "achieved": d["achieved"], "peak": d["peak"], "unit": UNIT,
                      "frac": d["frac"], "traffic": measured_traffic("realistic: " + dom), "kernel": dom,
                      "peak_basis": f"min(MUFU {ex2:.2f}/clk/SM / MUFU per pair, FFMA2 {fma:.1f} lanes/clk/SM / lanes "

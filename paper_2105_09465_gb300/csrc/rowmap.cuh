@@ -11,14 +11,17 @@
 // it is, leaving out pairs with t > kSkipT = 127 changes no result bit (the
 // FP32 rounding of t is below 1e-4 there, the unit of margin covers it). The
 // split form 2^(x'^2 - t) (v 2^(-x'^2)) could still carry a pair to t = 156,
-// at most 2^-126 |v|: there the same line is drawn, so that both forms leave
-// out a kernel value that FP32 does not hold. A line at 170 (156 and a margin),
+// at most 2^-126 |v| each (an absolute bound: with |v| above 2 such a term can be
+// a normal number, and a row with every source between 127 and 156 gives 0):
+// there the same line is drawn, so that both forms leave out a kernel value that
+// FP32 does not hold. A line at 170 (156 and a margin),
 // which served both forms before, takes in 1.34 times the area.
 //
 // Where the work is laid out. The range of grid rows that the chunks of a row
 // block share out, and the columns from which a tile's sub-segments are laid,
-// go by kLayT = 170: they set the order and the rounding of the sums, not
-// what is summed, and a row's sums keep their bits whatever kSkipT leaves out.
+// go by kLayT = 170: they set the order and the rounding of the sums, not what
+// is summed, so that in the unsplit form a row's sums keep their bits whatever
+// kSkipT leaves out.
 #pragma once
 #include "grid.cuh"
 
