@@ -12,7 +12,7 @@ int64_t grid_count(const lr_grid& g);
 lr_status launch_grid_points(const lr_grid& g, float2* out, cudaStream_t s);
 lr_status launch_raytrace(const lr_points* p, float2* beta, float2* alpha, cudaStream_t s);
 lr_status make_lens_grad_const(const lr_lens* lens, LensGradConst* out);
-size_t raytrace_vjp_ws(int64_t n, int32_t n_sub);
+size_t raytrace_vjp_ws(int64_t n, int32_t n_sub, int32_t profile);
 lr_status launch_raytrace_vjp(const lr_points* p, const float2* dbeta, double* d_lens, double* d_sub, void* ws,
                               cudaStream_t s);
 

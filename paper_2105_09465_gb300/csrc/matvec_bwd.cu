@@ -1774,7 +1774,7 @@ static lr_status plan_bwd(const lr_points* q, const lr_points* s, int32_t nrhs, 
     }
   }
   p.off_vjp = off;
-  if (p.want_lens) off += raytrace_vjp_ws(p.n, q->n_sub);
+  if (p.want_lens) off += raytrace_vjp_ws(p.n, q->n_sub, q->profile);
   p.bytes = off;
   *P = p;
   return LR_OK;

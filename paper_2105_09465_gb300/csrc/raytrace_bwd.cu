@@ -1076,12 +1076,22 @@ static bool vjp_planned(int64_t ntiles, const lr_points* p) {
   return p->profile == LR_PROFILE_TNFW && plan_fits(ntiles, p->n_sub);
 }
 
-// Phases P of the subhalo sums of tiles that do not choose their own: 1 when
-// n_sub slots waste at most 5 % of the last group of kVjThreads, else the P in
+// Whether tiles of a launch may not choose their own phases (vj_tile_sums): point
+// masses, more subhalos than a CTA orders, or tiles beyond one staged chunk. A
+// band of a grid may have one row more than the mean, so a tile holds at most
+// twice the mean points (one row of them each).
+static bool vjp_shared_phases(int64_t n, int32_t n_sub, int32_t profile) {
+  const int64_t per_cta = (n + vjp_tiles(n) - 1) / vjp_tiles(n);
+  return profile != LR_PROFILE_TNFW || n_sub > kVjMaxOrd || 2 * per_cta + 1 > kVjChunk;
+}
+
+// Phases P of the subhalo sums of tiles that do not choose their own (1 where
+// there are none, which leaves their slot sums out of the workspace): 1 when n_sub
+// slots waste at most 5 % of the last group of kVjThreads, else the P in
 // [1, kVjMaxPhases] whose slot count n_sub P wastes the fewest threads of the
 // last group (the smallest such P), keeping at least 128 points per slot.
-int vjp_phases(int64_t n, int32_t n_sub) {
-  if (n_sub <= 0 || n <= 0) return 1;
+int vjp_phases(int64_t n, int32_t n_sub, int32_t profile) {
+  if (n_sub <= 0 || n <= 0 || !vjp_shared_phases(n, n_sub, profile)) return 1;
   const int64_t per_cta = (n + vjp_tiles(n) - 1) / vjp_tiles(n);
   const int64_t pad1 = ((int64_t)n_sub + kVjThreads - 1) / kVjThreads * kVjThreads;
   if ((double)pad1 <= 1.05 * (double)n_sub) return 1;
@@ -1226,9 +1236,9 @@ struct VjWs {
   size_t bytes;
 };
 
-static VjWs vjp_ws_layout(void* ws, int64_t n, int32_t n_sub) {
+static VjWs vjp_ws_layout(void* ws, int64_t n, int32_t n_sub, int32_t profile) {
   const int64_t nt = vjp_tiles(n);
-  const int P = vjp_phases(n, n_sub);
+  const int P = vjp_phases(n, n_sub, profile);
   const bool plan = plan_fits(nt, n_sub);
   const size_t b_lens = align256(sizeof(double) * 7 * (size_t)nt);
   const size_t b_sub = align256(sizeof(float) * 4 * (size_t)n_sub * (size_t)nt);
@@ -1255,7 +1265,9 @@ static VjWs vjp_ws_layout(void* ws, int64_t n, int32_t n_sub) {
   return w;
 }
 
-size_t raytrace_vjp_ws(int64_t n, int32_t n_sub) { return vjp_ws_layout(nullptr, n, n_sub).bytes; }
+size_t raytrace_vjp_ws(int64_t n, int32_t n_sub, int32_t profile) {
+  return vjp_ws_layout(nullptr, n, n_sub, profile).bytes;
+}
 
 lr_status launch_raytrace_vjp(const lr_points* p, const float2* dbeta, double* d_lens, double* d_sub, void* ws,
                               cudaStream_t s) {
@@ -1274,12 +1286,12 @@ lr_status launch_raytrace_vjp(const lr_points* p, const float2* dbeta, double* d
     if (d_sub && p->n_sub) LR_CHECK_CUDA(cudaMemsetAsync(d_sub, 0, 4 * sizeof(double) * p->n_sub, s));
     return LR_OK;
   }
-  const VjWs w = vjp_ws_layout(ws, p->n, p->n_sub);
+  const VjWs w = vjp_ws_layout(ws, p->n, p->n_sub, p->profile);
   double* lens_part = w.lens_part;
   float* sub_part = w.sub_part;
   const GridDev g = p->xy ? GridDev{} : grid_dev(p->grid);
   const float2* xi = reinterpret_cast<const float2*>(p->xy);
-  const int P = vjp_phases(p->n, p->n_sub);
+  const int P = vjp_phases(p->n, p->n_sub, p->profile);
   const int bands = vjp_bands(nblk, p);
   int* fault = fault_ptr();
   LR_REQUIRE(fault != nullptr, "could not resolve the device fault word");
@@ -1332,10 +1344,10 @@ lr_status make_vjp_problem(const lr_points* p, const float2* dbeta, double* d_le
   v.sub = p->sub;
   v.n_sub = p->n_sub;
   v.profile = p->profile;
-  v.phases = vjp_phases(p->n, p->n_sub);
+  v.phases = vjp_phases(p->n, p->n_sub, p->profile);
   v.bands = vjp_bands(nblk, p);
   v.dbeta = dbeta;
-  const VjWs w = vjp_ws_layout(ws, p->n, p->n_sub);
+  const VjWs w = vjp_ws_layout(ws, p->n, p->n_sub, p->profile);
   v.lens_part = w.lens_part;
   v.sub_part = w.sub_part;
   v.slot_part = w.slot_part;
@@ -1355,7 +1367,7 @@ extern "C" lr_status lr_raytrace_vjp_workspace_size(const lr_points* pts, size_t
   LR_REQUIRE(bytes != nullptr, "lr_raytrace_vjp_workspace_size: bytes is NULL");
   lr_status st = lr::validate_points(pts, "lr_raytrace_vjp_workspace_size", true);
   if (st != LR_OK) return st;
-  *bytes = lr::raytrace_vjp_ws(pts->n, pts->n_sub);
+  *bytes = lr::raytrace_vjp_ws(pts->n, pts->n_sub, pts->profile);
   return LR_OK;
 }
 
@@ -1367,7 +1379,7 @@ extern "C" lr_status lens_raytrace_vjp(const lr_points* pts, const float* d_beta
   LR_REQUIRE(((uintptr_t)d_beta & 7u) == 0, "lens_raytrace_vjp: d_beta must be 8-byte aligned");
   LR_REQUIRE(((uintptr_t)d_lens & 7u) == 0 && ((uintptr_t)d_sub & 7u) == 0,
              "lens_raytrace_vjp: gradient outputs must be 8-byte aligned");
-  const size_t need = lr::raytrace_vjp_ws(pts->n, pts->n_sub);
+  const size_t need = lr::raytrace_vjp_ws(pts->n, pts->n_sub, pts->profile);
   LR_REQUIRE(workspace_bytes >= need, "lens_raytrace_vjp: workspace of %zu bytes, %zu needed", workspace_bytes, need);
   LR_REQUIRE(need == 0 || workspace != nullptr, "lens_raytrace_vjp: workspace is NULL");
   LR_REQUIRE(((uintptr_t)workspace & 255u) == 0, "lens_raytrace_vjp: workspace must be 256-byte aligned");

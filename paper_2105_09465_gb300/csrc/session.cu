@@ -165,7 +165,7 @@ lr_status size_request(Req* r) {
   r->o_train = carve(off, train_b);
   r->o_mrows = carve(off, mrows_b);
   r->o_dvp = carve(off, dv_b);
-  r->o_vjp = carve(off, raytrace_vjp_ws(n, r->n_sub));
+  r->o_vjp = carve(off, raytrace_vjp_ws(n, r->n_sub, r->profile));
   r->bytes = off;
   return LR_OK;
 }
