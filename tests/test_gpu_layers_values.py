@@ -27,7 +27,8 @@ def layers(x, src, v, ls, vs, cull):
 
 @pytest.mark.parametrize("what", ["weight nan", "weight inf", "source nan", "whole chunk nan"])
 @pytest.mark.parametrize("cull", [1, 0])
-@pytest.mark.parametrize("n", [5, 700, 400000])  # in parts, and (above the waves for them) one CTA per row block
+# all pairs, the culled sweep in parts, and (above the waves for them) one CTA per row block
+@pytest.mark.parametrize("n", [5, 700, 100000, 1000000])
 def test_not_finite_reaches_every_row(what, cull, n):
     rng = np.random.default_rng(n)
     m = 2000
