@@ -1108,6 +1108,9 @@ static const void* cull_kernel_ptr(int kind, int nw, int layers) {
   }
 }
 
+// The windowed backward's sweeps run in parts at every size.
+static constexpr bool parts_only(int kind) { return kind == kCullWinRows || kind == kCullWinCols; }
+
 static int cull_rows_per_thread(int kind, int nw, int layers) {
   if (kind == kCullLay) return nw / layers <= 2 ? 4 : 2;
   if (kind == kCullOut) return nw <= 2 ? 4 : 2;
@@ -1136,17 +1139,17 @@ lr_status plan_cull(int kind, int nrhs, int64_t n, const lr_grid* qlayout, int64
   P.row_blocks = row_block_count(P.map, n, P.rows_per_cta);
   int n_sm = 1, occ = 1;
   LR_CHECK(kernel_occupancy_of(cull_kernel_ptr(kind, P.nw, layers), kCullThreads, &occ, &n_sm));
-  // In parts (cull.cuh) where the row blocks are under kFewWaves waves of the
-  // resident CTA slots (above, one CTA per row block keeps its sums in
-  // registers, and a band of rows gives the whole problem's bits), and always for windowed points: they differ in reach by orders of
-  // magnitude (pixels next to the lens centre reach arcseconds, half the
-  // image), and so do their row blocks.
+  // In parts (cull.cuh) where there are more than kPartSources sources and the row
+  // blocks are under kFewWaves waves of the resident CTA slots (above, one CTA per
+  // row block keeps its sums in registers, and a band of rows gives the whole
+  // problem's bits). Windowed rows at any count: they differ in reach by orders of
+  // magnitude (pixels next to the lens centre reach arcseconds, half the image),
+  // and so do their row blocks; the windowed backward's merges take parts alone.
   const int64_t slots = (int64_t)(occ > 0 ? occ : 1) * n_sm;
-  const bool windowed = kind == kCullWin || kind == kCullWinRows || kind == kCullWinCols;
   P.R = cull_rows_per_thread(kind, P.nw, layers);
   P.extra = (int32_t)(kPartWaves * slots);
-  // (with no sources too: the windowed kinds have no other kernel, and their merge writes the outputs)
-  P.parts = P.row_blocks > 0 && (windowed || (allow_parts && m > kPartSources && P.row_blocks < kFewWaves * slots));
+  const bool few = kind == kCullWin || (allow_parts && P.row_blocks < kFewWaves * slots);
+  P.parts = P.row_blocks > 0 && P.L.n_groups > 0 && (parts_only(kind) || (m > kPartSources && few));
   P.K = cull_k(kind, P.nw, layers);
   size_t off = 0;
   P.off_rec = off;
@@ -1206,11 +1209,8 @@ static lr_status launch_prep_kernels(const CullPlan& P, CullPrepP& Q, char* ws, 
   Q.rec = ws + P.off_rec;
   Q.cbox = reinterpret_cast<float4*>(ws + P.off_cbox);
   Q.gbox = reinterpret_cast<float4*>(ws + P.off_gbox);
+  if (P.L.n_chunks == 0) return LR_OK;
   if (P.parts) Q.ticket = plan_ticket(P, ws);
-  if (P.L.n_chunks == 0) {  // no sources: the plan kernel still counts its CTAs
-    if (Q.ticket) LR_CHECK_CUDA(cudaMemsetAsync(Q.ticket, 0, 2 * sizeof(unsigned long long), s));
-    return LR_OK;
-  }
   cull_prep_kernel<<<(unsigned)P.L.n_groups, kPrepThreads, 0, s>>>(Q);
   LR_CHECK_CUDA(cudaGetLastError());
   return LR_OK;
@@ -1258,14 +1258,13 @@ lr_status launch_cull_prep_layers(const CullPlan& P, const float2* pts, const lr
 
 template <int KIND, int NW, int L = 1>
 static lr_status launch_sweep_t(const CullPlan& P, const CullArgs& A, cudaStream_t s) {
-  constexpr bool WINDOWED = KIND == kCullWin || KIND == kCullWinRows || KIND == kCullWinCols;
   if (P.parts)
     cull_kernel<KIND, NW, L, true><<<(unsigned)(P.row_blocks + P.extra), kCullThreads, 0, s>>>(A);
-  else if constexpr (!WINDOWED)
+  else if constexpr (!parts_only(KIND))
     cull_kernel<KIND, NW, L, false><<<(unsigned)P.row_blocks, kCullThreads, 0, s>>>(A);
   LR_CHECK_CUDA(cudaGetLastError());
   // the windowed backward kinds leave their partials to the caller's merge
-  if constexpr (KIND != kCullWinRows && KIND != kCullWinCols) {
+  if constexpr (!parts_only(KIND)) {
     if (P.parts && !A.count_out) {
       CullParts M{A.partial, A.start, P.map, A.n, P.rows_per_cta, P.R};
       cull_merge_kernel<KIND, CullTraits<KIND, NW, L>::K>

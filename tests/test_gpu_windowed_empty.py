@@ -1,14 +1,16 @@
-"""The windowed reduction with its likelihood over no sources: the model is
-f_in alone. Library entry only (the Python wrapper hands an empty tensor over as
-NULL, which the entry refuses)."""
+"""The windowed reduction over few sources: none (with its likelihood the model is
+f_in alone; library entry only, the Python wrapper hands an empty tensor over as
+NULL, which the entry refuses), and up to 512, where each row block is one CTA
+instead of parts, against the FP64 oracle within 2e-5 of the sum of absolute
+terms."""
 import ctypes
 
 import numpy as np
 import pytest
 import torch
 
-from paper_2105_09465_gb300 import abi, workloads as W
-from tests.gpu_util import dev, need_gpu
+from paper_2105_09465_gb300 import abi, api, workloads as W
+from tests.gpu_util import assert_matvec_close, dev, host, need_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -51,3 +53,27 @@ def test_likelihood_over_no_sources(n, layout, cull):
     np.testing.assert_allclose(g.cpu().numpy(), (f32 - d32) / s**2, rtol=1e-6, atol=1e-6)
     want = 0.5 * np.sum(((f32 - d32) / s) ** 2) + n * (np.log(s) + 0.5 * np.log(2 * np.pi))
     np.testing.assert_allclose(nll.item(), want, rtol=1e-6, atol=1e-6)
+
+
+@pytest.mark.parametrize("m", [1, 31, 512, 513])
+@pytest.mark.parametrize("n,layout", [(1, None), (300, None), (5000, (100, 50))])
+def test_few_sources(orc, n, m, layout):
+    rng = np.random.default_rng(n + m)
+    lay = W.Grid(layout[0], layout[1], 1, 0.02) if layout else None
+    p = orc.grid_points(*lay.astuple()) if lay else rng.uniform(-1, 1, (n, 2)).astype(np.float32)
+    a = rng.uniform(0.01, 0.05, (n, 2, 2))
+    z = np.stack([(a[:, 0] * a[:, 0]).sum(1), (a[:, 0] * a[:, 1]).sum(1), (a[:, 1] * a[:, 1]).sum(1)], 1)
+    z = z.astype(np.float32)
+    q, v = rng.uniform(-1, 1, (m, 2)).astype(np.float32), rng.standard_normal(m).astype(np.float32)
+    f, data = (rng.standard_normal(n).astype(np.float32) for _ in range(2))
+    ell, sigma = 0.05, 0.3
+    src = api.Points(xy=dev(q))
+    ref, ab = orc.windowed_matvec(p, z, q, v, ell)
+    got = api.gp_windowed_matvec(dev(p), dev(z), src, dev(v), ell, layout=lay)
+    assert_matvec_close(host(got), ref, ab, what="windowed")
+    out, g, nll = api.gp_windowed_matvec_nll(dev(p), dev(z), src, dev(v), ell, dev(data), sigma, f_in=dev(f), layout=lay)
+    assert_matvec_close(host(out), ref + f, ab + np.abs(f), what="model")
+    r = (host(out) - data) / np.float32(sigma)
+    np.testing.assert_allclose(host(g), r / np.float32(sigma), rtol=1e-5, atol=1e-5)
+    np.testing.assert_allclose(nll.item(), 0.5 * (r * r).sum() + n * (np.log(np.float64(np.float32(sigma)))
+                                                                      + 0.5 * np.log(2 * np.pi)), rtol=1e-5, atol=1e-5)
