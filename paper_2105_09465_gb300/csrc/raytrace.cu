@@ -528,19 +528,23 @@ __device__ __forceinline__ float4 rt_pair_add(float4 a, float4 b) {
   return make_float4(t.x, t.y, e.x, e.y);
 }
 
-// Whether the tile takes the expansion: where at least 40 + n_sub / 4 subhalos
-// are 12.5 half-diagonals from its centre. A far subhalo saves about 15 issue
-// slots per thread (two points); the expansion costs some 600 once and 500 per
-// 128 subhalos, far or not. 640k points: 200 subhalos 90 -> 59 us, 500 197 ->
-// 87 us; 16k points, 128 subhalos, few of them far, 24.5 us without and 26.9
-// with it.
+// Whether the tile takes the expansion: where it serves at least 40 + n_sub / 4
+// subhalos, those 12.5 half-diagonals from its centre and beyond the radius of
+// their series. By the distance alone, tiles took it for extended subhalos that it
+// then summed directly: 640k points x 200 of 1e7 to 1e10 solar masses 197 us, now
+// 189, and 186 without an expansion. A far subhalo saves about 15 issue slots per
+// thread (two points); the expansion costs some 600 once and 500 per 128 subhalos,
+// far or not. 640k points: 200 compact subhalos 90 -> 60 us, 500 197 -> 89 us; 16k
+// points, 128 subhalos, few of them far, 24.5 us without and 26.9 with it.
 __device__ __forceinline__ bool rt_expands(const float* __restrict__ sub, int n_sub, RtSmem& sm) {
   const float2 cen = make_float2(sm.exp.x, sm.exp.y);
-  const float hd2 = sm.exp.z;
+  const float hd2 = sm.exp.z, hd = sqrtf(hd2);
   int far = 0;
   for (int h = threadIdx.x; h < n_sub; h += kRtThreads) {
-    const float dx = cen.x - __ldg(sub + 5 * (int64_t)h), dy = cen.y - __ldg(sub + 5 * (int64_t)h + 1);
-    far += hd2 <= kExpRatio2 * fmaf(dx, dx, dy * dy);
+    const float* r = sub + 5 * (int64_t)h;
+    const float dx = cen.x - __ldg(r), dy = cen.y - __ldg(r + 1), r2 = fmaf(dx, dx, dy * dy);
+    const float reach = fmaf(8.0f * fabsf(__ldg(r + 3)), fmaxf(fabsf(__ldg(r + 4)), 2.0f), hd);
+    far += hd2 <= kExpRatio2 * r2 && reach * reach <= r2;
   }
   far = __reduce_add_sync(0xffffffffu, far);
   if ((threadIdx.x & 31) == 0) sm.lcnt[1][threadIdx.x >> 5] = far;  // rt_expand_window starts with the other half
