@@ -4,7 +4,6 @@
 #include <string.h>
 
 #include <mutex>
-#include <vector>
 
 #include "common.cuh"
 #include "tma.cuh"
@@ -30,23 +29,27 @@ lr_status kernel_occupancy_of(const void* fn, int threads, int* occ, int* n_sm) 
     const void* fn;
     int threads, dev, occ, n_sm;
   };
+  constexpr int kKnown = 256;  // a fixed table: nothing here throws through a C entry
   static std::mutex mu;
-  static std::vector<Known> known;  // one entry per kernel and device in use
+  static Known known[kKnown];  // one entry per kernel and device in use
+  static int n_known = 0;
   int dev = 0;
   LR_CHECK_CUDA(cudaGetDevice(&dev));
   {
     std::lock_guard<std::mutex> lock(mu);
-    for (const Known& k : known)
+    for (int i = 0; i < n_known; ++i) {
+      const Known& k = known[i];
       if (k.fn == fn && k.threads == threads && k.dev == dev) {
         *occ = k.occ;
         *n_sm = k.n_sm;
         return LR_OK;
       }
+    }
   }
   LR_CHECK_CUDA(cudaDeviceGetAttribute(n_sm, cudaDevAttrMultiProcessorCount, dev));
   LR_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, fn, threads, 0));
   std::lock_guard<std::mutex> lock(mu);
-  known.push_back({fn, threads, dev, *occ, *n_sm});
+  if (n_known < kKnown) known[n_known++] = {fn, threads, dev, *occ, *n_sm};  // past it: asked again
   return LR_OK;
 }
 
