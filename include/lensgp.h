@@ -109,7 +109,9 @@ lr_status lr_kernel_timer_read(int32_t kernel, int64_t* launches, double* total_
 
 /*
  * Exact skipping of far pairs in the reductions over explicit sources
- * (gp_kernel_matvec, gp_kernel_matvec_bwd). A pair whose exponent is below
+ * (gp_kernel_matvec, gp_kernel_matvec_bwd), over several layers
+ * (gp_kernel_matvec_layers) and over windows (gp_windowed_matvec and its
+ * likelihood and backward). A pair whose exponent is below
  * -126 contributes exactly 0 (the hardware exp2 flushes it), so a row block
  * leaves out every source chunk that is that far from all its rows.
  * lr_set_pair_culling(0) makes those entry points evaluate every pair, in
@@ -248,8 +250,8 @@ lr_status lens_jacobian(const lr_points* pts, float* jac_out, float* mu_out, lr_
  *   source  the y_j, or NULL for a self-kernel (y = x after ray-tracing)
  *   v       device float[m][nrhs]: nrhs = 1..4 right-hand sides reduced in
  *           one pass (one exponential per pair, nrhs FMA); with grid sources
- *           and nrhs > 1 the grid's points are written to the workspace and
- *           reduced like explicit sources
+ *           and nrhs > 1 the grid is reduced like explicit sources (its points
+ *           go into the sweep's records)
  *   out     device float[n][nrhs]
  *   beta_out device float[n][2] or NULL: receives the ray-traced query points
  *   workspace/workspace_bytes: caller-owned device scratch of at least

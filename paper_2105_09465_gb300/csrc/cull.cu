@@ -5,9 +5,9 @@
 // through the reduction, Sec. 3.3 and 3.6), and the windowed transmission of
 // the image-plane layers with its backward (Sec. 3.4, windows of Sec. 3.2).
 //
-// One CTA per (row block, group range). The CTA keeps its rows in registers
-// and lists, in ascending order, the groups and then the chunks within reach
-// of its bounding box. The listed chunks' record blocks are copied into
+// One CTA per row block, or per part of its list of chunks (cull.cuh, "Parts").
+// The CTA keeps its rows in registers and lists, in ascending order, the groups
+// and then the chunks within reach of its bounding box (of its part). The listed chunks' record blocks are copied into
 // shared memory by the bulk-copy engine (cp.async.bulk, completed through an
 // mbarrier with a bounded wait), two batches in flight: the next batch lands
 // while the warps work on the current one. Each warp then tests its own
@@ -224,7 +224,8 @@ struct CullTraits<kCullWinCols, 4> {
   static constexpr int K = 3, R = 1, BATCH = 8;
 };
 
-// Row outputs of one row (totals t[K]) for splits == 1, or of the merge.
+// Row outputs of one row from its totals t[K]: of a CTA with the whole row, or of
+// the merge.
 // Returns the row's scalar-gradient terms (d_l, d_var) through sl, sv.
 template <int KIND, int K>
 __device__ __forceinline__ void cull_finalize(const CullArgs& A, int64_t i, const float* t, float& sl, float& sv) {
@@ -567,9 +568,6 @@ constexpr int cull_min_blocks(int kind) {
   return kind == kCullWin || kind == kCullWinRows || kind == kCullWinCols ? 8 : 0;
 }
 
-// PARTS: one CTA per part (cull.cuh) instead of one per row block. A kernel of its
-// own: with both forms in one, the self-kernel backward at 2.56M points, which
-// takes one CTA per row block, went from 5.16 to 5.50 ms.
 // Folds the sums of a run of chunks into the row totals (Kahan; only nonzero
 // ones, so that chunks left out and chunks of exact zeros agree bitwise).
 constexpr int kLayFold = 4;  // consecutive chunk indices summed plainly
@@ -586,6 +584,9 @@ __device__ __forceinline__ void lay_fold(float2 (&acc)[R][K], float (&tot)[R][K]
     }
 }
 
+// PARTS: one CTA per part (cull.cuh) instead of one per row block. A kernel of its
+// own: with both forms in one, the self-kernel backward at 2.56M points, which
+// takes one CTA per row block, went from 5.16 to 5.50 ms.
 template <int KIND, int NW, int L, bool PARTS>
 __global__ void __launch_bounds__(kCullThreads, cull_min_blocks(KIND)) cull_kernel(const __grid_constant__ CullArgs A) {
   using T = CullTraits<KIND, NW, L>;

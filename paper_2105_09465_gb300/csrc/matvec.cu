@@ -325,7 +325,7 @@ struct MvPlan {
   bool q_raytrace, q_grid;   // query needs ray-tracing / grid materialisation
   bool s_raytrace;           // source needs ray-tracing
   bool s_grid;               // source read as a grid (no materialisation)
-  bool s_mat;                // grid source written out as points (several right-hand sides)
+  bool s_mat;                // grid source's points in the culled sweep's records (several right-hand sides)
   int32_t n_tiles, segs, chunks, row_blocks;
   RowMap map;                // row blocks: image tiles of a grid query, else index order
   CullPlan cull;             // explicit sources: the culled sweep

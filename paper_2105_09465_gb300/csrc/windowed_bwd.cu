@@ -6,11 +6,13 @@
 // Two culled sweeps over the pairs (cull.cu, explicit sources):
 //   rows:    per query row, sum_k v G [1, w, w w^T]     -> d_p, d_Z, d_l  (w = R d)
 //   columns: per source,    sum_i g G [1, u]            -> d_v, d_q
-// Inside a sweep the exponent uses u' = M' d with M' = -(log2 e / 2) M, so
-// that G = N 2^(d . u') and u = -2 ln2 u'; N = 1/(2 pi sqrt(det C)) is applied
-// per row. The sweeps leave their sums per group range; the merges here add
-// them in fixed order (Kahan) and form the gradients, the length-scale sum in
-// FP64, so results are deterministic.
+// Inside a sweep w = k R d with R^T R = M (upper Cholesky factor) and k^2 = log2 e
+// / 2 = 1 / (2 ln 2), so that G = N 2^(-|w|^2) and u = (2 ln 2) (k R)^T w (up to
+// the sign of d); N = 1/(2 pi sqrt(det C)) is applied per windowed point. The
+// row's own R is left out of its sums (w, w w^T); the columns form u' = (k R)^T w
+// per pair. The sweeps leave their sums per part of the chunk lists (cull.cuh);
+// the merges here add them in fixed order (Kahan), apply the factors and form the
+// gradients, the length-scale sum in FP64, so results are deterministic.
 #include <math.h>
 
 #include "cull.cuh"
