@@ -78,6 +78,7 @@ __device__ __forceinline__ bool lay_weights(const CullPrepP& P, int64_t i, bool 
   return __any_sync(0xffffffffu, bad);
 }
 
+template <bool LAY>
 __device__ __forceinline__ void prep_chunk(const CullPrepP& P, int c, int lane, float4& obox, float& oreach) {
   const int64_t i = chunk_point(P.L, c, lane);
   const bool valid = i >= 0;
@@ -88,7 +89,8 @@ __device__ __forceinline__ void prep_chunk(const CullPrepP& P, int c, int lane, 
   const int RB = rec_bytes(P.nw);
   char* rec = P.rec + (int64_t)c * RB;
   float* w = reinterpret_cast<float*>(rec + kRecHead + kRecXY);  // [nw][32], pairs consecutive
-  if (P.kind == kCullLay && lay_weights(P, i, valid, pv, w + lane)) box = kEveryBox;
+  if constexpr (LAY)
+    if (lay_weights(P, i, valid, pv, w + lane)) box = kEveryBox;
   obox = box;
   oreach = INFINITY;
   if (lane == 0) P.cbox[c] = box;
@@ -127,9 +129,9 @@ __device__ __forceinline__ void prep_chunk(const CullPrepP& P, int c, int lane, 
   const int pr = lane >> 1, half = lane & 1;
   xy[4 * pr + half] = p.x;
   xy[4 * pr + 2 + half] = p.y;
-  if (P.kind == kCullOut) {
+  if constexpr (LAY) {  // written above
+  } else if (P.kind == kCullOut) {
     for (int k = 0; k < P.nw; ++k) w[k * kChunkPts + lane] = valid ? P.a[i * P.stride + k] : 0.f;
-  } else if (P.kind == kCullLay) {  // written above
   } else if (P.kind == kCullWin || P.kind == kCullWinRows) {
     w[lane] = valid ? P.a[i] : 0.f;
   } else if (P.kind == kCullWinCols) {
@@ -146,6 +148,9 @@ __device__ __forceinline__ void prep_chunk(const CullPrepP& P, int c, int lane, 
   }
 }
 
+// LAY: kCullLay, a kernel of its own (in one, its weights' test spilled registers of
+// every kind's: a reconstruction of 114^2 points 42.0 -> 43.4 us).
+template <bool LAY>
 __global__ void __launch_bounds__(kPrepThreads) cull_prep_kernel(const __grid_constant__ CullPrepP P) {
   __shared__ float4 sbox[kGroupChunks];
   __shared__ float sreach[kGroupChunks];
@@ -154,7 +159,7 @@ __global__ void __launch_bounds__(kPrepThreads) cull_prep_kernel(const __grid_co
   for (int k = warp; k < kGroupChunks; k += kPrepThreads / 32) {
     float4 box;
     float reach;
-    prep_chunk(P, g * kGroupChunks + k, lane, box, reach);
+    prep_chunk<LAY>(P, g * kGroupChunks + k, lane, box, reach);
     if (lane == 0) {
       sbox[k] = box;
       sreach[k] = reach;
@@ -1212,7 +1217,10 @@ static lr_status launch_prep_kernels(const CullPlan& P, CullPrepP& Q, char* ws, 
   Q.gbox = reinterpret_cast<float4*>(ws + P.off_gbox);
   if (P.L.n_chunks == 0) return LR_OK;
   if (P.parts) Q.ticket = plan_ticket(P, ws);
-  cull_prep_kernel<<<(unsigned)P.L.n_groups, kPrepThreads, 0, s>>>(Q);
+  if (P.kind == kCullLay)
+    cull_prep_kernel<true><<<(unsigned)P.L.n_groups, kPrepThreads, 0, s>>>(Q);
+  else
+    cull_prep_kernel<false><<<(unsigned)P.L.n_groups, kPrepThreads, 0, s>>>(Q);
   LR_CHECK_CUDA(cudaGetLastError());
   return LR_OK;
 }
